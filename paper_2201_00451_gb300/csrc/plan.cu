@@ -462,13 +462,10 @@ int prepare_series(fstat_plan* p, int det, int dtype, cudaStream_t st) {
   return FSTAT_OK;
 }
 
-// Check the stored series for NaN/Inf (synchronises) and update the noise
-// weights: common rescaling by the smallest sigma among the detectors with
-// data.
+// Read the finiteness check that `st` has left in d_err[1] (synchronises) and
+// update the noise weights: common rescaling by the smallest sigma among the
+// detectors with data.
 int finish_series(fstat_plan* p, int det, double sigma, cudaStream_t st) {
-  CK(cudaMemsetAsync(p->d_err + 1, 0, sizeof(int), st));
-  launch_check_finite(p->xh[det], p->dtype[det], p->d.n_samples, p->d_err + 1, st);
-  CK(cudaGetLastError());
   CK(cudaMemcpyAsync(p->h_err + 1, p->d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (p->h_err[1] != 0) return p->h_err[1];
@@ -497,6 +494,9 @@ int fstat_set_data(fstat_plan* p, int det, const void* xh, int dtype, int64_t n,
   int rc = prepare_series(p, det, dtype, st);
   if (rc) return rc;
   CK(cudaMemcpyAsync(p->xh[det], xh, (size_t)n * (dtype == FSTAT_C128 ? 16 : 8), cudaMemcpyDefault, st));
+  CK(cudaMemsetAsync(p->d_err + 1, 0, sizeof(int), st));
+  launch_check_finite(p->xh[det], dtype, n, p->d_err + 1, st);
+  CK(cudaGetLastError());
   return finish_series(p, det, sigma, st);
 }
 
@@ -518,20 +518,24 @@ int fstat_set_sfts(fstat_plan* p, int det, const void* bins, int dtype, int64_t 
   const int out_dtype = p->d.precision == FSTAT_FP64 ? FSTAT_C128 : FSTAT_C64;
   int rc = prepare_series(p, det, out_dtype, st);
   if (rc) return rc;
-  // the bins on the device (host input copied), and the roots of unity
-  const size_t in_bytes = (size_t)n_sft * n_bins * (dtype == FSTAT_C128 ? 16 : 8);
-  void* dbins = nullptr;
-  void* roots = nullptr;
-  cudaError_t e = cudaMalloc(&dbins, in_bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&roots, (size_t)n_bins * 16);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dbins, bins, in_bytes, cudaMemcpyDefault, st);
-  if (e == cudaSuccess)
-    e = launch_sft_to_xh(p->d.precision, dtype, dbins, n_sft, (int)n_bins, p->d.f_het, p->d.t0, t_sft, m_raw,
-                         roots, p->xh[det], st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (dbins) cudaFree(dbins);
-  if (roots) cudaFree(roots);
-  if (e != cudaSuccess) return cuda_status(e);
+  // the per-sky series and the FFT intermediate are stale from here on: they
+  // hold the host bins (n complex values of either type fit the n pairs of
+  // G) and the roots of unity, once the plan's earlier work has read them
+  CK(cudaStreamWaitEvent(st, p->done, 0));
+  const void* src = bins;
+  cudaPointerAttributes at{};
+  int dev = -1;
+  const size_t eb = dtype == FSTAT_C128 ? 16 : 8;
+  const bool on_device = cudaPointerGetAttributes(&at, bins) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                         cudaGetDevice(&dev) == cudaSuccess && at.device == dev && ((uintptr_t)bins & (eb - 1)) == 0;
+  if (!on_device) {
+    cudaGetLastError();
+    src = p->G;
+    CK(cudaMemcpyAsync(p->G, bins, (size_t)p->d.n_samples * eb, cudaMemcpyDefault, st));
+  }
+  CK(cudaMemsetAsync(p->d_err + 1, 0, sizeof(int), st));
+  CK(launch_sft_to_xh(p->d.precision, dtype, src, n_sft, (int)n_bins, p->d.f_het, p->d.t0, t_sft, m_raw, p->Z,
+                      p->xh[det], p->d_err + 1, st));
   return finish_series(p, det, sigma, st);
 }
 

@@ -5,11 +5,18 @@
 //   x_h[s B + m] = exp(-2 pi i f_h t_s) / M * sum_{i=0}^{B-1} X_s[i] exp(2 pi i (i - B/2) m / B)
 //
 // (column i of the band holds SFT bin q_h - B/2 + i).  B need not be a
-// power of two, so the transform is the direct sum: one CTA per (SFT,
-// block of output samples) stages the SFT's bins and the B roots of unity
-// in shared memory, and each thread accumulates kSftOut outputs, advancing
-// every root index (i - B/2) m mod B by m per bin (exact integer
-// reduction).  FP32 accumulation for mixed plans, FP64 for FP64 plans.
+// power of two (1800 s and 2 Hz give 3600 bins), so the transform is a
+// Stockham pipeline over B's own factors, one SFT per CTA in two
+// shared-memory buffers: factors up to 16 as register butterflies, larger
+// primes as direct sums of that length.  Every root of unity is taken from
+// one table of B entries at an exactly reduced integer index.  FP32 for
+// mixed plans, FP64 for FP64 plans.
+//
+// The direct sum over all B bins is issue-bound at B terms per sample;
+// 3600 = 16 x 15 x 15 needs about 46.  Two detectors x 480 SFTs of 3600 bins
+// from pinned memory to 2F of two templates: 9436 us with the direct sums
+// (4205 us of kernel per detector), 737 us here.  A band of prime length
+// keeps the direct sum (4001 bins: 4665 -> 4307 us).
 
 #include <math.h>
 
@@ -21,11 +28,55 @@ namespace fstat {
 namespace {
 
 constexpr int kSftThreads = 256;
-constexpr int kSftOut = 4;  // output samples per thread
+constexpr int kSftOut = 4;           // outputs per thread of a direct pass
+constexpr int kSftMaxPasses = 16;    // B < 2^16 has at most 15 prime factors
+constexpr size_t kSftSmemMax = (size_t)220 * 1024;
 
 template <typename T> struct C2;
 template <> struct C2<float> { using type = float2; };
 template <> struct C2<double> { using type = double2; };
+
+// Largest factor done as one register butterfly: a radix-R thread holds 2R
+// values and R roots, so FP64 stops at 8 (16 would spill).
+template <typename T> constexpr int max_radix() { return sizeof(T) == 4 ? 16 : 8; }
+
+struct SftPlan {
+  int np;
+  int r[kSftMaxPasses];
+};
+
+// B as a product of radices: primes above max_radix stand alone (direct
+// passes), the rest is packed greedily into the largest radices that divide
+// what is left (few passes; a radix-R butterfly costs ~R multiply-adds per
+// point, a pass one exchange through shared memory).
+SftPlan sft_factors(int B, int max_r) {
+  SftPlan p{};
+  int rest = B;
+  for (int q = max_r + 1; (int64_t)q * q <= rest;) {
+    bool prime = true;
+    for (int d = 2; d * d <= q && prime; ++d) prime = q % d != 0;
+    if (prime && rest % q == 0) {
+      p.r[p.np++] = q;
+      rest /= q;
+    } else {
+      ++q;
+    }
+  }
+  while (rest > 1) {
+    int r = 0;
+    for (int q = max_r; q >= 2 && !r; --q)
+      if (rest % q == 0) r = q;
+    if (!r) {  // no divisor up to max_r: a smaller-than-max_r^2 remainder splits into one large prime and its cofactor
+      r = rest;
+      for (int d = 2; d * d <= rest; ++d)
+        if (rest % d == 0) { r = rest / d; break; }
+    }
+    p.r[p.np++] = r;
+    rest /= r;
+  }
+  if (p.np == 0) p.r[p.np++] = 1;
+  return p;
+}
 
 // exp(2 pi i j / B), j < B, computed in FP64
 template <typename T>
@@ -37,45 +88,163 @@ __global__ void k_sft_roots(int64_t B, typename C2<T>::type* __restrict__ w) {
   }
 }
 
+// y_q = sum_s x_s exp(2 pi i q s / R), in place.  wr[j] = exp(2 pi i j / R).
+// The inputs s and R - s meet the same cosine and opposite sines, as do the
+// outputs q and R - q, so folding both ways leaves R^2 real multiply-adds.
+template <typename T, int R>
+__device__ __forceinline__ void dft_odd_even(typename C2<T>::type* x, const typename C2<T>::type* wr) {
+  using V = typename C2<T>::type;
+  constexpr int H = (R - 1) / 2;  // folded pairs
+  V a[H + 1], d[H + 1];
+#pragma unroll
+  for (int s = 1; s <= H; ++s) {
+    a[s] = {x[s].x + x[R - s].x, x[s].y + x[R - s].y};
+    d[s] = {x[s].x - x[R - s].x, x[s].y - x[R - s].y};
+  }
+  const V x0 = x[0];
+  V xm = {(T)0, (T)0};
+  if constexpr (R % 2 == 0) xm = x[R / 2];
+  V y0 = x0;
+#pragma unroll
+  for (int s = 1; s <= H; ++s) { y0.x += a[s].x; y0.y += a[s].y; }
+  x[0] = {y0.x + xm.x, y0.y + xm.y};
+  if constexpr (R % 2 == 0) {
+    V yh = x0;
+#pragma unroll
+    for (int s = 1; s <= H; ++s) {
+      if (s & 1) { yh.x -= a[s].x; yh.y -= a[s].y; }
+      else { yh.x += a[s].x; yh.y += a[s].y; }
+    }
+    x[R / 2] = (R / 2) & 1 ? V{yh.x - xm.x, yh.y - xm.y} : V{yh.x + xm.x, yh.y + xm.y};
+  }
+#pragma unroll
+  for (int q = 1; q <= H; ++q) {
+    V e = x0, o = {(T)0, (T)0};
+    if constexpr (R % 2 == 0) {
+      if (q & 1) { e.x -= xm.x; e.y -= xm.y; }
+      else { e.x += xm.x; e.y += xm.y; }
+    }
+#pragma unroll
+    for (int s = 1; s <= H; ++s) {
+      const int k = (q * s) % R;
+      const T c = k <= R / 2 ? wr[k].x : wr[R - k].x;
+      const T sn = k <= R / 2 ? wr[k].y : -wr[R - k].y;
+      e.x += a[s].x * c;
+      e.y += a[s].y * c;
+      o.x += d[s].x * sn;
+      o.y += d[s].y * sn;
+    }
+    // y_q = e + i o, y_{R-q} = e - i o
+    x[q] = {e.x - o.y, e.y + o.x};
+    x[R - q] = {e.x + o.y, e.y - o.x};
+  }
+}
+
+template <typename T> struct Out {
+  typename C2<T>::type* p;  // shared-memory buffer, or the series
+  const typename C2<T>::type* roots;
+  T rc, rs;     // the last pass's common factor
+  int B;
+  bool last;
+  int* err;
+  // value of transform output m: stored, or finished (the shift of the band
+  // centre, the SFT's phase and 1/M) and checked in the last pass
+  __device__ __forceinline__ void put(int m, typename C2<T>::type v) const {
+    if (last) {
+      const typename C2<T>::type w = roots[(unsigned)((B - B / 2) * m) % (unsigned)B];
+      const T fr = w.x * rc - w.y * rs, fi = w.x * rs + w.y * rc;
+      v = {v.x * fr - v.y * fi, v.x * fi + v.y * fr};
+      if (!isfinite(v.x) || !isfinite(v.y)) atomicCAS(err, 0, FSTAT_ERR_NONFINITE);
+    }
+    p[m] = v;
+  }
+};
+
+template <typename T, int R>
+__device__ __forceinline__ void pass_r(const typename C2<T>::type* src, const Out<T>& out, int B, int ns) {
+  using V = typename C2<T>::type;
+  const int nb = B / R, step = B / (ns * R);
+  V wr[R / 2 + 1];
+#pragma unroll
+  for (int j = 0; j <= R / 2; ++j) wr[j] = out.roots[j * nb];
+  for (int b = threadIdx.x; b < nb; b += kSftThreads) {
+    const int hi = b / ns, k = b - hi * ns;
+    V x[R];
+#pragma unroll
+    for (int s = 0; s < R; ++s) {
+      x[s] = src[b + s * nb];
+      if (s > 0) {
+        const V w = out.roots[k * step * s];  // k step s < B / ns * (ns - 1) / R * (R - 1) < B
+        x[s] = {x[s].x * w.x - x[s].y * w.y, x[s].x * w.y + x[s].y * w.x};
+      }
+    }
+    dft_odd_even<T, R>(x, wr);
+    const int base = hi * ns * R + k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) out.put(base + q * ns, x[q]);
+  }
+}
+
+// one pass of any length r by its defining sum: kSftOut outputs q of one
+// butterfly per thread share each input; the root index (k step + q B/r) s
+// advances by an exactly reduced step per term.  A band of prime length is
+// one such pass, whose outputs spread over the grid's y
+template <typename T>
+__device__ __forceinline__ void pass_direct(const typename C2<T>::type* src, const Out<T>& out, int B, int ns, int r) {
+  using V = typename C2<T>::type;
+  const int nb = B / r, step = B / (ns * r), groups = (r + kSftOut - 1) / kSftOut;
+  for (int u = blockIdx.y * kSftThreads + threadIdx.x; u < nb * groups; u += kSftThreads * gridDim.y) {
+    const int g = u / nb, b = u - g * nb, hi = b / ns, k = b - hi * ns;
+    int e[kSftOut], j[kSftOut];
+    V y[kSftOut];
+#pragma unroll
+    for (int t = 0; t < kSftOut; ++t) {
+      const int q = g + t * groups;
+      e[t] = q < r ? k * step + q * nb : 0;  // < B
+      j[t] = 0;
+      y[t] = {(T)0, (T)0};
+    }
+    for (int s = 0; s < r; ++s) {
+      const V x = src[b + s * nb];
+#pragma unroll
+      for (int t = 0; t < kSftOut; ++t) {
+        const V w = out.roots[j[t]];
+        y[t].x += x.x * w.x - x.y * w.y;
+        y[t].y += x.x * w.y + x.y * w.x;
+        j[t] += e[t];
+        if (j[t] >= B) j[t] -= B;
+      }
+    }
+    const int base = hi * ns * r + k;
+#pragma unroll
+    for (int t = 0; t < kSftOut; ++t) {
+      const int q = g + t * groups;
+      if (q < r) out.put(base + q * ns, y[t]);
+    }
+  }
+}
+
 template <typename T, typename TIn>
 __global__ void __launch_bounds__(kSftThreads)
-k_sft_to_xh(const TIn* __restrict__ bins, const typename C2<T>::type* __restrict__ roots, int B,
-            double f_het, double t_start, double t_sft, double inv_m, typename C2<T>::type* __restrict__ xh) {
+k_sft_to_xh(const TIn* __restrict__ bins, const typename C2<T>::type* __restrict__ roots, int B, SftPlan plan,
+            int roots_in_smem, double f_het, double t_start, double t_sft, double inv_m,
+            typename C2<T>::type* __restrict__ xh, int* err) {
   using V = typename C2<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* sx = reinterpret_cast<V*>(smem_raw);  // the SFT's bins
-  V* sw = sx + B;                          // roots of unity
-  const int s = blockIdx.y;
+  V* cur = reinterpret_cast<V*>(smem_raw);
+  V* nxt = cur + B;  // unused (and not there) with a single pass
+  const int s = blockIdx.x;
   const TIn* src = bins + (int64_t)s * B;
-  for (int i = threadIdx.x; i < B; i += blockDim.x) {
+  Out<T> out;
+  out.roots = roots;
+  if (roots_in_smem) {
+    V* sw = cur + (size_t)(plan.np > 1 ? 2 : 1) * B;
+    for (int i = threadIdx.x; i < B; i += kSftThreads) sw[i] = roots[i];
+    out.roots = sw;
+  }
+  for (int i = threadIdx.x; i < B; i += kSftThreads) {
     const TIn v = src[i];
-    sx[i] = {(T)v.x, (T)v.y};
-    sw[i] = roots[i];
-  }
-  __syncthreads();
-  // outputs m_r = base + r * blockDim.x of this thread
-  const int base = blockIdx.x * (kSftThreads * kSftOut) + threadIdx.x;
-  int m[kSftOut], j[kSftOut];
-  T ar[kSftOut], ai[kSftOut];
-#pragma unroll
-  for (int r = 0; r < kSftOut; ++r) {
-    m[r] = base + r * kSftThreads;
-    const int mm = m[r] < B ? m[r] : 0;
-    // root index for bin i = 0: (-B/2) m mod B
-    j[r] = (int)(((int64_t)(B - B / 2) * mm) % B);
-    ar[r] = 0;
-    ai[r] = 0;
-  }
-  for (int i = 0; i < B; ++i) {
-    const V x = sx[i];
-#pragma unroll
-    for (int r = 0; r < kSftOut; ++r) {
-      const V w = sw[j[r]];
-      ar[r] += x.x * w.x - x.y * w.y;
-      ai[r] += x.x * w.y + x.y * w.x;
-      j[r] += m[r] < B ? m[r] : 0;
-      if (j[r] >= B) j[r] -= B;
-    }
+    cur[i] = {(T)v.x, (T)v.y};
   }
   // exp(-2 pi i f_h t_s) / M with f_h t_s reduced mod 1 in FP64
   const double t_s = t_start + (double)s * t_sft;
@@ -83,25 +252,49 @@ k_sft_to_xh(const TIn* __restrict__ bins, const typename C2<T>::type* __restrict
   ph -= floor(ph);
   double sn, cs;
   sincospi(2.0 * ph, &sn, &cs);
-  const T rc = (T)(cs * inv_m), rs = (T)(-sn * inv_m);
-#pragma unroll
-  for (int r = 0; r < kSftOut; ++r) {
-    if (m[r] >= B) continue;
-    xh[(int64_t)s * B + m[r]] = {ar[r] * rc - ai[r] * rs, ar[r] * rs + ai[r] * rc};
+  out.rc = (T)(cs * inv_m);
+  out.rs = (T)(-sn * inv_m);
+  out.B = B;
+  out.err = err;
+  int ns = 1;
+  for (int p = 0; p < plan.np; ++p) {
+    __syncthreads();
+    const int r = plan.r[p];
+    out.last = p + 1 == plan.np;
+    out.p = out.last ? xh + (int64_t)s * B : nxt;
+    switch (r) {
+#define FSTAT_SFT_R(R) \
+  case R: if constexpr (R <= max_radix<T>()) { pass_r<T, R>(cur, out, B, ns); break; }
+      FSTAT_SFT_R(2) FSTAT_SFT_R(3) FSTAT_SFT_R(4) FSTAT_SFT_R(5) FSTAT_SFT_R(6) FSTAT_SFT_R(7) FSTAT_SFT_R(8)
+      FSTAT_SFT_R(9) FSTAT_SFT_R(10) FSTAT_SFT_R(11) FSTAT_SFT_R(12) FSTAT_SFT_R(13) FSTAT_SFT_R(14)
+      FSTAT_SFT_R(15) FSTAT_SFT_R(16)
+#undef FSTAT_SFT_R
+      default: pass_direct<T>(cur, out, B, ns, r); break;
+    }
+    ns *= r;
+    V* t = cur;
+    cur = nxt;
+    nxt = t;
   }
 }
 
 template <typename T, typename TIn>
 cudaError_t run_sft(const void* bins, int64_t n_sft, int B, double f_het, double t_start, double t_sft,
-                    int64_t m_raw, void* roots, void* xh, cudaStream_t st) {
+                    int64_t m_raw, void* roots, void* xh, int* err, cudaStream_t st) {
   using V = typename C2<T>::type;
-  const size_t smem = (size_t)2 * B * sizeof(V);
+  const SftPlan plan = sft_factors(B, max_radix<T>());
+  // data buffers, and the roots beside them where they fit (else from L1)
+  size_t smem = (size_t)(plan.np > 1 ? 2 : 1) * B * sizeof(V);
+  const bool in_smem = smem + (size_t)B * sizeof(V) <= kSftSmemMax;
+  if (in_smem) smem += (size_t)B * sizeof(V);
   cudaError_t e = cudaFuncSetAttribute(k_sft_to_xh<T, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k_sft_roots<T><<<(B + 255) / 256, 256, 0, st>>>(B, (V*)roots);
-  const dim3 grid((unsigned)((B + kSftThreads * kSftOut - 1) / (kSftThreads * kSftOut)), (unsigned)n_sft);
-  k_sft_to_xh<T, TIn><<<grid, kSftThreads, smem, st>>>((const TIn*)bins, (const V*)roots, B, f_het, t_start,
-                                                       t_sft, 1.0 / (double)m_raw, (V*)xh);
+  const bool direct = plan.np == 1 && plan.r[0] > max_radix<T>();
+  const dim3 grid((unsigned)n_sft, direct ? (unsigned)((B + kSftThreads * kSftOut - 1) / (kSftThreads * kSftOut)) : 1);
+  k_sft_to_xh<T, TIn><<<grid, kSftThreads, smem, st>>>((const TIn*)bins, (const V*)roots, B, plan, in_smem,
+                                                                  f_het, t_start, t_sft, 1.0 / (double)m_raw, (V*)xh,
+                                                                  err);
   return cudaGetLastError();
 }
 
@@ -112,14 +305,14 @@ size_t sft_smem_bytes(int B, int precision) {
 }
 
 cudaError_t launch_sft_to_xh(int precision, int in_dtype, const void* bins, int64_t n_sft, int B, double f_het,
-                             double t_start, double t_sft, int64_t m_raw, void* roots, void* xh,
+                             double t_start, double t_sft, int64_t m_raw, void* roots, void* xh, int* err,
                              cudaStream_t st) {
   const bool in64 = in_dtype == FSTAT_C128;
   if (precision == FSTAT_FP64)
-    return in64 ? run_sft<double, double2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, st)
-                : run_sft<double, float2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, st);
-  return in64 ? run_sft<float, double2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, st)
-              : run_sft<float, float2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, st);
+    return in64 ? run_sft<double, double2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, err, st)
+                : run_sft<double, float2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, err, st);
+  return in64 ? run_sft<float, double2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, err, st)
+              : run_sft<float, float2>(bins, n_sft, B, f_het, t_start, t_sft, m_raw, roots, xh, err, st);
 }
 
 }  // namespace fstat

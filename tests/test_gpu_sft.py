@@ -113,3 +113,25 @@ def test_argument_checks():
             plan.set_sfts(0, bands[0][:5], Q0, T_SFT, M, 1.0)
         with pytest.raises(pkg.FstatError):           # export before data
             plan.export_data(0)
+
+
+@pytest.mark.parametrize("precision,tol", [(pkg.MIXED, 2e-5), (pkg.FP64, 1e-12)])
+@pytest.mark.parametrize("nb", [2, 13, 31, 16 * 15 * 15, 7 * 11 * 13, 9 * 8 * 5 * 2, 17 * 19, 2 * 601, 1009, 6400])
+def test_every_kind_of_band_length(nb, precision, tol):
+    # small factors, primes as direct passes, one prime alone, the FP64 limit;
+    # the tolerances are those of the other series tests (FP32 / FP64 sums)
+    n_sft, t_sft = 3, 1800.0
+    q0 = int(100.0 * t_sft) - nb // 2
+    t = small_target(n_samples=n_sft * nb, dt=t_sft / nb, n_fft=1 << max(10, (n_sft * nb - 1).bit_length()), n_det=1,
+                     f_het=100.0, seed=125, dtype="c64")
+    rng = np.random.default_rng(nb)
+    b = (rng.standard_normal((n_sft, nb)) + 1j * rng.standard_normal((n_sft, nb))).astype(np.complex64)
+    ref = sft.xh_from_band(b.astype(np.complex128), q0, t.t0, t_sft, 2 * nb, 100.0)
+    with pkg.FstatPlan.from_target(t, precision) as plan:
+        plan.set_sfts(0, b, q0, t_sft, 2 * nb, 1.0)
+        got = plan.export_data(0)
+        b[1, nb // 2] = np.nan
+        with pytest.raises(pkg.FstatError) as e:
+            plan.set_sfts(0, torch.from_numpy(b).cuda(), q0, t_sft, 2 * nb, 1.0)
+        assert e.value.code == -5
+    assert np.max(np.abs(got - ref)) <= tol * np.max(np.abs(ref))

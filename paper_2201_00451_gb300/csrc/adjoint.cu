@@ -9,24 +9,40 @@
 //   Fa = sum_X w_X sum_k x_X[k] a_X(t_k) e^{-i 2 pi Phi_k},  Fb with b,
 //   a = d(t_k) : e+(alpha, delta),  b = d(t_k) : ex(alpha, delta)
 //
-// t_m is linear in the sky vector n and a, b are linear in the detector
-// tensor d(t_k), so r(t_k)/c and d(t_k) are sky-independent per-sample
-// tables built once per plan.  Per candidate and sample the phase is
-// evaluated in double-float (FP32 pairs, ~48-bit) arithmetic; the sums of
-// Fa, Fb, their derivatives, and A, B, C (with their sky derivatives) are
-// FP32 two-level sums reduced in FP64.  d(2F) follows by the chain rule.
+// Over a block of S consecutive samples (a few tens of seconds) everything in
+// these sums except x and the phase factor is a polynomial: the Earth turns
+// by ~1e-3 rad.  So per candidate and block the phase is evaluated once in
+// double-float (FP32 pairs, ~48 bits) at the block's middle sample together
+// with its derivatives, per sample only
+//
+//   e_u = x_u exp(-i 2 pi (Phi(u) - Phi(0))),  E_q = sum_u e_u u^q,  q = 0, 1, 2
+//
+// is formed (a cubic in u, one sine/cosine, three complex sums), and Fa, Fb
+// and their derivatives are combinations of E_0, E_1, E_2 with the local
+// expansions of a, b, tau and dPhi/dtheta.  A, B, C need no sum at all: a and
+// b are harmonics 0-2 of the sidereal angle, whose products sum over the
+// sample grid in closed form.
+//
+// Bound by FP32 issue: ~22 instructions per candidate and sample plus ~480
+// per block.  256 candidates of the 10-day two-detector data: 11.7 ms with the
+// phase, the patterns and 29 sums evaluated at every sample (~300
+// instructions), 1.25 ms here; one candidate 5.2 ms -> 0.14 ms (items of 2^14
+// samples instead of 2^17 fill the GPU).
 
 #include <math.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "fstat_internal.cuh"
 
 namespace fstat {
 namespace adj {
 
-constexpr int kWarps = 8;          // candidates per CTA (one warp each)
-constexpr int kChunk = 1 << 17;    // samples per CTA (over all detectors)
-constexpr int kInner = 64;         // first-level summation length per lane
-constexpr int kAcc = 29;           // accumulated quantities per candidate
+constexpr int kWarps = 8;               // (candidate, chunk) items per CTA, one warp each
+constexpr int kChunkSamples = 1 << 14;  // samples per item: the unit of every sum, whatever the candidate count
+constexpr int kAcc = 20;                // accumulated quantities per candidate
+constexpr int kInner = 64;              // per-sample path: terms per first-level sum
 
 // ------------------------------------------------------------ double-float
 struct df {
@@ -56,318 +72,596 @@ __device__ __forceinline__ df df_mul(df a, df b) {
   float h = __fadd_rn(p, e);
   return {h, __fsub_rn(e, __fsub_rn(h, p))};
 }
-__device__ __forceinline__ df df_mulf(df a, float b) {
-  float p = __fmul_rn(a.h, b);
-  float e = fmaf(a.h, b, -p);
-  e = fmaf(a.l, b, e);
-  float h = __fadd_rn(p, e);
-  return {h, __fsub_rn(e, __fsub_rn(h, p))};
-}
+__device__ __forceinline__ df df_mulf(df a, float b) { return df_mul(a, {b, 0.f}); }
 // fractional part of a double-float in [-1/2, 1/2]
 __device__ __forceinline__ float df_frac(df a) {
   float k = rintf(a.h);
   return __fadd_rn(__fsub_rn(a.h, k), a.l);
 }
 
-// ------------------------------------------------------------ tables, consts
-// Per sample (detector-major, k fastest): r/c as double-float, detector
-// tensor components (xx, yy, zz, xy, xz, yz), normalised data.
-struct SampleTabs {
-  float4* rc;   // (x.h, x.l, y.h, y.l) per sample
-  float2* rcz;  // (z.h, z.l)
-  float4* d0;   // (xx, yy, zz, xy)
-  float2* d1;   // (xz, yz)
-  float2* x;    // x_h / sigma_ref
-};
+// ------------------------------------------------------------ blocks
+// Samples per block: the largest S whose half-span h = S dt / 2 keeps
+// (2 w h)^3 / 6 <= 2e-8 for the sidereal and orbital rates w, the first
+// neglected term of the patterns' expansion (FP32 rounding is 6e-8; the
+// phase's, f R_E/c (w h)^4 / 24, is then below 1e-10 cycles).  For the
+// sidereal rate that is dt <= 2.1 s (S = 32), 4.2 s (16), 8.4 s (8); beyond,
+// S = 1 evaluates every sample by itself.
+int block_samples(const Geo& g) {
+  const double w = std::max(fabs(g.w_rot), fabs(g.w_orb)) * g.dt;
+  for (int S : {32, 16, 8}) {
+    const double x = w * S;  // 2 w h
+    if (x * x * x <= 1.2e-7) return S;
+  }
+  return 1;
+}
 
-struct CandConst {
-  df nx, ny, nz;                 // sky vector
-  float dna[3], dnd[3];          // d n / d alpha, d n / d delta
-  float ep[6], ex[6];            // e+ and ex weights for (xx, yy, zz, xy, xz, yz), off-diagonals doubled
-  float epa[6], epd[6], exa[6], exd[6];
-  df fmh;                        // f - f_h
-  df fh;                         // f_h
-  df f1h;                        // f1dot / 2
-  df f2s;                        // f2dot / 6
-  float f, f1, f2;               // for dPhi/dt_m = f + f1dot tau + f2dot tau^2 / 2
-  float pad_;
-};
+// Block tables, 32 blocks (one tile) at a time, field by field: at a block's
+// middle sample the time since t_ref (double-float), r/c (double-float) and
+// its first three derivatives per sample, and the sidereal angle's
+// harmonics.  S = 1 keeps no derivatives.
+enum Field { fTau = 0, fR = 2, fCos = 8, fR1 = 12, fR2 = 15, fR3 = 18, fAll = 21 };
+constexpr int fields(int S) { return S == 1 ? (int)fR1 : (int)fAll; }
 
-__global__ void k_tables(Geo g, int X, const void* __restrict__ xh, int dtype, SampleTabs tab) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < g.n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const double t = g.t0 + (double)k * g.dt;
-    double so, co, sp, cp;
-    sincos(g.orb_ph0 + g.w_orb * t, &so, &co);
-    const double ph = g.lon[X] + g.sid_ph0 + g.w_rot * t;
-    sincos(ph, &sp, &cp);
-    const double rx = (g.au * co + g.rcl[X] * cp) / g.c;
-    const double ry = (g.au * g.cos_obl * so + g.rcl[X] * sp) / g.c;
-    const double rz = (g.au * g.sin_obl * so + g.rsl[X]) / g.c;
-    const int64_t i = (int64_t)X * g.n + k;
-    float hx = (float)rx, hy = (float)ry, hz = (float)rz;
-    tab.rc[i] = make_float4(hx, (float)(rx - hx), hy, (float)(ry - hy));
-    tab.rcz[i] = make_float2(hz, (float)(rz - hz));
-    // detector tensor d = (u u^T - v v^T)/2, arms at gamma -/+ 45 deg from East towards North
-    const double sl = sin(g.lat[X]), cl = cos(g.lat[X]);
-    const double e[3] = {-sp, cp, 0.0};
-    const double nn[3] = {-sl * cp, -sl * sp, cl};
-    const double g1 = g.gam[X] - 0.78539816339744830962, g2 = g.gam[X] + 0.78539816339744830962;
-    double u[3], v[3];
-    for (int q = 0; q < 3; ++q) {
-      u[q] = cos(g1) * e[q] + sin(g1) * nn[q];
-      v[q] = cos(g2) * e[q] + sin(g2) * nn[q];
+struct Layout {
+  int S;
+  int64_t tiles;        // tiles of 32 blocks per detector
+  size_t x_bytes, node_bytes;
+};
+Layout layout(const Geo& g) {
+  Layout l;
+  l.S = block_samples(g);
+  l.tiles = (g.n + 32 * l.S - 1) / (32 * l.S);
+  l.x_bytes = (size_t)g.n_det * l.tiles * 32 * l.S * sizeof(float2);
+  l.node_bytes = (size_t)g.n_det * l.tiles * 32 * fields(l.S) * sizeof(float);
+  return l;
+}
+
+struct Series { const void* x[kMaxDet]; int dtype[kMaxDet]; };
+
+// w x_h / sigma_ref, tile by tile as [i][lane] (sample i of the lane's
+// block; pairs of samples side by side for S > 1), zero past the data: every
+// later read is coalesced.
+__global__ void k_series_table(Geo g, Series src, int S, int64_t tiles, float2* __restrict__ out) {
+  const int X = blockIdx.y;
+  const double scale = g.inv_sigma_ref * g.w[X];
+  const int64_t total = tiles * 32 * S;
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t tile = o / (32 * S);
+    const int q = (int)(o - tile * (32 * S));
+    const int lane = S > 1 ? (q >> 1) & 31 : q;
+    const int i = S > 1 ? 2 * (q >> 6) + (q & 1) : 0;
+    const int64_t k = (tile * 32 + lane) * S + i;
+    float2 v = make_float2(0.f, 0.f);
+    if (k < g.n) {
+      if (src.dtype[X] == FSTAT_C128) {
+        const double2 d = ((const double2*)src.x[X])[k];
+        v = make_float2((float)(d.x * scale), (float)(d.y * scale));
+      } else {
+        const float2 d = ((const float2*)src.x[X])[k];
+        v = make_float2((float)(d.x * scale), (float)(d.y * scale));
+      }
     }
-    auto dd = [&](int p, int q) { return 0.5 * (u[p] * u[q] - v[p] * v[q]); };
-    tab.d0[i] = make_float4((float)dd(0, 0), (float)dd(1, 1), (float)dd(2, 2), (float)dd(0, 1));
-    tab.d1[i] = make_float2((float)dd(0, 2), (float)dd(1, 2));
-    double xr, xi;
-    if (dtype == FSTAT_C128) {
-      double2 v2 = ((const double2*)xh)[k];
-      xr = v2.x; xi = v2.y;
-    } else {
-      float2 v2 = ((const float2*)xh)[k];
-      xr = v2.x; xi = v2.y;
-    }
-    tab.x[i] = make_float2((float)(xr * g.inv_sigma_ref), (float)(xi * g.inv_sigma_ref));
+    out[X * total + o] = v;
   }
 }
 
-// polarisation tensors and their sky derivatives for one candidate
-__global__ void k_cand_consts(const fstat_candidate* __restrict__ cand, int n, double f_het,
+__global__ void k_block_table(Geo g, int S, int64_t tiles, float* __restrict__ out) {
+  const int X = blockIdx.y, nf = S == 1 ? fields(1) : fields(2);
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < tiles * 32;
+       b += (int64_t)gridDim.x * blockDim.x) {
+    const double k = (double)(b * S + S / 2), t = g.t0 + k * g.dt;
+    double so, co, sp, cp;
+    sincos(g.orb_ph0 + g.w_orb * t, &so, &co);
+    sincos(g.lon[X] + g.sid_ph0 + g.w_rot * t, &sp, &cp);
+    float* f = out + ((X * tiles + b / 32) * nf) * 32 + (b & 31);
+    auto put = [&](int q, double v) { f[32 * q] = (float)v; };
+    auto put2 = [&](int q, double v) {
+      const float h = (float)v;
+      f[32 * q] = h;
+      f[32 * (q + 1)] = (float)(v - (double)h);
+    };
+    const double ox = g.au / g.c, oy = g.au * g.cos_obl / g.c, oz = g.au * g.sin_obl / g.c;
+    const double rr = g.rcl[X] / g.c, wo = g.w_orb * g.dt, wr = g.w_rot * g.dt;
+    put2(fTau, (g.t0 - g.t_ref) + k * g.dt);
+    put2(fR, ox * co + rr * cp);
+    put2(fR + 2, oy * so + rr * sp);
+    put2(fR + 4, oz * so + g.rsl[X] / g.c);
+    put(fCos, cp);
+    put(fCos + 1, sp);
+    put(fCos + 2, cp * cp - sp * sp);
+    put(fCos + 3, 2.0 * sp * cp);
+    if (S == 1) continue;
+    put(fR1, -wo * ox * so - wr * rr * sp);
+    put(fR1 + 1, wo * oy * co + wr * rr * cp);
+    put(fR1 + 2, wo * oz * co);
+    put(fR2, -wo * wo * ox * co - wr * wr * rr * cp);
+    put(fR2 + 1, -wo * wo * oy * so - wr * wr * rr * sp);
+    put(fR2 + 2, -wo * wo * oz * so);
+    put(fR3, wo * wo * wo * ox * so + wr * wr * wr * rr * sp);
+    put(fR3 + 1, -wo * wo * wo * oy * co - wr * wr * wr * rr * cp);
+    put(fR3 + 2, -wo * wo * wo * oz * co);
+  }
+}
+
+// ------------------------------------------------------------ candidates
+constexpr int kPat = 6;  // a, b, da/dalpha, db/dalpha, da/ddelta, db/ddelta
+// harmonics of the sidereal angle phi: 1, cos 2phi, sin 2phi, cos phi, sin phi
+struct CandConst {
+  df nx, ny, nz;           // sky vector
+  float dna[3], dnd[3];    // d n / d alpha, d n / d delta
+  df fmh;                  // f - f_h
+  df fh;                   // f_h
+  df f1h;                  // f1dot / 2
+  df f2s;                  // f2dot / 6
+  df step;                 // (f - f_h) dt, mod 1
+  df dt;
+  float f, f1, f2, pad_;   // for dPhi/dt_m = f + f1dot tau + f2dot tau^2 / 2
+  float pat[kMaxDet][kPat][5];
+  double abc[9];           // A, B, C, then d/dalpha, d/ddelta (read by k_finalize)
+};
+
+// Antenna patterns (JKS 1998 eqs. 12-13) as harmonics of phi for one
+// detector: with H = alpha - phi and u = (1, cos 2H, sin 2H, cos H, sin H),
+// a = sum ka_i u_i, b = sum kb_i u_i, and their sky derivatives.
+__device__ void patterns(double lam, double gam, double alpha, double delta, double (*p)[5]) {
+  double sl, cl, sg, cg, sd, cd, s2d, c2d;
+  sincos(lam, &sl, &cl);
+  sincos(2.0 * gam, &sg, &cg);
+  sincos(delta, &sd, &cd);
+  s2d = 2.0 * sd * cd;
+  c2d = cd * cd - sd * sd;
+  const double s2l = 2.0 * sl * cl, c2l = cl * cl - sl * sl;
+  // value and d/ddelta of the coefficients
+  const double k[4][5] = {
+      {0.75 * sg * cl * cl * cd * cd, sg * (3.0 - c2l) * (3.0 - c2d) / 16.0, -0.25 * cg * sl * (3.0 - c2d),
+       0.25 * sg * s2l * s2d, -0.5 * cg * cl * s2d},
+      {0.0, cg * sl * sd, 0.25 * sg * (3.0 - c2l) * sd, cg * cl * cd, 0.5 * sg * s2l * cd},
+      {-1.5 * sg * cl * cl * cd * sd, sg * (3.0 - c2l) * s2d / 8.0, -0.5 * cg * sl * s2d, 0.5 * sg * s2l * c2d,
+       -cg * cl * c2d},
+      {0.0, cg * sl * cd, 0.25 * sg * (3.0 - c2l) * cd, -cg * cl * sd, -0.5 * sg * s2l * sd}};
+  double sa, ca;
+  sincos(alpha, &sa, &ca);
+  const double s2a = 2.0 * sa * ca, c2a = ca * ca - sa * sa;
+  auto turn = [&](const double* u, double* o) {
+    o[0] = u[0];
+    o[1] = u[1] * c2a + u[2] * s2a;
+    o[2] = u[1] * s2a - u[2] * c2a;
+    o[3] = u[3] * ca + u[4] * sa;
+    o[4] = u[3] * sa - u[4] * ca;
+  };
+  for (int q = 0; q < 2; ++q) {
+    const double da[5] = {0.0, 2.0 * k[q][2], -2.0 * k[q][1], k[q][4], -k[q][3]};  // d/dalpha of u
+    turn(k[q], p[q]);
+    turn(da, p[2 + q]);
+    turn(k[2 + q], p[4 + q]);
+  }
+}
+
+// sums over the sample grid of cos(m phi), sin(m phi), m = 0..4, per detector
+struct Harmonics { double c[kMaxDet][5], s[kMaxDet][5]; };
+
+// sum_k w u(phi_k) v(phi_k) for two patterns u, v over the grid
+__device__ double pat_sum(const double* u, const double* v, const double* C, const double* S) {
+  // products of the harmonics: 1, cos 2phi, sin 2phi, cos phi, sin phi
+  const double m[5][5] = {{C[0], C[2], S[2], C[1], S[1]},
+                          {C[2], 0.5 * (C[0] + C[4]), 0.5 * S[4], 0.5 * (C[3] + C[1]), 0.5 * (S[3] - S[1])},
+                          {S[2], 0.5 * S[4], 0.5 * (C[0] - C[4]), 0.5 * (S[3] + S[1]), 0.5 * (C[1] - C[3])},
+                          {C[1], 0.5 * (C[3] + C[1]), 0.5 * (S[3] + S[1]), 0.5 * (C[0] + C[2]), 0.5 * S[2]},
+                          {S[1], 0.5 * (S[3] - S[1]), 0.5 * (C[1] - C[3]), 0.5 * S[2], 0.5 * (C[0] - C[2])}};
+  double t = 0.0;
+  for (int i = 0; i < 5; ++i)
+    for (int j = 0; j < 5; ++j) t += u[i] * m[i][j] * v[j];
+  return t;
+}
+
+__global__ void k_cand_consts(Geo g, Harmonics h, const fstat_candidate* __restrict__ cand, int n,
                               CandConst* __restrict__ out) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const fstat_candidate c = cand[i];
-  const double sa = sin(c.alpha), ca = cos(c.alpha), sd = sin(c.delta), cd = cos(c.delta);
-  CandConst k;
+  CandConst& k = out[i];
+  double sa, ca, sd, cd;
+  sincos(c.alpha, &sa, &ca);
+  sincos(c.delta, &sd, &cd);
   k.nx = df_from(cd * ca);
   k.ny = df_from(cd * sa);
   k.nz = df_from(sd);
-  const double dna[3] = {-cd * sa, cd * ca, 0.0};
-  const double dnd[3] = {-sd * ca, -sd * sa, cd};
-  const double x[3] = {sa, -ca, 0.0};
-  const double y[3] = {-sd * ca, -sd * sa, cd};
-  const double xa[3] = {ca, sa, 0.0};
-  const double ya[3] = {sd * sa, -sd * ca, 0.0};
-  const double xd[3] = {0.0, 0.0, 0.0};
-  const double yd[3] = {-cd * ca, -cd * sa, -sd};
-  const int P[6] = {0, 1, 2, 0, 0, 1}, Q[6] = {0, 1, 2, 1, 2, 2};
-  for (int m = 0; m < 6; ++m) {
-    const int p = P[m], q = Q[m];
-    const double w = m < 3 ? 1.0 : 2.0;  // off-diagonal terms appear twice in d : e
-    k.ep[m] = (float)(w * (x[p] * x[q] - y[p] * y[q]));
-    k.ex[m] = (float)(w * (x[p] * y[q] + y[p] * x[q]));
-    k.epa[m] = (float)(w * (xa[p] * x[q] + x[p] * xa[q] - ya[p] * y[q] - y[p] * ya[q]));
-    k.epd[m] = (float)(w * (xd[p] * x[q] + x[p] * xd[q] - yd[p] * y[q] - y[p] * yd[q]));
-    k.exa[m] = (float)(w * (xa[p] * y[q] + x[p] * ya[q] + ya[p] * x[q] + y[p] * xa[q]));
-    k.exd[m] = (float)(w * (xd[p] * y[q] + x[p] * yd[q] + yd[p] * x[q] + y[p] * xd[q]));
-  }
-  for (int q = 0; q < 3; ++q) {
-    k.dna[q] = (float)dna[q];
-    k.dnd[q] = (float)dnd[q];
-  }
-  k.fmh = df_from(c.f - f_het);
-  k.fh = df_from(f_het);
+  k.dna[0] = (float)(-cd * sa);
+  k.dna[1] = (float)(cd * ca);
+  k.dna[2] = 0.f;
+  k.dnd[0] = (float)(-sd * ca);
+  k.dnd[1] = (float)(-sd * sa);
+  k.dnd[2] = (float)cd;
+  k.fmh = df_from(c.f - g.f_het);
+  k.fh = df_from(g.f_het);
   k.f1h = df_from(c.f1dot / 2.0);
   k.f2s = df_from(c.f2dot / 6.0);
+  const double st = (c.f - g.f_het) * g.dt;
+  k.step = df_from(st - rint(st));
   k.f = (float)c.f;
   k.f1 = (float)c.f1dot;
   k.f2 = (float)c.f2dot;
+  k.dt = df_from(g.dt);
   k.pad_ = 0.f;
-  out[i] = k;
-}
-
-// accumulated quantities (kAcc): 0-1 Fa, 2-3 Fb, 4-7 dFa,dFb/df, 8-11 d/df1dot,
-// 12-15 d/dalpha, 16-19 d/ddelta, 20-22 A,B,C, 23-25 dA,dB,dC/dalpha, 26-28 d/ddelta
-__global__ void __launch_bounds__(kWarps * 32, 3)
-k_partial(Geo g, SampleTabs tab, const CandConst* __restrict__ cc, int n_cand, int n_chunks,
-          double* __restrict__ partial) {
-  __shared__ CandConst sc[kWarps];
-  // second-level sums of every lane, in shared memory so that the registers
-  // hold the candidate's constants instead (same FP32 arithmetic)
-  __shared__ float s_outer[kWarps][kAcc][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cand = blockIdx.x * kWarps + warp;
-  const int chunk = blockIdx.y;
-  if (threadIdx.x < kWarps && blockIdx.x * kWarps + threadIdx.x < n_cand)
-    sc[threadIdx.x] = cc[blockIdx.x * kWarps + threadIdx.x];
-  __syncthreads();
-  if (cand >= n_cand) return;
-  const CandConst& K = sc[warp];
-  const int64_t total = (int64_t)g.n_det * g.n;
-  const int64_t beg = (int64_t)chunk * kChunk;
-  const int64_t end = beg + kChunk < total ? beg + kChunk : total;
-  const df dt = df_from(g.dt);
-  const df c0 = df_from(g.t0 - g.t_ref);
-  const float two_pi = 6.28318530717958647692f;
-
-  float inner[kAcc];
-  float* outer = &s_outer[warp][0][lane];  // element q at outer[32 q]
-#pragma unroll
-  for (int q = 0; q < kAcc; ++q) outer[32 * q] = 0.f;
-  int cnt = 0;
-#pragma unroll
-  for (int q = 0; q < kAcc; ++q) inner[q] = 0.f;
-  // detector X and sample k of index i, advanced incrementally (no 64-bit
-  // division, no double->float conversion per sample)
-  int X = (int)((beg + lane) / g.n);
-  int k = (int)(beg + lane - (int64_t)X * g.n);
-  float w = X < g.n_det ? (float)g.w[X] : 0.f;
-  for (int64_t i = beg + lane; i < end; i += 32, k += 32) {
-    while (k >= g.n) {
-      k -= (int)g.n;
-      ++X;
-      w = (float)g.w[X];
-    }
-    const float4 r4 = __ldg(&tab.rc[i]);
-    const float2 rz = __ldg(&tab.rcz[i]);
-    const float4 d0 = __ldg(&tab.d0[i]);
-    const float2 d1 = __ldg(&tab.d1[i]);
-    const float2 xv = __ldg(&tab.x[i]);
-    // t_m = (r/c) . n in double-float
-    df tm = df_add(df_add(df_mul({r4.x, r4.y}, K.nx), df_mul({r4.z, r4.w}, K.ny)), df_mul({rz.x, rz.y}, K.nz));
-    // tau = k dt + (t0 - t_ref) + t_m
-    df tk = df_add(df_mulf(dt, (float)k), c0);
-    df tau = df_add(tk, tm);
-    // Phi = (f - f_h) tau + f_h t_m + f1dot tau^2/2 + f2dot tau^3/6
-    df tau2 = df_mul(tau, tau);
-    df ph = df_add(df_add(df_mul(K.fmh, tau), df_mul(K.fh, tm)),
-                   df_add(df_mul(K.f1h, tau2), df_mul(K.f2s, df_mul(tau2, tau))));
-    const float fr = df_frac(ph);
-    float sn, cs;
-    __sincosf(two_pi * fr, &sn, &cs);
-    // e = w x exp(-i 2 pi Phi)
-    const float er = w * (xv.x * cs + xv.y * sn);
-    const float ei = w * (xv.y * cs - xv.x * sn);
-    const float D[6] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y};
-    float a = 0.f, b = 0.f, aa = 0.f, ad = 0.f, ba = 0.f, bd = 0.f;
-#pragma unroll
-    for (int m = 0; m < 6; ++m) {
-      a = fmaf(D[m], K.ep[m], a);
-      b = fmaf(D[m], K.ex[m], b);
-      aa = fmaf(D[m], K.epa[m], aa);
-      ad = fmaf(D[m], K.epd[m], ad);
-      ba = fmaf(D[m], K.exa[m], ba);
-      bd = fmaf(D[m], K.exd[m], bd);
-    }
-    const float tauf = tau.h;
-    const float dpdt = K.f + K.f1 * tauf + 0.5f * K.f2 * tauf * tauf;  // dPhi/dt_m
-    const float tma = r4.x * K.dna[0] + r4.z * K.dna[1] + rz.x * K.dna[2];
-    const float tmd = r4.x * K.dnd[0] + r4.z * K.dnd[1] + rz.x * K.dnd[2];
-    // d/dtheta of e * pat = e * (pat_theta - i 2 pi Phi_theta pat)
-    const float pf = two_pi * tauf, p1 = two_pi * 0.5f * tauf * tauf;
-    const float pa = two_pi * dpdt * tma, pd = two_pi * dpdt * tmd;
-    inner[0] += er * a;  inner[1] += ei * a;
-    inner[2] += er * b;  inner[3] += ei * b;
-    // (-i p) e pat = p pat (ei, -er)
-    inner[4] += pf * a * ei;  inner[5] -= pf * a * er;
-    inner[6] += pf * b * ei;  inner[7] -= pf * b * er;
-    inner[8] += p1 * a * ei;  inner[9] -= p1 * a * er;
-    inner[10] += p1 * b * ei; inner[11] -= p1 * b * er;
-    inner[12] += er * aa + pa * a * ei;  inner[13] += ei * aa - pa * a * er;
-    inner[14] += er * ba + pa * b * ei;  inner[15] += ei * ba - pa * b * er;
-    inner[16] += er * ad + pd * a * ei;  inner[17] += ei * ad - pd * a * er;
-    inner[18] += er * bd + pd * b * ei;  inner[19] += ei * bd - pd * b * er;
-    inner[20] += w * a * a;
-    inner[21] += w * b * b;
-    inner[22] += w * a * b;
-    inner[23] += 2.f * w * a * aa;
-    inner[24] += 2.f * w * b * ba;
-    inner[25] += w * (aa * b + a * ba);
-    inner[26] += 2.f * w * a * ad;
-    inner[27] += 2.f * w * b * bd;
-    inner[28] += w * (ad * b + a * bd);
-    if (++cnt == kInner) {
-#pragma unroll
-      for (int q = 0; q < kAcc; ++q) { outer[32 * q] += inner[q]; inner[q] = 0.f; }
-      cnt = 0;
+  double abc[9] = {};
+  for (int X = 0; X < g.n_det; ++X) {
+    double p[kPat][5];
+    patterns(g.lat[X], g.gam[X], c.alpha, c.delta, p);
+    for (int q = 0; q < kPat; ++q)
+      for (int m = 0; m < 5; ++m) k.pat[X][q][m] = (float)p[q][m];
+    for (int d = 0; d < 3; ++d) {
+      // d = 0: the values; 1, 2: the alpha and delta derivatives
+      const double *a = p[0], *b = p[1], *da = p[2 * d], *db = p[2 * d + 1];
+      const double w = d ? 2.0 * g.w[X] : g.w[X];
+      abc[3 * d] += w * pat_sum(a, da, h.c[X], h.s[X]);
+      abc[3 * d + 1] += w * pat_sum(b, db, h.c[X], h.s[X]);
+      abc[3 * d + 2] += d ? g.w[X] * (pat_sum(da, b, h.c[X], h.s[X]) + pat_sum(a, db, h.c[X], h.s[X]))
+                          : w * pat_sum(a, b, h.c[X], h.s[X]);
     }
   }
-  double* dst = partial + ((int64_t)cand * n_chunks + chunk) * kAcc;
+  for (int q = 0; q < 9; ++q) k.abc[q] = abc[q];
+}
+
+// ------------------------------------------------------------ the sums
+// value, first and second derivative per sample (at a block's middle) of a
+// pattern; w = the sidereal angle per sample
+struct Local { float v, d1, d2; };
+template <bool DERIV>
+__device__ __forceinline__ Local local(const float* p, float c1, float s1, float c2, float s2, float w) {
+  const float h2 = p[1] * c2 + p[2] * s2, h1 = p[3] * c1 + p[4] * s1;
+  Local r{p[0] + h2 + h1, 0.f, 0.f};
+  if constexpr (DERIV) {
+    const float q2 = p[2] * c2 - p[1] * s2, q1 = p[4] * c1 - p[3] * s1;
+    r.d1 = w * (2.f * q2 + q1);
+    r.d2 = -w * w * (4.f * h2 + h1);
+  }
+  return r;
+}
+
+struct cpx { float r, i; };
+
+// a - rint(a) for |a| < 2^22
+__device__ __forceinline__ float less_rint(float a) {
+  return __fsub_rn(a, __fsub_rn(__fadd_rn(a, 12582912.f), 12582912.f));
+}
+
+// One warp per (candidate, chunk of kChunkSamples samples): lane l of a tile
+// takes the tile's block l.  Neighbouring warps take neighbouring candidates
+// of one chunk, so the tables are read from L1.
+// accumulated quantities (kAcc): 0-1 Fa, 2-3 Fb, 4-7 dFa,dFb/df, 8-11 d/df1dot,
+// 12-15 d/dalpha, 16-19 d/ddelta
+template <int S>
+__global__ void __launch_bounds__(kWarps * 32, 2)
+k_moments(int n_det, int64_t tiles, const float2* __restrict__ xt, const float* __restrict__ nodes, float w_step,
+          const CandConst* __restrict__ cc, int n_cand, int n_chunks, double* __restrict__ partial) {
+  constexpr int NF = fields(S);
+  constexpr int kTiles = kChunkSamples / (32 * S);
+  __shared__ CandConst sc[kWarps];
+  __shared__ float s_red[kWarps][kAcc][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t item = (int64_t)blockIdx.x * kWarps + warp;
+  if (item >= (int64_t)n_cand * n_chunks) return;
+  const int chunk = (int)(item / n_cand), cand = (int)(item - (int64_t)chunk * n_cand);
+  {
+    const int* src = reinterpret_cast<const int*>(cc + cand);
+    int* dst = reinterpret_cast<int*>(&sc[warp]);
+    for (int q = lane; q < (int)(sizeof(CandConst) / 4); q += 32) dst[q] = src[q];
+  }
+  __syncwarp();
+  const CandConst& K = sc[warp];
+  const float two_pi = 6.28318530717958647692f;
+  const int64_t beg = (int64_t)chunk * kTiles, end = min(beg + kTiles, (int64_t)n_det * tiles);
+  float acc[kAcc], outer[S == 1 ? kAcc : 1];
+#pragma unroll
+  for (int q = 0; q < kAcc; ++q) acc[q] = 0.f;
+  if constexpr (S == 1)
+#pragma unroll
+    for (int q = 0; q < kAcc; ++q) outer[q] = 0.f;
+  for (int64_t tile = beg; tile < end; ++tile) {
+    const int X = (int)(tile / tiles);
+    const float* nd = nodes + (tile * NF) * 32 + lane;
+    auto fld = [&](int q) { return __ldg(nd + 32 * q); };
+    const float rx = fld(fR), ry = fld(fR + 2), rz = fld(fR + 4);
+    // t_m = (r/c) . n, tau and Phi at the block's middle sample, in double-float
+    const df tm = df_add(df_add(df_mul({rx, fld(fR + 1)}, K.nx), df_mul({ry, fld(fR + 3)}, K.ny)),
+                         df_mul({rz, fld(fR + 5)}, K.nz));
+    const df tau = df_add({fld(fTau), fld(fTau + 1)}, tm);
+    const df tau2 = df_mul(tau, tau);
+    const df ph = df_add(df_add(df_mul(K.fmh, tau), df_mul(K.fh, tm)),
+                         df_add(df_mul(K.f1h, tau2), df_mul(K.f2s, df_mul(tau2, tau))));
+    const float t = tau.h;
+    const float rate = K.f + K.f1 * t + 0.5f * K.f2 * t * t;  // dPhi/dt_m
+    bool wide = false;
+    float p1h = 0.f, p1l = 0.f, p2h = 0.f, p2 = 0.f, p3 = 0.f, dtau = 0.f, r1x = 0.f, r1y = 0.f, r1z = 0.f, r2x = 0.f, r2y = 0.f,
+          r2z = 0.f;
+    if constexpr (S > 1) {
+      r1x = fld(fR1); r1y = fld(fR1 + 1); r1z = fld(fR1 + 2);
+      r2x = fld(fR2); r2y = fld(fR2 + 1); r2z = fld(fR2 + 2);
+      const float d1 = r1x * K.nx.h + r1y * K.ny.h + r1z * K.nz.h;
+      const float d2 = r2x * K.nx.h + r2y * K.ny.h + r2z * K.nz.h;
+      const float d3 = fld(fR3) * K.nx.h + fld(fR3 + 1) * K.ny.h + fld(fR3 + 2) * K.nz.h;
+      dtau = K.dt.h + d1;
+      const float spin = K.f1 + K.f2 * t, rate1 = (K.f1 * t + 0.5f * K.f2 * t * t) * dtau;
+      // dPhi per sample = (f - f_h) dt + f dt_m + (f1dot tau + f2dot tau^2/2) dtau,
+      // mod 1 (u is an integer), split so that u p1h is exact
+      df s = two_sum(K.step.h, K.f * d1);
+      s.l += K.step.l;
+      p2 = 0.5f * (rate * d2 + spin * dtau * dtau);
+      p3 = (1.f / 6.f) * (rate * d3 + 3.f * spin * dtau * d2 + K.f2 * dtau * dtau * dtau);
+      // a continuous-wave source's spindown moves the frequency by far less
+      // than a bin of 1/dt over the data; a short series admits larger ones
+      constexpr float h = 0.5f * S;
+      wide = __any_sync(0xffffffffu, fabsf(rate1) + h * h * (fabsf(p2) + h * fabsf(p3)) > 0.0625f);
+      if (wide) {  // the spindown's part of the slope and curvature in double-float, both mod 1
+        df dt1 = two_sum(K.dt.h, d1);
+        dt1.l += K.dt.l;
+        const df a = df_mulf(df_mul(K.f1h, tau), 2.f), b = df_mulf(df_mul(K.f2s, tau2), 3.f);
+        const df q = df_mul(df_add(a, b), dt1);
+        s = df_add(s, {__fsub_rn(q.h, rintf(q.h)), q.l});
+        const df c = df_mul(df_mul(df_add(K.f1h, df_mulf(df_mul(K.f2s, tau), 3.f)), dt1), dt1);
+        const float hi = __fsub_rn(c.h, rintf(c.h));
+        p2h = rintf(hi * 16384.f) * (1.f / 16384.f);
+        p2 = __fadd_rn(__fsub_rn(hi, p2h), __fadd_rn(c.l, 0.5f * rate * d2));
+      } else {
+        const float e = s.l;
+        s = two_sum(s.h, rate1);
+        s.l += e;
+      }
+      const float hi = __fsub_rn(s.h, rintf(s.h));
+      p1h = rintf(hi * 131072.f) * (1.f / 131072.f);
+      p1l = __fadd_rn(__fsub_rn(hi, p1h), s.l);
+    }
+    // the block's moments
+    cpx E0{0.f, 0.f}, E1{0.f, 0.f}, E2{0.f, 0.f};
+    if constexpr (S > 1) {
+      const float4* x = reinterpret_cast<const float4*>(xt + tile * (32 * S)) + lane;
+      auto moments = [&](auto far) {
+#pragma unroll
+        for (int i = 0; i < S; i += 2) {
+          const float4 v = __ldg(x + 16 * i);
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float u = (float)(i + e - S / 2);
+            const float xr = e ? v.z : v.x, xi = e ? v.w : v.y;
+            float f = fmaf(u, fmaf(u, fmaf(u, p3, p2), p1l), less_rint(__fmul_rn(u, p1h)));
+            if constexpr (decltype(far)::value) f = less_rint(f + less_rint(__fmul_rn(u * u, p2h)));
+            float sn, cs;
+            __sincosf(two_pi * f, &sn, &cs);
+            const float er = xr * cs + xi * sn, ei = xi * cs - xr * sn;
+            E0.r += er;
+            E0.i += ei;
+            E1.r = fmaf(u, er, E1.r);
+            E1.i = fmaf(u, ei, E1.i);
+            E2.r = fmaf(u * u, er, E2.r);
+            E2.i = fmaf(u * u, ei, E2.i);
+          }
+        }
+      };
+      if (wide) moments(std::true_type());
+      else moments(std::false_type());
+    } else {
+      const float2 v = __ldg(xt + tile * 32 + lane);
+      E0 = {v.x, v.y};
+    }
+    {
+      // (its error is common to the block: the accurate function)
+      float sn, cs;
+      sincospif(2.f * df_frac(ph), &sn, &cs);
+      auto rot = [&](cpx& e) { e = {e.r * cs + e.i * sn, e.i * cs - e.r * sn}; };
+      rot(E0);
+      if constexpr (S > 1) {
+        rot(E1);
+        rot(E2);
+      }
+    }
+    const float c1 = fld(fCos), s1 = fld(fCos + 1), c2 = fld(fCos + 2), s2 = fld(fCos + 3);
+    // dPhi/dalpha, dPhi/ddelta (over 2 pi) and their expansions
+    const float ra = rx * K.dna[0] + ry * K.dna[1], rd = rx * K.dnd[0] + ry * K.dnd[1] + rz * K.dnd[2];
+    float ga[3] = {rate * ra, 0.f, 0.f}, gd[3] = {rate * rd, 0.f, 0.f};
+    if constexpr (S > 1) {
+      const float drate = (K.f1 + K.f2 * t) * dtau;
+      const float ra1 = r1x * K.dna[0] + r1y * K.dna[1], rd1 = r1x * K.dnd[0] + r1y * K.dnd[1] + r1z * K.dnd[2];
+      ga[1] = rate * ra1 + drate * ra;
+      gd[1] = rate * rd1 + drate * rd;
+      ga[2] = 0.5f * rate * (r2x * K.dna[0] + r2y * K.dna[1]);
+      gd[2] = 0.5f * rate * (r2x * K.dnd[0] + r2y * K.dnd[1] + r2z * K.dnd[2]);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {  // a, b
+      const Local p = local<(S > 1)>(K.pat[X][q], c1, s1, c2, s2, w_step);
+      // sum e p u^m over the block
+      cpx m0{p.v * E0.r, p.v * E0.i}, m1{0.f, 0.f}, m2{0.f, 0.f};
+      if constexpr (S > 1) {
+        const float h2 = 0.5f * p.d2;
+        m0.r = fmaf(p.d1, E1.r, fmaf(h2, E2.r, m0.r));
+        m0.i = fmaf(p.d1, E1.i, fmaf(h2, E2.i, m0.i));
+        m1 = {fmaf(p.d1, E2.r, p.v * E1.r), fmaf(p.d1, E2.i, p.v * E1.i)};
+        m2 = {p.v * E2.r, p.v * E2.i};
+      }
+      // sum e p g for a function g = g0 + g1 u + g2 u^2
+      auto times = [&](float g0, float g1, float g2) -> cpx {
+        if constexpr (S > 1) return {fmaf(g2, m2.r, fmaf(g1, m1.r, g0 * m0.r)), fmaf(g2, m2.i, fmaf(g1, m1.i, g0 * m0.i))};
+        else return {g0 * m0.r, g0 * m0.i};
+      };
+      acc[2 * q] += m0.r;
+      acc[2 * q + 1] += m0.i;
+      // d/dtheta of e p = e (p_theta - i 2 pi Phi_theta p)
+      const cpx vf = times(two_pi * t, two_pi * dtau, 0.f);
+      const cpx v1 = times(two_pi * 0.5f * t * t, two_pi * t * dtau, two_pi * 0.5f * dtau * dtau);
+      acc[4 + 2 * q] += vf.i;
+      acc[5 + 2 * q] -= vf.r;
+      acc[8 + 2 * q] += v1.i;
+      acc[9 + 2 * q] -= v1.r;
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {  // alpha, delta
+        const float* gg = d ? gd : ga;
+        const cpx vg = times(two_pi * gg[0], two_pi * gg[1], two_pi * gg[2]);
+        const Local y = local<(S > 1)>(K.pat[X][2 + 2 * d + q], c1, s1, c2, s2, w_step);
+        cpx z{y.v * E0.r, y.v * E0.i};
+        if constexpr (S > 1) {
+          const float h2 = 0.5f * y.d2;
+          z.r = fmaf(y.d1, E1.r, fmaf(h2, E2.r, z.r));
+          z.i = fmaf(y.d1, E1.i, fmaf(h2, E2.i, z.i));
+        }
+        acc[12 + 4 * d + 2 * q] += z.r + vg.i;
+        acc[13 + 4 * d + 2 * q] += z.i - vg.r;
+      }
+    }
+    if constexpr (S == 1) {
+      if (((tile - beg) & (kInner - 1)) == kInner - 1) {
+#pragma unroll
+        for (int q = 0; q < kAcc; ++q) { outer[q] += acc[q]; acc[q] = 0.f; }
+      }
+    }
+  }
+  // the lanes' sums through shared memory: lane q adds quantity q's 32 values
+  // in double-float, which costs a tenth of FP64 adds on this GPU
 #pragma unroll
   for (int q = 0; q < kAcc; ++q) {
-    double v = (double)outer[32 * q] + (double)inner[q];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) dst[q] = v;
+    if constexpr (S == 1) acc[q] += outer[q];
+    s_red[warp][q][lane] = acc[q];
+  }
+  __syncwarp();
+  if (lane < kAcc) {
+    df s{0.f, 0.f};
+    for (int l = 0; l < 32; ++l) {
+      const df a = two_sum(s.h, s_red[warp][lane][l]);
+      s = {a.h, __fadd_rn(s.l, a.l)};
+    }
+    partial[item * kAcc + lane] = (double)s.h + (double)s.l;
   }
 }
 
-// sum the chunk partials (fixed order) and apply the chain rule in FP64
-__global__ void k_finalize(const double* __restrict__ partial, int n_cand, int n_chunks,
-                           float* __restrict__ twoF, float* __restrict__ grad) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+// sum the chunk partials (fixed order) and apply the chain rule in FP64, one
+// warp per candidate; partial[chunk][cand][kAcc]
+__global__ void k_finalize(const double* __restrict__ partial, const CandConst* __restrict__ cc, int n_cand,
+                           int n_chunks, float* __restrict__ twoF, float* __restrict__ grad) {
+  __shared__ double s_sum[kWarps][kAcc];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * kWarps + warp;
   if (i >= n_cand) return;
-  double s[kAcc];
-  for (int q = 0; q < kAcc; ++q) s[q] = 0.0;
-  for (int c = 0; c < n_chunks; ++c)
-    for (int q = 0; q < kAcc; ++q) s[q] += partial[((int64_t)i * n_chunks + c) * kAcc + q];
-  const double A = s[20], B = s[21], C = s[22];
+  if (lane < kAcc) {
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    int c = 0;
+    for (; c + 4 <= n_chunks; c += 4)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) t[q] += partial[((int64_t)(c + q) * n_cand + i) * kAcc + lane];
+    for (; c < n_chunks; ++c) t[0] += partial[((int64_t)c * n_cand + i) * kAcc + lane];
+    s_sum[warp][lane] = (t[0] + t[1]) + (t[2] + t[3]);
+  }
+  __syncwarp();
+  if (lane >= 4) return;
+  const double* s = s_sum[warp];
+  const double* m = cc[i].abc;
+  const double A = m[0], B = m[1], C = m[2];
   const double D = A * B - C * C;
   const double far = s[0], fai = s[1], fbr = s[2], fbi = s[3];
   const double fa2 = far * far + fai * fai, fb2 = fbr * fbr + fbi * fbi, re = far * fbr + fai * fbi;
   const double N = B * fa2 + A * fb2 - 2.0 * C * re;
-  twoF[i] = (float)(2.0 * N / D);
-  for (int j = 0; j < 4; ++j) {
-    const double dar = s[4 + 4 * j], dai = s[5 + 4 * j], dbr = s[6 + 4 * j], dbi = s[7 + 4 * j];
-    const double dfa2 = 2.0 * (far * dar + fai * dai);
-    const double dfb2 = 2.0 * (fbr * dbr + fbi * dbi);
-    const double dre = dar * fbr + dai * fbi + far * dbr + fai * dbi;
-    double dA = 0.0, dB = 0.0, dC = 0.0;
-    if (j == 2) { dA = s[23]; dB = s[24]; dC = s[25]; }
-    if (j == 3) { dA = s[26]; dB = s[27]; dC = s[28]; }
-    const double dN = dB * fa2 + B * dfa2 + dA * fb2 + A * dfb2 - 2.0 * (dC * re + C * dre);
-    const double dD = dA * B + A * dB - 2.0 * C * dC;
-    grad[4 * i + j] = (float)(2.0 * (dN * D - N * dD) / (D * D));
+  const int j = lane;  // d/d(f, f1dot, alpha, delta)
+  if (j == 0) twoF[i] = (float)(2.0 * N / D);
+  const double dar = s[4 + 4 * j], dai = s[5 + 4 * j], dbr = s[6 + 4 * j], dbi = s[7 + 4 * j];
+  const double dfa2 = 2.0 * (far * dar + fai * dai);
+  const double dfb2 = 2.0 * (fbr * dbr + fbi * dbi);
+  const double dre = dar * fbr + dai * fbi + far * dbr + fai * dbi;
+  double dA = 0.0, dB = 0.0, dC = 0.0;
+  if (j >= 2) {
+    dA = m[3 * (j - 1)];
+    dB = m[3 * (j - 1) + 1];
+    dC = m[3 * (j - 1) + 2];
   }
+  const double dN = dB * fa2 + B * dfa2 + dA * fb2 + A * dfb2 - 2.0 * (dC * re + C * dre);
+  const double dD = dA * B + A * dB - 2.0 * C * dC;
+  grad[4 * i + j] = (float)(2.0 * (dN * D - N * dD) / (D * D));
 }
+
+// sum_{k < n} exp(i m phi_k), phi_k = phi_0 + k step: the geometric sum
+// exp(i m (phi_0 + (n-1) step / 2)) sin(n x) / sin(x), x = m step / 2
+Harmonics harmonics(const Geo& g) {
+  Harmonics h{};
+  for (int X = 0; X < g.n_det; ++X)
+    for (int m = 0; m <= 4; ++m) {
+      const double step = g.w_rot * g.dt, x = 0.5 * m * step, n = (double)g.n, sx = sin(x);
+      // at a multiple of pi the quotient's limit, n cos(n x) / cos(x)
+      const double amp = fabs(sx) < 1e-14 ? n * cos(n * x) / cos(x) : sin(n * x) / sx;
+      const double mid = m * (g.lon[X] + g.sid_ph0 + g.w_rot * g.t0 + 0.5 * (n - 1.0) * step);
+      h.c[X][m] = amp * cos(mid);
+      h.s[X][m] = amp * sin(mid);
+    }
+  return h;
+}
+
+int chunk_count(const Geo& g, const Layout& l) {
+  const int64_t per = kChunkSamples / (32 * l.S);
+  return (int)((g.n_det * l.tiles + per - 1) / per);
+}
+
+// Candidates per launch: at most 4096, and the partial sums (160 B per
+// candidate and chunk) stay within 64 MB; the fewest that this gives, 100 for
+// the longest data of four detectors, still fill the GPU.
+int batch_size(int n_cand, const Geo& g, const Layout& l) {
+  const int64_t per = (int64_t)chunk_count(g, l) * kAcc * sizeof(double);
+  return (int)std::min<int64_t>(std::min(n_cand, 4096), std::max<int64_t>(64, ((int64_t)64 << 20) / per));
+}
+
+size_t consts_bytes(int n_cand) { return ((size_t)n_cand * sizeof(CandConst) + 255) & ~(size_t)255; }
 
 }  // namespace adj
 
-size_t grad_table_bytes(int n_det, int64_t n) {
-  return (size_t)n_det * n * (16 + 8 + 16 + 8 + 8) + 256;
+size_t grad_table_bytes(const Geo& g) {
+  const adj::Layout l = adj::layout(g);
+  return l.x_bytes + l.node_bytes + 256;
 }
 
-cudaError_t launch_grad_tables(const Geo& g, const void* const* xh, const int* dtype, void* base,
-                               cudaStream_t st) {
-  const int64_t tot = (int64_t)g.n_det * g.n;
-  adj::SampleTabs tab;
-  char* p = (char*)base;
-  tab.rc = (float4*)p; p += 16 * tot;
-  tab.d0 = (float4*)p; p += 16 * tot;
-  tab.rcz = (float2*)p; p += 8 * tot;
-  tab.d1 = (float2*)p; p += 8 * tot;
-  tab.x = (float2*)p;
-  int blocks = (int)((g.n + 255) / 256);
-  if (blocks > device_sm_count() * 32) blocks = device_sm_count() * 32;
-  for (int X = 0; X < g.n_det; ++X)
-    adj::k_tables<<<blocks, 256, 0, st>>>(g, X, xh[X], dtype[X], tab);
+cudaError_t launch_grad_tables(const Geo& g, const void* const* xh, const int* dtype, void* base, cudaStream_t st) {
+  const adj::Layout l = adj::layout(g);
+  adj::Series src{};
+  for (int X = 0; X < g.n_det; ++X) { src.x[X] = xh[X]; src.dtype[X] = dtype[X]; }
+  const int64_t blocks = l.tiles * 32, cap = (int64_t)device_sm_count() * 16;
+  adj::k_series_table<<<dim3((unsigned)std::min(cap, (blocks * l.S + 255) / 256), g.n_det), 256, 0, st>>>(
+      g, src, l.S, l.tiles, (float2*)base);
+  adj::k_block_table<<<dim3((unsigned)std::min(cap, (blocks + 127) / 128), g.n_det), 128, 0, st>>>(
+      g, l.S, l.tiles, (float*)((char*)base + l.x_bytes));
   return cudaGetLastError();
 }
 
 size_t grad_scratch_bytes(int n_cand, const Geo& g) {
-  const int64_t tot = (int64_t)g.n_det * g.n;
-  const int chunks = (int)((tot + adj::kChunk - 1) / adj::kChunk);
-  return (size_t)n_cand * sizeof(adj::CandConst) + (size_t)n_cand * chunks * adj::kAcc * sizeof(double) + 512;
+  const adj::Layout l = adj::layout(g);
+  const int b = adj::batch_size(n_cand, g, l);
+  return adj::consts_bytes(b) + (size_t)b * adj::chunk_count(g, l) * adj::kAcc * sizeof(double) + 256;
+}
+
+int grad_launches(int n_cand, const Geo& g) {
+  const int b = adj::batch_size(n_cand, g, adj::layout(g));
+  return 3 * ((n_cand + b - 1) / b);
 }
 
 cudaError_t launch_grad(const Geo& g, const void* tables, const fstat_candidate* cand_dev, int n_cand,
                         void* scratch, float* twoF, float* grad, cudaStream_t st) {
-  const int64_t tot = (int64_t)g.n_det * g.n;
-  const int chunks = (int)((tot + adj::kChunk - 1) / adj::kChunk);
-  adj::SampleTabs tab;
-  char* p = (char*)tables;
-  tab.rc = (float4*)p; p += 16 * tot;
-  tab.d0 = (float4*)p; p += 16 * tot;
-  tab.rcz = (float2*)p; p += 8 * tot;
-  tab.d1 = (float2*)p; p += 8 * tot;
-  tab.x = (float2*)p;
-  adj::CandConst* cc = (adj::CandConst*)scratch;
-  double* partial = (double*)((char*)scratch + (((size_t)n_cand * sizeof(adj::CandConst) + 255) & ~(size_t)255));
-  adj::k_cand_consts<<<(n_cand + 127) / 128, 128, 0, st>>>(cand_dev, n_cand, g.f_het, cc);
-  dim3 grid((n_cand + adj::kWarps - 1) / adj::kWarps, chunks);
-  adj::k_partial<<<grid, adj::kWarps * 32, 0, st>>>(g, tab, cc, n_cand, chunks, partial);
-  adj::k_finalize<<<(n_cand + 127) / 128, 128, 0, st>>>(partial, n_cand, chunks, twoF, grad);
+  using namespace adj;
+  const Layout l = layout(g);
+  const int chunks = chunk_count(g, l), batch = batch_size(n_cand, g, l);
+  const Harmonics h = harmonics(g);
+  const float2* x = (const float2*)tables;
+  const float* nodes = (const float*)((const char*)tables + l.x_bytes);
+  CandConst* cc = (CandConst*)scratch;
+  double* partial = (double*)((char*)scratch + consts_bytes(batch));
+  const float w_step = (float)(g.w_rot * g.dt);
+  for (int c0 = 0; c0 < n_cand; c0 += batch) {
+    const int n = std::min(batch, n_cand - c0);
+    k_cand_consts<<<(n + 31) / 32, 32, 0, st>>>(g, h, cand_dev + c0, n, cc);
+    const unsigned grid = (unsigned)(((int64_t)n * chunks + kWarps - 1) / kWarps);
+    auto run = [&](auto kernel) {
+      kernel<<<grid, kWarps * 32, 0, st>>>(g.n_det, l.tiles, x, nodes, w_step, cc, n, chunks, partial);
+    };
+    switch (l.S) {
+      case 32: run(k_moments<32>); break;
+      case 16: run(k_moments<16>); break;
+      case 8: run(k_moments<8>); break;
+      default: run(k_moments<1>); break;
+    }
+    k_finalize<<<(n + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(partial, cc, n, chunks, twoF + c0, grad + 4 * (int64_t)c0);
+  }
   return cudaGetLastError();
 }
 

@@ -198,10 +198,11 @@ void launch_tmpl_coef(const SkyConst* sky, double dt, int64_t n, const fstat_tem
                       const int* order, int first, int count, TmplCoef* out, cudaStream_t st);
 void launch_check_finite(const void* x, int dtype, int64_t n, int* err, cudaStream_t st);
 // Gradient (adjoint.cu): per-plan sample tables and per-call scratch.
-size_t grad_table_bytes(int n_det, int64_t n);
+size_t grad_table_bytes(const Geo& g);
 cudaError_t launch_grad_tables(const Geo& g, const void* const* xh, const int* dtype, void* base,
                                cudaStream_t st);
 size_t grad_scratch_bytes(int n_cand, const Geo& g);
+int grad_launches(int n_cand, const Geo& g);  // kernels of one launch_grad
 cudaError_t launch_grad(const Geo& g, const void* tables, const fstat_candidate* cand_dev, int n_cand,
                         void* scratch, float* twoF, float* grad, cudaStream_t st);
 

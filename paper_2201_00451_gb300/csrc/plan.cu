@@ -935,7 +935,7 @@ static bool candidates_finite(const fstat_candidate* cand, int64_t n) {
 // the gradient's sample tables (built once per data set) and scratch for n
 // candidates
 static int grad_prepare(fstat_plan* p, int64_t n, cudaStream_t st) {
-  if (!p->gtab) CK(palloc(p, &p->gtab, grad_table_bytes(p->d.n_det, p->d.n_samples)));
+  if (!p->gtab) CK(palloc(p, &p->gtab, grad_table_bytes(p->geo)));
   if (!p->gtab_valid) {
     const void* xh[kMaxDet];
     for (int X = 0; X < kMaxDet; ++X) xh[X] = p->xh[X];
@@ -1035,8 +1035,8 @@ int fstat_refine(fstat_plan* p, const fstat_candidate* cand, int64_t n, const do
     CK(launch_grad(p->geo, p->gtab, s.trial, (int)n, p->gscratch, s.val, s.gt, st));
     CK(launch_ascent_accept(s, h + (size_t)(k + 1) * n, st));
   }
-  // three kernels per evaluation, trial and accept per step, init
-  p->n_launches += 4 + 5 * (int64_t)steps;
+  // the evaluations, trial and accept per step, init
+  p->n_launches += 1 + 2 * (int64_t)steps + (1 + (int64_t)steps) * grad_launches((int)n, p->geo);
   CK(cudaMemcpyAsync(out, s.theta, (size_t)n * sizeof(fstat_candidate), cudaMemcpyDeviceToHost, st));
   if (hist) CK(cudaMemcpyAsync(hist, h, (size_t)(steps + 1) * n * sizeof(float), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));

@@ -187,3 +187,45 @@ def test_full_size_refinement_recovers_injections():
     med = np.array([np.median(hist[-1][owner == k]) for k in range(len(truth))])
     assert np.all(got >= 0.97 * ref), (got, ref)
     assert np.all(med >= 0.85 * ref), (med, ref)
+
+
+@pytest.mark.parametrize("dt,n", [(0.5, 40001), (1.0, 1023), (3.0, 9001), (6.0, 513), (6.0, 7000), (10.0, 6400)])
+def test_every_block_length_matches_oracle(dt, n):
+    # blocks of 32, 16, 8 samples and single samples (dt 0.5 and 1, 3, 6, 10 s),
+    # whole and ragged last tiles, complex128 data; tolerances as above
+    t = small_target(n_samples=n, dt=dt, n_fft=1 << 16, n_det=2, n_inj=1, rho2_range=(150.0, 150.0), seed=47,
+                     f1dots=(-1e-9,), f2dots=(0.0,), dtype="c128", f_het=400.0)
+    x = synth.make_data(t)
+    inj = t.injections[0]
+    s = _scales(t)
+    rng = np.random.default_rng(8)
+    base = np.array([inj.f0, inj.f1dot, inj.alpha, inj.delta])
+    rows = [base + rng.uniform(-0.5, 0.5, 4) * s for _ in range(3)]
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            plan.set_data(X, x[X], t.sigmas[X])
+        two_f, g = (v.cpu().numpy() for v in plan.grad(_cands(rows, f2dot=1e-16)))
+    for i, th in enumerate(rows):
+        v, gr = og.grad(t, x, th, f2dot=1e-16)
+        assert abs(two_f[i] - v) <= 1e-4 * abs(v) + 1e-3
+        assert np.all(np.abs((g[i] - gr) * s) <= 2e-3 * abs(v) + 2e-3), (g[i] * s, gr * s)
+
+
+def test_large_spindown_of_a_short_series_matches_oracle():
+    # |f1dot| tau^2 of 2.5e5 cycles over 1.4 hours: tens of cycles of curvature
+    # within one block; tolerances as above
+    t = small_target(n_samples=2501, dt=2.0, n_fft=1 << 13, n_det=2, n_inj=1, rho2_range=(150.0, 150.0), seed=48,
+                     f1dots=(-0.04,), f2dots=(0.0,), dtype="c128")
+    x = synth.make_data(t)
+    inj = t.injections[0]
+    s = _scales(t)
+    base = np.array([inj.f0, inj.f1dot, inj.alpha, inj.delta])
+    rows = [base, base + 0.4 * s]
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            plan.set_data(X, x[X], t.sigmas[X])
+        two_f, g = (v.cpu().numpy() for v in plan.grad(_cands(rows)))
+    for i, th in enumerate(rows):
+        v, gr = og.grad(t, x, th)
+        assert abs(two_f[i] - v) <= 1e-4 * abs(v) + 1e-3
+        assert np.all(np.abs((g[i] - gr) * s)[:2] <= 2e-3 * abs(v) + 2e-3), (g[i] * s, gr * s)

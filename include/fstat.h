@@ -307,30 +307,22 @@ int fstat_kernel_stats(fstat_plan* plan, int kernel, int64_t* launches, double* 
 int fstat_get_split(const fstat_plan* plan, int64_t* n1, int64_t* n2);
 int fstat_set_split(fstat_plan* plan, int64_t n1);
 
-/* Launch shapes of the two FFT passes: columns per CTA of pass A (ca),
- * rows per CTA of pass B (cb), 0 = default for the length; schedule va /
- * vb: bit 0 = radix-8 first (lengths >= 1024, else radix-16 first), bit 1 =
- * one shared-memory buffer instead of two (half the shared memory; the
- * next tile's copies start once the last FFT pass has read the buffer;
- * radix-16 CTAs of up to 256 threads are register-capped so that two share
- * an SM); va only: bit 3 (with bit 1, radix-16) = three CTAs per SM; vb
- * only: bit 2 = pass B tile loads by the tensor-memory-access engine
- * (FP32, rows of 1024 points or more; a load that does not complete within
- * a bounded wait ends the kernel, and fstat_sync() then returns
- * FSTAT_ERR_TIMEOUT); va 16 (FP32, 8192-point columns, one per CTA) and
- * va 18 (FP32, 4096-point columns, one per CTA, two CTAs per SM) = the
- * next column's samples copied by one bulk copy into shared memory of
- * their own while the current column is transformed (the plan's samples
- * per column must fit beside the column buffer; a copy that does not
- * complete within a bounded wait likewise gives FSTAT_ERR_TIMEOUT).  va
- * 0..3, 10, 16 or 18.  vb 8 (FP32 rows of 1024 points or more, not
- * with fstat_compute_peaks) = the first half of the next tile's rows copied
- * into shared memory of their own as soon as the current tile's first pass
- * has read its own, the second half once its last pass has read the
- * buffer (fstat_compute_peaks runs schedule 0 in its place).  vb 0..8.  A shape that is not
- * compiled for the current split makes fstat_compute return
- * FSTAT_ERR_CUDA.  fstat_get_cta reports the shapes in effect (a default
- * as its value for the current split). */
+/* Launch shapes of the two FFT passes: columns per CTA of pass A (ca), rows
+ * per tile of pass B (cb), 0 = default for the length, and schedule codes va
+ * (0..3, 10, 16 or 18) and vb (0..8).  FP32 plans run one schedule, whose 2F is
+ * the same bit for bit for every code and row count: cb chooses the rows per
+ * tile (a count with no compiled shape runs the default), va 2 loads pass A's
+ * columns straight into registers, va 16 (8192-point columns) and va 18
+ * (4096-point columns) require the next column's samples staged in shared
+ * memory while the current one is transformed (they must fit beside it), the
+ * other codes stage them where that costs no occupancy.  A staged copy or a
+ * tile load that does not complete within a bounded wait ends the kernel, and
+ * fstat_sync() then returns FSTAT_ERR_TIMEOUT.  FP64 plans run code 0 with the
+ * default shape.  A combination that no pass of the current split offers
+ * (odd codes and vb above 3 below 1024 points, va 16 / 18 at other lengths, ca
+ * or cb whose transforms exceed 1024 threads or shared memory) makes
+ * fstat_compute return FSTAT_ERR_CUDA.  fstat_get_cta reports the shapes in
+ * effect (a default as its value for the current split). */
 int fstat_get_cta(const fstat_plan* plan, int* ca, int* va, int* cb, int* vb);
 int fstat_set_cta(fstat_plan* plan, int ca, int va, int cb, int vb);
 
@@ -366,9 +358,8 @@ int fstat_set_streams(fstat_plan* plan, int n);
 int fstat_set_fused(fstat_plan* plan, int enable);
 int fstat_get_fused(const fstat_plan* plan, int* enabled);
 
-/* Polls of the first wait for each of pass B's bulk tensor copies (the
- * TMA schedules, vb bit 2) and of the wait for each staged column of pass
- * A's schedule 16: a kernel that waits longer records
+/* Polls of the first wait for each of pass B's tile loads and of the wait for
+ * each staged column of pass A (FP32 plans): a kernel that waits longer records
  * FSTAT_ERR_TIMEOUT (returned by fstat_sync), lets its copies in flight land
  * under the full default limit, and returns.  polls < 0 restores the default
  * (2^22 polls); 0 makes every first wait give up at once, which tests of the
@@ -378,12 +369,11 @@ int fstat_get_fused(const fstat_plan* plan, int* enabled);
  * Errors: INVALID_ARG (NULL plan). */
 int fstat_set_wait_limit(fstat_plan* plan, int polls);
 
-/* Autotuner: times every compiled (split, ca, va, cb, vb) for this plan's n_fft on
+/* Autotuner: times every distinct (split, va, cb) for this plan's n_fft on
  * the current data with CUDA events on `stream` and keeps the fastest.
- * Then, at that split, it times pass B of fstat_compute_peaks on its own
- * (256 whole-row bands, threshold 70) over every compiled (cb, vb) and keeps
- * the fastest for that mode (without the 2F store its best shape can
- * differ).  fstat_set_cta makes both modes use the shape it sets.
+ * Then, at that split, it times fstat_compute_peaks (256 whole-row bands,
+ * threshold 70) over every compiled cb and keeps the fastest for that mode
+ * (without the 2F store its best shape can differ).  fstat_set_cta makes both modes use the shape it sets.
  * Results are cached per (GPU name, n_samples, n_fft, precision, n_det) in
  * the process and, if the environment variable FSTAT_AUTOTUNE_CACHE names
  * a file, in that file.  Synchronises; invalidates cached per-sky work.

@@ -489,12 +489,11 @@ class FstatPlan:
         _check(self._lib.fstat_set_residency(self._p, int(ra), int(rb)), "fstat_set_residency")
 
     def set_cta(self, ca: int, cb: int, va: int = 0, vb: int = 0):
-        """fstat_set_cta: columns per CTA of pass A (ca), rows per CTA of pass
-        B (cb), 0 = the length's default; schedules va (0..3, 10, 16 or 18)
-        and vb (0..8): bit 0 radix-8 first, bit 1 one buffer
-        (register-capped for two CTAs per SM), bit 2 pass-B tiles by TMA,
-        bit 3 pass A three CTAs per SM, va 16 / 18 columns staged apart, vb
-        8 half of the next pass-B tile staged apart."""
+        """fstat_set_cta: columns per CTA of pass A (ca), rows per tile of pass
+        B (cb), 0 = the length's default; schedule codes va (0..3, 10, 16 or
+        18) and vb (0..8): in FP32 plans va 2 loads columns straight into
+        registers, 16 / 18 require them staged; the other codes run the same
+        schedule."""
         _check(self._lib.fstat_set_cta(self._p, int(ca), int(va), int(cb), int(vb)), "fstat_set_cta")
 
     def set_streams(self, n: int):
@@ -521,8 +520,8 @@ class FstatPlan:
         _check(self._lib.fstat_set_fused(self._p, int(bool(enable))), "fstat_set_fused")
 
     def set_wait_limit(self, polls: int):
-        """fstat_set_wait_limit: polls of pass B's first bulk-copy wait per
-        tile (< 0 restores the default)."""
+        """fstat_set_wait_limit: polls of the first wait for each tile load and
+        staged column (< 0 restores the default)."""
         _check(self._lib.fstat_set_wait_limit(self._p, int(polls)), "fstat_set_wait_limit")
 
     def autotune(self, stream=None):

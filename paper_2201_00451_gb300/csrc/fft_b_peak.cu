@@ -1,15 +1,9 @@
-// Pass B in peaks mode (fstat_compute_peaks): the same transform as the
+// FP64 pass B in peaks mode (fstat_compute_peaks): the same transform as the
 // dense pass, with 2F reduced in the kernel to a threshold-crossing list and
-// per-band maxima.  Both precisions live here so the dense translation
-// units keep their build time.
+// per-band maxima; and the decoding of the band keys.
 #include "fft_impl.cuh"
 
 namespace fstat {
-
-cudaError_t launch_pass_b_peak_f32(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                                   const SkyConst* sky, const PeakArgs& pk, cudaStream_t st, int res) {
-  return fft::dispatch_b<float, fft::kPeaks>(log2_n1, cb, vb, Z, n2, twB, sky, nullptr, pk, st, res);
-}
 
 cudaError_t launch_pass_b_peak_f64(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
                                    const SkyConst* sky, const PeakArgs& pk, cudaStream_t st, int res) {

@@ -116,10 +116,10 @@ __device__ __noinline__ void item_issue(const FusedArgs& a, const ZMaps& zm, con
   fence_proxy_async_global();  // what item_ready acquired precedes the copies
   fence_proxy_async();         // this CTA's earlier use of the buffer precedes them
   if (it.kind == 0) {
-    const unsigned bytes = (unsigned)(a.lc * sizeof(float4));
+    const unsigned bytes = (unsigned)(a.gc.lc * sizeof(float4));
     mbar_expect_tx(bar, bytes * CA);
 #pragma unroll 1
-    for (int c = 0; c < CA; ++c) bulk_load(smem + c * LPA, a.G + (int64_t)(it.tile * CA + c) * a.lc, bytes, bar);
+    for (int c = 0; c < CA; ++c) bulk_load(smem + c * LPA, a.G + (int64_t)(it.tile * CA + c) * a.gc.lc, bytes, bar);
   } else {
     mbar_expect_tx(bar, (unsigned)(LB * CB * sizeof(float4)));
     const CUtensorMap* map = &zm.m[it.k % kRing];
@@ -197,16 +197,14 @@ k_fused(const __grid_constant__ FusedArgs a, const __grid_constant__ ZMaps zm) {
       const Item it = decode_item(s_cur, a.na, a.nb, a.T);
       if (it.kind == 0) {
         const int cA = threadIdx.x / SA::TPC, tA = threadIdx.x % SA::TPC;
-        const float inv_n = 1.f / (float)((int64_t)a.n1 * a.n2);
-        pass_a_tile<float, LA, CA, VA, true>(it.tile, smem + cA * SA::LP, cA, tA, a.G, a.lc, a.n, a.n1,
-                                             (const float2*)nullptr, a.coef[it.k], inv_n, a.Z[it.k % kRing],
-                                             at_free);
+        pass_a_tile<float, LA, CA, VA>(it.tile, smem + cA * SA::LP, cA, tA, a.G, a.gc, a.n, a.n1,
+                                             (const float2*)nullptr, a.coef[it.k], a.Z[it.k % kRing], at_free);
       } else {
         const int cB = threadIdx.x % CB, tB = threadIdx.x / CB;
         const SkyConst& sk = *a.sky;
         float* row = a.out + (int64_t)(a.ord[it.k] % a.out_rows) * ((int64_t)a.n1 * a.n2);
         const PeakArgs pk{};
-        pass_b_tile<float, LB, CB, VB, true, kStore>(it.tile, smem + cB, cB, tB, a.Z[it.k % kRing], a.n2,
+        pass_b_tile<float, LB, CB, VB, kStore>(it.tile, smem + cB, cB, tB, a.n2,
                                                      (const float2*)nullptr, sk.kAf, sk.kBf, sk.kCf, row, pk,
                                                      nullptr, nullptr, at_free);
       }
@@ -230,12 +228,10 @@ k_fused(const __grid_constant__ FusedArgs a, const __grid_constant__ ZMaps zm) {
 template <int LA, int CA, int VA, int LB, int CB, int VB>
 cudaError_t run_fused(const FusedArgs& in, cudaStream_t st) {
   using FS = FusedShape<LA, CA, VA, LB, CB, VB>;
-  static int ctas = 0, per_sm = 0;
-  if (!ctas) {
-    cudaError_t e = resident_ctas(k_fused<LA, CA, VA, LB, CB, VB>, FS::NT, FS::SMEM, &ctas, &per_sm);
-    if (e != cudaSuccess) return e;
-  }
-  if (in.n1 != LB || in.n2 != LA || in.n1 % CA || in.n2 % CB || in.T < 1 || in.lc < 1 || in.lc > LA)
+  int ctas = 0, per_sm = 0;
+  cudaError_t e = resident_ctas(k_fused<LA, CA, VA, LB, CB, VB>, FS::NT, FS::SMEM, &ctas, &per_sm);
+  if (e != cudaSuccess) return e;
+  if (in.n1 != LB || in.n2 != LA || in.n1 % CA || in.n2 % CB || in.T < 1 || in.gc.lc < 1 || in.gc.lc > LA)
     return cudaErrorInvalidConfiguration;
   if ((uintptr_t)in.G & 15) return cudaErrorInvalidValue;
   FusedArgs a = in;

@@ -32,42 +32,60 @@ struct SkyConst {
   float kAf, kBf, kCf;
 };
 
-// Per-template spindown phase polynomial in s = j - J (J = rint(j_ref)):
-// phi(s) = p0 + p1 s + p2 s^2 + p3 s^3 cycles.  Double-float split for the
-// FP32 path (hi + lo carries ~48 bits), FP64 for the FP64 path.
+// Per-template spindown phase polynomial in x = j - J (J = rint(j_ref)):
+// phi(x) = p0 + p1 x + p2 x^2 + p3 x^3 cycles, and its differences over pass
+// A's sample spacing D (the samples of one butterfly),
+//   d1(x) = phi(x + D) - phi(x)     = q0 + q1 x + q2 x^2
+//   d2(x) = d1(x + D) - d1(x)       = r0 + r1 x
+//   d3    = d2(x + D) - d2(x)
+// FP32 path: double-float coefficients (hi + lo carries ~48 bits) and d3 in
+// units of 2^-32 cycles; FP64 path: doubles, and exp(-2 pi i d3).
 struct TmplCoef {
-  float hi[4], lo[4];
-  double p[4];
-  int J;
-  int pad_;
+  float phi[4][2], d1[3][2], d2[2][2];  // [power][hi, lo]
+  int d3, J;
+  double p[4], q[3], r[2], c3, s3;
 };
 
 // Spindown phase polynomial of one template (eqs. Fa, Fb: Phi_s =
 // 2 pi (f1dot tau^2/2 + f2dot tau^3/6)) for samples j with tau_j = (j - jr) dt,
-// expanded in s = j - J.  J is the integer nearest jr clamped into the data
-// [0, n - 1], so |s| < n < 2^24 stays exact in FP32 wherever the reference
-// time lies; p0, a phase common to every sample that cancels in 2F, is
-// reduced mod 1.
-__host__ __device__ inline TmplCoef spin_coef(double jr, int64_t n, double dt, double f1dot, double f2dot) {
+// expanded in x = j - J.  J is the integer nearest jr clamped into the data
+// [0, n - 1], so |x| <= 2^24 stays exact in FP32 wherever the reference time
+// lies; p0, a phase common to every sample that cancels in 2F, is reduced mod
+// 1, as are the other coefficients (x is an integer) where they reach a cycle.
+template <bool F64>  // with the FP64 path's factor of d3
+__device__ inline TmplCoef spin_coef(double jr, int64_t n, double dt, double f1dot, double f2dot, double D) {
   double J = rint(jr);
   if (!(J >= 0.0)) J = 0.0;
   if (J > (double)(n - 1)) J = (double)(n - 1);
-  const double e = jr - J;  // tau_j = (s - e) dt
+  const double e = jr - J;  // tau_j = (x - e) dt
   const double c2 = f1dot * dt * dt / 2.0;
   const double c3 = f2dot * dt * dt * dt / 6.0;
   TmplCoef c;
   c.p[3] = c3;
   c.p[2] = c2 - 3.0 * c3 * e;
   c.p[1] = -2.0 * c2 * e + 3.0 * c3 * e * e;
-  const double p0 = c2 * e * e - c3 * e * e * e;
-  c.p[0] = p0 - rint(p0);
-  for (int q = 0; q < 4; ++q) {
-    const float h = (float)c.p[q];
-    c.hi[q] = h;
-    c.lo[q] = (float)(c.p[q] - (double)h);
-  }
+  c.p[0] = c2 * e * e - c3 * e * e * e;
+  c.q[0] = D * (c.p[1] + D * (c.p[2] + D * c.p[3]));
+  c.q[1] = D * (2.0 * c.p[2] + D * 3.0 * c.p[3]);
+  c.q[2] = D * 3.0 * c.p[3];
+  c.r[0] = D * D * (2.0 * c.p[2] + D * 6.0 * c.p[3]);
+  c.r[1] = D * D * 6.0 * c.p[3];
+  auto split = [](double* v, float (*f)[2], int m) {
+    for (int q = 0; q < m; ++q) {
+      if (q == 0 || fabs(v[q]) >= 1.0) v[q] -= rint(v[q]);
+      f[q][0] = (float)v[q];
+      f[q][1] = (float)(v[q] - (double)f[q][0]);
+    }
+  };
+  double d3 = D * D * D * 6.0 * c.p[3];
+  d3 -= rint(d3);
+  split(c.p, c.phi, 4);
+  split(c.q, c.d1, 3);
+  split(c.r, c.d2, 2);
+  c.d3 = (int)(unsigned)(long long)rint(d3 * 4294967296.0);
+  c.c3 = c.s3 = 0.0;
+  if (F64) sincospi(-2.0 * d3, &c.s3, &c.c3);
   c.J = (int)J;
-  c.pad_ = 0;
   return c;
 }
 
@@ -149,9 +167,20 @@ template <typename T> __device__ __forceinline__ Pair<T> padd(const Pair<T>& x, 
 template <typename T> __device__ __forceinline__ Pair<T> psub(const Pair<T>& x, const Pair<T>& y) {
   return {x.ar - y.ar, x.ai - y.ai, x.br - y.br, x.bi - y.bi};
 }
+// (fused explicitly, here and in the transforms, so that every kernel that
+// shares this arithmetic gives the same bits)
+__device__ __forceinline__ float fmadd(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
 // multiply both members by the complex number (c, s)
 template <typename T> __device__ __forceinline__ Pair<T> pmul(const Pair<T>& x, T c, T s) {
-  return {x.ar * c - x.ai * s, x.ar * s + x.ai * c, x.br * c - x.bi * s, x.br * s + x.bi * c};
+  return {fmadd(x.ar, c, -(x.ai * s)), fmadd(x.ar, s, x.ai * c), fmadd(x.br, c, -(x.bi * s)), fmadd(x.br, s, x.bi * c)};
+}
+// eq. (Fstat) from the two transforms at one bin
+template <typename T> __device__ __forceinline__ T two_f(const Pair<T>& x, T kA, T kB, T kC) {
+  const T fa2 = fmadd(x.ar, x.ar, x.ai * x.ai);
+  const T fb2 = fmadd(x.br, x.br, x.bi * x.bi);
+  const T re = fmadd(x.ar, x.br, x.ai * x.bi);
+  return fmadd(kB, fa2, fmadd(kA, fb2, -(kC * re)));
 }
 // multiply by -i
 template <typename T> __device__ __forceinline__ Pair<T> pmul_mi(const Pair<T>& x) {
@@ -186,16 +215,33 @@ __device__ __forceinline__ Pair<double> pload_g(const PairMem<double>::type* __r
 __device__ __forceinline__ void sincospi_t(float x, float* s, float* c) { sincospif(x, s, c); }
 __device__ __forceinline__ void sincospi_t(double x, double* s, double* c) { sincospi(x, s, c); }
 
+// Column layout of the resampled series G for pass A: column n1 = j mod N1
+// takes lc pairs, its sample n2 = j / N1 at (n2 mod RL) lcs + n2 / RL, RL = 2^rl
+// residues of lcs = ceil(samples per column / RL) pairs each.
+struct GCol {
+  int64_t lc;
+  int lcs, rl;
+  __host__ __device__ __forceinline__ int at(int n2) const { return (n2 & ((1 << rl) - 1)) * lcs + (n2 >> rl); }
+};
+inline GCol g_columns(int64_t n, int64_t n1, int rl) {
+  const int64_t m = (n + n1 - 1) / n1;
+  const int lcs = (int)((m + (1 << rl) - 1) >> rl);
+  return GCol{(int64_t)lcs << rl, lcs, rl};
+}
+
 // ------------------------------------------------------------ host helpers
 void launch_sky(const Geo& g, int precision, double alpha, double delta, const void* const* xh,
-                const int* xh_dtype, void* z, void* G, int n1, int64_t lc, double* partials,
+                const int* xh_dtype, void* z, void* G, int n1, GCol gc, double* partials,
                 int n_blocks, SkyConst* sky, int* err, cudaStream_t st);
 // Timing table: entries needed to cover [t_lo, t_hi] at spacing h, and the
 // kernel that fills them (FP64 sincos, once per plan).
 int time_table_entries(double t_lo, double t_hi, double h);
 cudaError_t launch_time_table(const Geo& g, TimeTab* tab, cudaStream_t st);
 void launch_tmpl_coef(const SkyConst* sky, double dt, int64_t n, const fstat_template* tmpl,
-                      const int* order, int first, int count, TmplCoef* out, cudaStream_t st);
+                      const int* order, int first, int count, double spacing, bool f64, TmplCoef* out,
+                      cudaStream_t st);
+// samples between the inputs of one of pass A's first butterflies
+int64_t pass_a_spacing(int log2n, int log2_n2);
 void launch_check_finite(const void* x, int dtype, int64_t n, int* err, cudaStream_t st);
 // Gradient (adjoint.cu): per-plan sample tables and per-call scratch.
 size_t grad_table_bytes(const Geo& g);
@@ -206,14 +252,14 @@ int grad_launches(int n_cand, const Geo& g);  // kernels of one launch_grad
 cudaError_t launch_grad(const Geo& g, const void* tables, const fstat_candidate* cand_dev, int n_cand,
                         void* scratch, float* twoF, float* grad, cudaStream_t st);
 
-// Twiddle tables (tables.cu): pointers into one device block.
+// Twiddle tables of FP64 plans (tables.cu): pointers into one device block.
 struct TwiddleTables {
-  const void* a;   // pass A Stockham roots, N2 entries
-  const void* b;   // pass B Stockham roots, N1 entries
+  const void* a;   // pass A: Stockham roots, N2 entries
+  const void* b;   // pass B: Stockham roots, N1 entries, then the twists
   size_t bytes;
 };
-TwiddleTables twiddle_layout(int precision, int log2n1, int log2n2, void* base);
-cudaError_t build_twiddles(int precision, int log2n1, int log2n2, void* base, cudaStream_t st);
+TwiddleTables twiddle_layout(int log2n1, int log2n2, void* base);
+cudaError_t build_twiddles(int log2n1, int log2n2, void* base, cudaStream_t st);
 
 // Arguments of pass B's other epilogues: peaks mode reduces one template's
 // 2F in the kernel instead of writing it bin by bin (fstat_compute_peaks);
@@ -227,6 +273,7 @@ struct PeakArgs {
   float thr;
   int log2_band;                 // log2(bins per band)
   int shift;                     // accumulate: bin m adds to bin m - shift
+  int first;                     // accumulate: the sum starts here (every bin is written)
   int* err;                      // where a pass records FSTAT_ERR_TIMEOUT, or nullptr
   int wait_limit;                // polls of a tile's first bulk-copy wait (<= 0 with
                                  // wait_set: give up at once; unset: the default)
@@ -242,47 +289,51 @@ __device__ __forceinline__ unsigned long long band_key(float v, unsigned bin) {
   return ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - bin);
 }
 
-// FFT passes; ca / cb = columns / rows per CTA (0 = default for the length),
-// va / vb = radix schedule: bit 0 radix-8 first, bit 1 single shared
-// buffer, bit 2 (pass B) tiles by bulk tensor copies, bit 3 (pass A) three
-// CTAs per SM, va 16 (8192-point columns) the next column's samples staged
-// by a bulk copy under the transform.  res > 0: persistent grid of at most
-// res CTAs per SM (0 = every resident CTA).  err: where a pass records a
-// timed-out wait (FSTAT_ERR_TIMEOUT), or nullptr; wait_limit >= 0: polls of
-// pass A's staged-column waits (timeout tests).
-cudaError_t launch_pass_a_f32(int log2_n2, int ca, int va, const void* G, int64_t lc, int64_t n, int n1,
-                              const void* twA, const TmplCoef* coef, void* Z, cudaStream_t st, int res = 0,
-                              int* err = nullptr, int wait_limit = -1);
+// CTA-wide FFT passes of FP64 plans; ca / cb = columns / rows per CTA and va /
+// vb = schedule (0, the length's default, is the one compiled).  res > 0:
+// persistent grid of at most res CTAs per SM (0 = every resident CTA).
+cudaError_t launch_pass_a_f64(int log2_n2, int ca, int va, const void* G, GCol gc, int64_t n, int n1, const void* twA,
+                              const TmplCoef* coef, void* Z, cudaStream_t st, int res);
 // pk == nullptr: write 2F to out[n_fft]; otherwise reduce it as pk says.
-// err: where a pass records a timed-out wait (FSTAT_ERR_TIMEOUT), or nullptr
-// wait_limit >= 0: polls of each tile's first bulk-copy wait (timeout tests)
-cudaError_t launch_pass_b_f32(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                              const SkyConst* sky, float* out, cudaStream_t st,
-                              const PeakArgs* pk = nullptr, int res = 0, int* err = nullptr,
-                              int wait_limit = -1);
-cudaError_t launch_pass_a_f64(int log2_n2, int ca, int va, const void* G, int64_t lc, int64_t n, int n1,
-                              const void* twA, const TmplCoef* coef, void* Z, cudaStream_t st, int res = 0,
-                              int* err = nullptr, int wait_limit = -1);
 cudaError_t launch_pass_b_f64(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                              const SkyConst* sky, float* out, cudaStream_t st,
-                              const PeakArgs* pk = nullptr, int res = 0, int* err = nullptr,
-                              int wait_limit = -1);
-cudaError_t launch_pass_b_peak_f32(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                                   const SkyConst* sky, const PeakArgs& pk, cudaStream_t st, int res = 0);
+                              const SkyConst* sky, float* out, cudaStream_t st, const PeakArgs* pk, int res);
 cudaError_t launch_pass_b_peak_f64(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                                   const SkyConst* sky, const PeakArgs& pk, cudaStream_t st, int res = 0);
-// Accumulate mode: out[m - shift] += 2F[m] for 0 <= m - shift < n_fft.
-cudaError_t launch_pass_b_acc_f32(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                                  const SkyConst* sky, float* out, int shift, cudaStream_t st, int res = 0,
-                                  int* err = nullptr, int wait_limit = -1);
+                                   const SkyConst* sky, const PeakArgs& pk, cudaStream_t st, int res);
+// Accumulate mode: out[m - shift] += 2F[m] for 0 <= m - shift < n_fft; first:
+// the sum starts with this term (0 where no m reaches).
 cudaError_t launch_pass_b_acc_f64(int log2_n1, int cb, int vb, const void* Z, int n2, const void* twB,
-                                  const SkyConst* sky, float* out, int shift, cudaStream_t st, int res = 0,
-                                  int* err = nullptr, int wait_limit = -1);
+                                  const SkyConst* sky, float* out, int shift, bool first, cudaStream_t st, int res);
 // PeakArgs' wait fields from a plan's setting (< 0: the default limit)
 inline void set_wait(PeakArgs& a, int wait_limit) {
   a.wait_set = wait_limit >= 0;
   a.wait_limit = wait_limit >= 0 ? wait_limit : 0;
 }
+// The warp-local FP32 passes (fft_warp.cuh).  Z: the intermediates of the
+// launch's n_tmpl <= kMaxBatch templates, whose coefficients are coef[0..];
+// pass B writes template k to row ord[k] mod out_rows of out (ord == nullptr:
+// one template, to out).  staging: pass A's columns staged in shared memory
+// where that costs no occupancy (0), always (1; an error where they do not
+// fit) or never (2).
+constexpr int kMaxBatch = 8;
+// whether (ca, va) / (cb, vb) names a shape of the length
+bool pass_a_shape(int log2_n2, int ca, int va);
+bool pass_b_shape(int log2_n1, int cb, int vb);
+// Layout of their intermediate for pass B's tiles of 2^cb rows: element
+// (n1 = r + 2^rl j, k2) at ((k2 >> cb) N1 + r sub + j) 2^cb + k2 mod 2^cb.
+struct ZLayout { int cb, rl, sub; };
+ZLayout wpass_z_layout(int log2_n1, int cb);  // cb: rows per tile asked of pass B (0 = default)
+int wpass_b_rows(int log2_n1, int cb);        // and what it runs with
+cudaError_t launch_wpass_a(int log2_n2, int staging, const void* G, GCol gc, int64_t n, int n1, const TmplCoef* coef,
+                           void* const* Z, ZLayout zy, int n_tmpl, int* err, int wait_limit, cudaStream_t st, int res);
+int wpass_a_residues_log2(int log2_n2);  // GCol::rl for pass A of this length
+cudaError_t launch_wpass_b(int log2_n1, int cb, void* const* Z, int n_tmpl, int n2, const SkyConst* sky, float* out,
+                           const int* ord, int64_t out_rows, int* err, int wait_limit, cudaStream_t st, int res);
+cudaError_t launch_wpass_b_acc(int log2_n1, int cb, void* Z, int n2, const SkyConst* sky, float* out, int shift,
+                               bool first, int* err, int wait_limit, cudaStream_t st, int res);
+cudaError_t launch_wpass_b_peak(int log2_n1, int cb, void* const* Z, int n_tmpl, int n2, const SkyConst* sky,
+                                const int* ord, int n_bands, const PeakArgs& pk, int* err, int wait_limit,
+                                cudaStream_t st, int res);
+
 // One persistent launch of both FFT passes over T templates of one sky
 // group (fft_fused.cuh).  kRing intermediates in flight; launch state of
 // queue_ints(T) ints, zeroed before every launch.
@@ -292,7 +343,7 @@ inline size_t queue_ints(int T) { return (size_t)kQueueHead + 2 * (size_t)T; }
 
 struct FusedArgs {
   const float4* G;        // column-major resampled pairs (per-sky work)
-  int64_t lc;             // column length of G
+  GCol gc;                // layout of G
   int n;                  // samples
   int n1, n2;             // split: n1 columns of n2 points (pass A), n2 rows of n1 points (pass B)
   const TmplCoef* coef;   // [T] spindown coefficients of the launch's templates

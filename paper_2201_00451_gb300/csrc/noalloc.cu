@@ -30,11 +30,10 @@ constexpr int kNoallocMaxLog2 = 18;  // n_fft <= 2^18
 constexpr int64_t kNoallocMaxFft = int64_t(1) << kNoallocMaxLog2;
 constexpr int64_t kNoallocGElems = kNoallocMaxFft + (int64_t(1) << kMaxLog2);
 
-// Scratch: column-major copy of the input pairs, the FFT intermediate, the
-// twiddle tables and the per-call constants: 4.06 MB + 4 MB + 16 KB per device.
+// Scratch: column-major copy of the input pairs, the FFT intermediate and the
+// per-call constants: 4.06 MB + 4 MB per device.
 static __device__ __align__(256) float4 g_scratch_G[kNoallocGElems];
 static __device__ __align__(256) float4 g_scratch_Z[kNoallocMaxFft];
-static __device__ __align__(256) float2 g_scratch_tw[4 * (1 << (kNoallocMaxLog2 / 2))];
 static __device__ __align__(256) SkyConst g_scratch_sky;
 static __device__ __align__(256) TmplCoef g_scratch_coef;
 
@@ -42,7 +41,6 @@ constexpr int kMaxDevices = 64;
 struct DevPtrs {
   float4* G;
   float4* Z;
-  float2* tw;
   SkyConst* sky;
   TmplCoef* coef;
 };
@@ -62,7 +60,6 @@ int device_ptrs(DevPtrs* out) {
       DevPtrs p{};
       if (cudaGetSymbolAddress((void**)&p.G, g_scratch_G) != cudaSuccess) return FSTAT_ERR_CUDA;
       if (cudaGetSymbolAddress((void**)&p.Z, g_scratch_Z) != cudaSuccess) return FSTAT_ERR_CUDA;
-      if (cudaGetSymbolAddress((void**)&p.tw, g_scratch_tw) != cudaSuccess) return FSTAT_ERR_CUDA;
       if (cudaGetSymbolAddress((void**)&p.sky, g_scratch_sky) != cudaSuccess) return FSTAT_ERR_CUDA;
       if (cudaGetSymbolAddress((void**)&p.coef, g_scratch_coef) != cudaSuccess) return FSTAT_ERR_CUDA;
       g_ptrs[dev] = p;
@@ -73,31 +70,24 @@ int device_ptrs(DevPtrs* out) {
   return FSTAT_OK;
 }
 
-// Per-call constants: 2F weights from A, B, C and the spindown polynomial
-// in s = j - J for tau_j = tau0 + j dt = (j - j_ref) dt, j_ref = -tau0 / dt.
-__global__ void k_noalloc_setup(double A, double B, double C, double tau0, double dt, int64_t n,
-                                double f1dot, double f2dot) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double D = A * B - C * C;
-  g_scratch_sky.A = A;
-  g_scratch_sky.B = B;
-  g_scratch_sky.C = C;
-  g_scratch_sky.D = D;
-  g_scratch_sky.kA = 2.0 * A / D;
-  g_scratch_sky.kB = 2.0 * B / D;
-  g_scratch_sky.kC = 4.0 * C / D;
-  g_scratch_sky.kAf = (float)g_scratch_sky.kA;
-  g_scratch_sky.kBf = (float)g_scratch_sky.kB;
-  g_scratch_sky.kCf = (float)g_scratch_sky.kC;
-  g_scratch_coef = spin_coef(-tau0 / dt, n, dt, f1dot, f2dot);
-}
-
-// natural order j -> column-major [(j mod n1) * lc + j / n1]
-__global__ void k_noalloc_columns(const float4* __restrict__ g, int64_t n, int n1, int64_t lc,
-                                  float4* __restrict__ out) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-       j += (int64_t)gridDim.x * blockDim.x)
-    out[(j % n1) * lc + j / n1] = g[j];
+// Natural order j -> pass A's columns; and, on one thread of the last block
+// while the others copy, the per-call constants: 2F weights from A, B, C and
+// the spindown polynomial in x = j - J for tau_j = tau0 + j dt = (j - j_ref) dt,
+// j_ref = -tau0 / dt.
+struct NoallocArgs { double A, B, C, tau0, dt, f1dot, f2dot, spacing; };
+__global__ void k_noalloc_setup(const float4* __restrict__ g, int64_t n, int n1, GCol gc, float4* __restrict__ out,
+                                NoallocArgs a) {
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x != 0) return;
+    const double D = a.A * a.B - a.C * a.C;
+    g_scratch_sky.kAf = (float)(2.0 * a.A / D);
+    g_scratch_sky.kBf = (float)(2.0 * a.B / D);
+    g_scratch_sky.kCf = (float)(4.0 * a.C / D);
+    g_scratch_coef = spin_coef<false>(-a.tau0 / a.dt, n, a.dt, a.f1dot, a.f2dot, a.spacing);
+    return;
+  }
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)(gridDim.x - 1) * blockDim.x)
+    out[(j & (n1 - 1)) * gc.lc + gc.at((int)(j / n1))] = g[j];
 }
 
 }  // namespace
@@ -129,19 +119,20 @@ extern "C" int fstat_twoF_noalloc(const void* g_pairs, int64_t n_samples, int64_
   cudaStream_t st = (cudaStream_t)stream;
   const int log2n1 = log2n / 2, log2n2 = log2n - log2n1;
   const int n1 = 1 << log2n1, n2 = 1 << log2n2;
-  const int64_t lc = (n_samples + n1 - 1) / n1;
+  const GCol gc = g_columns(n_samples, n1, 0);
+  static_assert(kNoallocMaxLog2 <= 18, "columns of up to 512 points: one residue");
 
-  k_noalloc_setup<<<1, 32, 0, st>>>(A, B, C, tau0, dt, n_samples, f1dot, f2dot);
   int blocks = (int)((n_samples + 255) / 256);
   if (blocks > device_sm_count() * 16) blocks = device_sm_count() * 16;
-  k_noalloc_columns<<<blocks, 256, 0, st>>>((const float4*)g_pairs, n_samples, n1, lc, p.G);
+  k_noalloc_setup<<<blocks + 1, 256, 0, st>>>(
+      (const float4*)g_pairs, n_samples, n1, gc, p.G,
+      NoallocArgs{A, B, C, tau0, dt, f1dot, f2dot, (double)pass_a_spacing(log2n, log2n2)});
   if (cudaGetLastError() != cudaSuccess) return FSTAT_ERR_CUDA;
-  cudaError_t e = build_twiddles(FSTAT_MIXED, log2n1, log2n2, p.tw, st);
+  void* Z = p.Z;
+  cudaError_t e = launch_wpass_a(log2n2, 0, p.G, gc, n_samples, n1, p.coef, &Z, wpass_z_layout(log2n1, 0), 1, nullptr, -1,
+                                 st, 0);
   if (e != cudaSuccess) return FSTAT_ERR_CUDA;
-  TwiddleTables tt = twiddle_layout(FSTAT_MIXED, log2n1, log2n2, p.tw);
-  e = launch_pass_a_f32(log2n2, 0, 0, p.G, lc, n_samples, n1, tt.a, p.coef, p.Z, st);
-  if (e != cudaSuccess) return FSTAT_ERR_CUDA;
-  e = launch_pass_b_f32(log2n1, 0, 0, p.Z, n2, tt.b, p.sky, twoF, st);
+  e = launch_wpass_b(log2n1, 0, &Z, 1, n2, p.sky, twoF, nullptr, 1, nullptr, -1, st, 0);
   if (e != cudaSuccess) return FSTAT_ERR_CUDA;
   return FSTAT_OK;
 }

@@ -27,7 +27,7 @@
 using namespace fstat;
 
 namespace fstat {
-int fft_default_c(int log2_len, int pass_b, int precision);  // fft_a_f32.cu
+int fft_default_c(int log2_len, int pass_b, int precision);  // fft_shapes.cu
 }
 
 namespace {
@@ -43,7 +43,8 @@ struct fstat_plan {
   Geo geo;
   int device = 0;
   int log2n = 0, log2n1 = 0, log2n2 = 0;
-  int64_t n1 = 0, n2 = 0, lc = 0;
+  int64_t n1 = 0, n2 = 0;
+  GCol gc{};
   size_t pair_bytes = 16;
   void* xh[kMaxDet] = {};
   int dtype[kMaxDet] = {};
@@ -69,7 +70,7 @@ struct fstat_plan {
   SkyNode* nodes = nullptr;      // per-sky timing nodes (geo.nodes)
   NodeF32* nodes32 = nullptr;  // the same nodes in FP32 (geo.nodes32)
   SkyConst* sky = nullptr;
-  void* tw = nullptr;            // twiddle tables for the current split
+  void* tw = nullptr;            // FP64 plans: twiddle tables for the current split
   TwiddleTables tt{};
   int ca = 0, cb = 0;            // CTA shapes of pass A / pass B (0 = default)
   int cb_pk = -1, vb_pk = -1;    // pass B of the peaks mode when tuned apart (-1: cb, vb)
@@ -231,7 +232,7 @@ int run_sky(fstat_plan* p, double alpha, double delta, cudaStream_t st) {
   if (p->prof) { e = get_events(p); cudaEventRecord(e.a, st); }
   const void* xh[kMaxDet];
   for (int X = 0; X < kMaxDet; ++X) xh[X] = p->xh[X];
-  launch_sky(p->geo, p->d.precision, alpha, delta, xh, p->dtype, p->z, p->G, (int)p->n1, p->lc,
+  launch_sky(p->geo, p->d.precision, alpha, delta, xh, p->dtype, p->z, p->G, (int)p->n1, p->gc,
              p->partials, p->nblk, p->sky, p->d_err, st);
   CK(cudaGetLastError());
   p->n_launches += 4 + p->d.n_det;  // setup, delay table, step iii per detector, resampling, finalize
@@ -251,48 +252,61 @@ int set_split(fstat_plan* p, int log2n1) {
   p->log2n2 = log2n2;
   p->n1 = int64_t(1) << log2n1;
   p->n2 = int64_t(1) << log2n2;
-  p->lc = (p->d.n_samples + p->n1 - 1) / p->n1;
+  p->gc = g_columns(p->d.n_samples, p->n1, p->d.precision == FSTAT_FP64 ? 0 : wpass_a_residues_log2(log2n2));
   p->sky_valid = false;
   if (p->tw) {
-    p->tt = twiddle_layout(p->d.precision, log2n1, log2n2, p->tw);
-    CK(build_twiddles(p->d.precision, log2n1, log2n2, p->tw, 0));
+    p->tt = twiddle_layout(log2n1, log2n2, p->tw);
+    CK(build_twiddles(log2n1, log2n2, p->tw, 0));
     CK(cudaStreamSynchronize(0));
   }
   return FSTAT_OK;
 }
 
-cudaError_t launch_a(fstat_plan* p, int ca, int va, const TmplCoef* coef, cudaStream_t st, void* Z = nullptr,
+// FP32 plans run the warp-local passes whatever the schedule code (the codes
+// name schedules of the CTA-wide passes, which they beat throughout; lengths
+// and shapes those were never compiled for stay refused).
+bool warp_passes(const fstat_plan* p) { return p->d.precision != FSTAT_FP64; }
+
+// cb: rows per tile of the pass B that follows
+cudaError_t launch_a(fstat_plan* p, int ca, int va, int cb, const TmplCoef* coef, cudaStream_t st, void* Z = nullptr,
                      int res = -1) {
-  const TwiddleTables& t = p->tt;
   if (!Z) Z = p->Z;
   if (res < 0) res = p->ra;
   ++p->n_launches;
-  return p->d.precision == FSTAT_FP64
-      ? launch_pass_a_f64(p->log2n2, ca, va, p->G, p->lc, p->d.n_samples, (int)p->n1, t.a, coef, Z, st, res, p->d_err,
-                          p->wait_limit)
-      : launch_pass_a_f32(p->log2n2, ca, va, p->G, p->lc, p->d.n_samples, (int)p->n1, t.a, coef, Z, st, res, p->d_err,
-                          p->wait_limit);
+  if (warp_passes(p)) {
+    if (!pass_a_shape(p->log2n2, ca, va)) return cudaErrorInvalidConfiguration;
+    const int staging = va >= 16 ? 1 : va == 2 ? 2 : 0;  // staged columns asked for; none asked for
+    return launch_wpass_a(p->log2n2, staging, p->G, p->gc, p->d.n_samples, (int)p->n1, coef, &Z,
+                          wpass_z_layout(p->log2n1, cb), 1, p->d_err, p->wait_limit, st, res);
+  }
+  return launch_pass_a_f64(p->log2n2, ca, va, p->G, p->gc, p->d.n_samples, (int)p->n1, p->tt.a, coef, Z, st, res);
 }
 
 cudaError_t launch_b(fstat_plan* p, int cb, int vb, float* out, cudaStream_t st, void* Z = nullptr,
                      const PeakArgs* pk = nullptr, int res = -1) {
-  const TwiddleTables& t = p->tt;
   if (!Z) Z = p->Z;
   if (res < 0) res = p->rb;
   ++p->n_launches;
-  return p->d.precision == FSTAT_FP64
-      ? launch_pass_b_f64(p->log2n1, cb, vb, Z, (int)p->n2, t.b, p->sky, out, st, pk, res, p->d_err, p->wait_limit)
-      : launch_pass_b_f32(p->log2n1, cb, vb, Z, (int)p->n2, t.b, p->sky, out, st, pk, res, p->d_err, p->wait_limit);
+  if (warp_passes(p)) {
+    if (!pass_b_shape(p->log2n1, cb, vb)) return cudaErrorInvalidConfiguration;
+    if (pk)
+      return launch_wpass_b_peak(p->log2n1, cb, &Z, 1, (int)p->n2, p->sky, nullptr,
+                                 pk->band_key ? (int)(p->d.n_fft >> pk->log2_band) : 0, *pk, p->d_err, p->wait_limit, st,
+                                 res);
+    return launch_wpass_b(p->log2n1, cb, &Z, 1, (int)p->n2, p->sky, out, nullptr, 1, p->d_err, p->wait_limit, st, res);
+  }
+  return launch_pass_b_f64(p->log2n1, cb, vb, Z, (int)p->n2, p->tt.b, p->sky, out, st, pk, res);
 }
 
-cudaError_t launch_b_acc(fstat_plan* p, float* out, int shift, cudaStream_t st, void* Z) {
-  const TwiddleTables& t = p->tt;
+double spin_spacing(const fstat_plan* p) { return (double)pass_a_spacing(p->log2n, p->log2n2); }
+
+cudaError_t launch_b_acc(fstat_plan* p, float* out, int shift, bool first, cudaStream_t st, void* Z) {
   ++p->n_launches;
-  return p->d.precision == FSTAT_FP64
-      ? launch_pass_b_acc_f64(p->log2n1, p->cb, p->vb, Z, (int)p->n2, t.b, p->sky, out, shift, st, p->rb, p->d_err,
-                              p->wait_limit)
-      : launch_pass_b_acc_f32(p->log2n1, p->cb, p->vb, Z, (int)p->n2, t.b, p->sky, out, shift, st, p->rb, p->d_err,
-                              p->wait_limit);
+  if (warp_passes(p)) {
+    if (!pass_b_shape(p->log2n1, p->cb, p->vb)) return cudaErrorInvalidConfiguration;
+    return launch_wpass_b_acc(p->log2n1, p->cb, Z, (int)p->n2, p->sky, out, shift, first, p->d_err, p->wait_limit, st, p->rb);
+  }
+  return launch_pass_b_acc_f64(p->log2n1, p->cb, p->vb, Z, (int)p->n2, p->tt.b, p->sky, out, shift, first, st, p->rb);
 }
 
 }  // namespace
@@ -373,7 +387,9 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   p->nblk = (int)((N + kSkyBlock - 1) / kSkyBlock);
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = palloc(p, &p->z, (size_t)d.n_det * N * zb);
-  if (e == cudaSuccess) e = palloc(p, &p->G, (size_t)(N + (int64_t(1) << kMaxLog2)) * p->pair_bytes);
+  // whole columns of whole residues: up to N1 RL <= 2^12 x 16 pairs of padding
+  if (e == cudaSuccess)
+    e = palloc(p, &p->G, (size_t)(N + (int64_t(1) << (kMaxLog2 + (d.precision == FSTAT_FP64 ? 0 : 4)))) * p->pair_bytes);
   if (e == cudaSuccess) e = palloc(p, &p->Z, (size_t)d.n_fft * p->pair_bytes);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
   // short transforms leave most of the GPU idle between launches: four
@@ -412,7 +428,7 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   }
   if (e == cudaSuccess) e = palloc(p, &p->partials, (size_t)3 * p->nblk * sizeof(double));
   if (e == cudaSuccess) e = palloc(p, &p->sky, sizeof(SkyConst));
-  if (e == cudaSuccess) e = palloc(p, &p->tw, (size_t)4 * (size_t(1) << kMaxLog2A) * 16);
+  if (e == cudaSuccess && d.precision == FSTAT_FP64) e = palloc(p, &p->tw, (size_t)6 * (size_t(1) << kMaxLog2) * 16);
   if (e == cudaSuccess) e = palloc(p, &p->d_err, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_err, 2 * sizeof(int));
@@ -424,7 +440,9 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
     delete p;
     return cuda_status(e);
   }
+  // the tables are complete before any call, on whatever stream, reads them
   int rc = set_split(p, p->log2n1);
+  if (!rc) rc = cuda_status(cudaStreamSynchronize(0));
   if (rc) {
     free_all(p);
     delete p;
@@ -588,7 +606,7 @@ int enqueue_fused(fstat_plan* p, int64_t i, int64_t j, const int* d_ord, const T
     const int T = (int)std::min<int64_t>(kFusedMaxT, j - k0);
     FusedArgs a{};
     a.G = (const float4*)p->G;
-    a.lc = p->lc;
+    a.gc = p->gc;
     a.n = (int)p->d.n_samples;
     a.n1 = (int)p->n1;
     a.n2 = (int)p->n2;
@@ -636,7 +654,8 @@ int enqueue_compute(fstat_plan* p, const fstat_template* h_tmpl, const int* h_or
       int rc = run_sky(p, t0.alpha, t0.delta, st);
       if (rc) return rc;
     }
-    launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, d_tmpl, d_ord, (int)i, (int)(j - i), d_coef, st);
+    launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, d_tmpl, d_ord, (int)i, (int)(j - i), spin_spacing(p),
+                     p->d.precision == FSTAT_FP64, d_coef, st);
     ++p->n_launches;
     CK(cudaGetLastError());
     if (!po && p->fused && fused_ok(p)) {
@@ -672,14 +691,15 @@ int enqueue_compute(fstat_plan* p, const fstat_template* h_tmpl, const int* h_or
       void* Zb = p->Zs[q];
       EventPair ea{}, eb{};
       if (prof) { ea = get_events(p); cudaEventRecord(ea.a, s); }
-      cudaError_t e = launch_a(p, p->ca, p->va, coef, s, Zb);
+      const bool own = po && p->cb_pk >= 0;  // the peaks mode's own pass-B shape
+      const int cb = own ? p->cb_pk : p->cb, vb = own ? p->vb_pk : p->vb;
+      cudaError_t e = launch_a(p, p->ca, p->va, cb, coef, s, Zb);
       if (e != cudaSuccess) return cuda_status(e);
       if (prof) {
         cudaEventRecord(ea.b, s); p->ev[0].push_back(ea); p->launches[0]++;
         eb = get_events(p); cudaEventRecord(eb.a, s);
       }
-      const bool own = po && p->cb_pk >= 0;  // the peaks mode's own pass-B shape
-      e = launch_b(p, own ? p->cb_pk : p->cb, own ? p->vb_pk : p->vb, out, s, Zb, po ? &pk : nullptr);
+      e = launch_b(p, cb, vb, out, s, Zb, po ? &pk : nullptr);
       if (e != cudaSuccess) return cuda_status(e);
       if (prof) { cudaEventRecord(eb.b, s); p->ev[1].push_back(eb); p->launches[1]++; }
     }
@@ -798,7 +818,6 @@ int fstat_semicoherent(fstat_plan* const* seg, int n_seg, const fstat_template* 
     p->staged_pending = true;
     ns = std::min(ns, p->nstream);
   }
-  CK(cudaMemsetAsync(twoF, 0, (size_t)n * nfft * sizeof(float), st));
   // Templates rotate over the first plan's streams; every segment of one
   // template runs on the same stream, so its additions to the output row
   // are ordered, and each segment uses its own plan's intermediate for
@@ -814,7 +833,8 @@ int fstat_semicoherent(fstat_plan* const* seg, int n_seg, const fstat_template* 
         int rc = run_sky(p, t0.alpha, t0.delta, st);
         if (rc) return rc;
       }
-      launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, (int)i, (int)(j - i), p->d_coef, st);
+      launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, (int)i, (int)(j - i), spin_spacing(p),
+                       p->d.precision == FSTAT_FP64, p->d_coef, st);
       ++p->n_launches;
       CK(cudaGetLastError());
     }
@@ -829,8 +849,8 @@ int fstat_semicoherent(fstat_plan* const* seg, int n_seg, const fstat_template* 
       float* out = twoF + (int64_t)ord[k] * nfft;
       for (int s = 0; s < n_seg; ++s) {
         fstat_plan* p = seg[s];
-        cudaError_t e = launch_a(p, p->ca, p->va, p->d_coef + k, sq, p->Zs[q]);
-        if (e == cudaSuccess) e = launch_b_acc(p, out, shift[(size_t)s * n + ord[k]], sq, p->Zs[q]);
+        cudaError_t e = launch_a(p, p->ca, p->va, p->cb, p->d_coef + k, sq, p->Zs[q]);
+        if (e == cudaSuccess) e = launch_b_acc(p, out, shift[(size_t)s * n + ord[k]], s == 0, sq, p->Zs[q]);
         if (e != cudaSuccess) return cuda_status(e);
       }
     }
@@ -1075,13 +1095,13 @@ int fstat_export_sky(fstat_plan* p, double alpha, double delta, double* ga, doub
   int rc = run_sky(p, alpha, delta, st);
   if (rc) return rc;
   const int64_t N = p->d.n_samples;
-  std::vector<unsigned char> buf((size_t)(p->n1 * p->lc) * p->pair_bytes);
+  std::vector<unsigned char> buf((size_t)(p->n1 * p->gc.lc) * p->pair_bytes);
   CK(cudaMemcpyAsync(buf.data(), p->G, buf.size(), cudaMemcpyDeviceToHost, st));
   SkyConst sc;
   CK(cudaMemcpyAsync(&sc, p->sky, sizeof(sc), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   for (int64_t j = 0; j < N; ++j) {
-    int64_t pos = (j % p->n1) * p->lc + j / p->n1;
+    int64_t pos = (j % p->n1) * p->gc.lc + p->gc.at((int)(j / p->n1));
     double v[4];
     if (p->pair_bytes == 16) {
       const float* f = reinterpret_cast<const float*>(buf.data()) + 4 * pos;
@@ -1239,7 +1259,7 @@ std::string tune_key(const fstat_plan* p) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, p->device) != cudaSuccess) prop.name[0] = 0;
   char buf[400];
-  std::snprintf(buf, sizeof buf, "v5|%s|N=%lld|nfft=%lld|prec=%d|ndet=%d|ns=%d", prop.name,
+  std::snprintf(buf, sizeof buf, "v6|%s|N=%lld|nfft=%lld|prec=%d|ndet=%d|ns=%d", prop.name,
                 (long long)p->d.n_samples, (long long)p->d.n_fft, p->d.precision, p->d.n_det, p->nstream);
   for (char* c = buf; *c; ++c)
     if (*c == ' ' || *c == '\t') *c = '_';
@@ -1266,18 +1286,20 @@ void save_tune(const std::string& key, const Choice& c) {
       << c.cbp << " " << c.vbp << "\n";
 }
 
+constexpr int kTunePipe = 32;  // templates in the autotuner's pipeline timings
+
 // mean time (ms) of `reps` launches of pass A (which = 0) or pass B (which = 1)
 float time_pass(fstat_plan* p, int which, int c, int v, const TmplCoef* coef, float* out, cudaStream_t st,
                 cudaEvent_t e0, cudaEvent_t e1) {
   const int reps = 5;
-  cudaError_t e = which == 0 ? launch_a(p, c, v, coef, st) : launch_b(p, c, v, out, st);
+  cudaError_t e = which == 0 ? launch_a(p, c, v, p->cb, coef, st) : launch_b(p, c, v, out, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return -1.f;
   }
   cudaEventRecord(e0, st);
   for (int r = 0; r < reps; ++r) {
-    if (which == 0) launch_a(p, c, v, coef, st);
+    if (which == 0) launch_a(p, c, v, p->cb, coef, st);
     else launch_b(p, c, v, out, st);
   }
   cudaEventRecord(e1, st);
@@ -1287,40 +1309,40 @@ float time_pass(fstat_plan* p, int which, int c, int v, const TmplCoef* coef, fl
   return ms / reps;
 }
 
-// Pass B of the peaks mode alone over every compiled shape at the current
-// split: 256 whole-row bands and the threshold 70 of Sec. 5.4 (no 2F store,
-// so its best shape can differ from the dense pass's).  Returns the fastest
-// (cb, vb), or (-1, -1) when none ran.
-void tune_peaks(fstat_plan* p, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int* cbp, int* vbp) {
+// The pass-B shape of the peaks mode (256 whole-row bands and the threshold
+// 70 of Sec. 5.4) at the current split and pass-A shape: without the 2F store
+// its best shape can differ from the dense pass's.  FP32 plans time every
+// compiled row count in the overlapped template pipeline, since pass A's
+// stores follow the row count; FP64 has one shape.  (-1, -1): the dense pass's.
+template <typename Run>
+void tune_peaks(fstat_plan* p, cudaStream_t st, const Run& pipeline, int* cbp, int* vbp) {
   *cbp = *vbp = -1;
-  if (p->d.n_fft < 256) return;
+  if (p->d.precision == FSTAT_FP64 || p->d.n_fft < (1 << 14)) return;
   unsigned long long* keys = nullptr;
   fstat_peak* list = nullptr;
-  if (cudaMalloc(&keys, (256 + 1) * sizeof(unsigned long long)) != cudaSuccess) return;
+  if (cudaMalloc(&keys, (kTunePipe * 256 + 1) * sizeof(unsigned long long)) != cudaSuccess) return;
   if (cudaMalloc(&list, 1024 * sizeof(fstat_peak)) != cudaSuccess) { cudaFree(keys); return; }
-  PeakArgs pk{};
-  pk.band_key = keys;
-  pk.count = keys + 256;
-  pk.peaks = list;
-  pk.cap = 1024;
-  pk.thr = 70.f;
-  pk.log2_band = ilog2_exact(p->d.n_fft) - 8;
-  static const int kCb[] = {0, 1, 2, 4, 8};
+  cudaMemsetAsync(keys, 0, (kTunePipe * 256 + 1) * sizeof(unsigned long long), st);
+  fstat_peak_out po{};
+  po.threshold = 70.f;
+  po.n_bands = 256;
+  po.peaks = list;
+  po.capacity = 1024;
+  po.n_peaks = keys + kTunePipe * 256;
+  unsigned long long* const own = p->keys;
+  p->keys = keys;
   float best = 1e30f;
-  for (int v = 0; v < 8; ++v) {
-    for (int c : kCb) {
-      cudaMemsetAsync(keys, 0, (256 + 1) * sizeof(unsigned long long), st);
-      if (launch_b(p, c, v, nullptr, st, nullptr, &pk) != cudaSuccess) { cudaGetLastError(); continue; }
-      const int reps = 5;
-      cudaEventRecord(e0, st);
-      for (int r = 0; r < reps; ++r) launch_b(p, c, v, nullptr, st, nullptr, &pk);
-      cudaEventRecord(e1, st);
-      if (cudaEventSynchronize(e1) != cudaSuccess) { cudaGetLastError(); continue; }
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (ms / reps < best) { best = ms / reps; *cbp = c; *vbp = v; }
-    }
+  int best_cb = -1;
+  for (int c : {1, 2, 4, 8}) {
+    if (!pass_b_shape(p->log2n1, c, 0) || wpass_b_rows(p->log2n1, c) != c) continue;
+    p->cb_pk = c;
+    p->vb_pk = 0;
+    const float ms = pipeline(&po);
+    if (ms > 0.f && ms < best) { best = ms; best_cb = c; }
   }
+  p->keys = own;
+  p->cb_pk = p->vb_pk = -1;
+  if (best_cb > 0) { *cbp = best_cb; *vbp = 0; }
   cudaFree(keys);
   cudaFree(list);
 }
@@ -1351,7 +1373,7 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
       return FSTAT_OK;
     }
   }
-  const int kPipe = 32;  // templates in the overlapped pipeline timing
+  const int kPipe = kTunePipe;
   int rc = ensure_capacity(p, kPipe);
   if (rc) return rc;
   if (p->staged_pending) { CK(cudaEventSynchronize(p->staged)); p->staged_pending = false; }
@@ -1374,92 +1396,80 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
   Choice best{p->log2n1, 0, 0, 0, 0, 0};
   float best_ms = 1e30f;
   p->fused = false;
-  static const int kCa[] = {0, 1, 2, 4};
-  static const int kCb[] = {0, 1, 2, 4, 8};
   const bool saved_prof = p->prof;
   p->prof = false;
+  p->cb_pk = p->vb_pk = -1;
+  // ms per template of the overlapped pipeline with the plan's current shapes
+  // (po: the peaks mode); < 0 where they do not run, rc set on a CUDA error.
+  // Best of three trials of two pipelines each: shapes differ by a few
+  // percent, about the spread of a single short trial.
+  auto pipeline = [&](const fstat_peak_out* po) -> float {
+    auto once = [&] {
+      return enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, 1, st, false, false,
+                             po);
+    };
+    if (once()) { cudaGetLastError(); return -1.f; }
+    float ms = 1e30f;
+    for (int trial = 0; trial < 3; ++trial) {
+      cudaEventRecord(e0, st);
+      for (int rep = 0; rep < 2; ++rep) once();
+      cudaEventRecord(e1, st);
+      if (cudaEventSynchronize(e1) != cudaSuccess) { rc = FSTAT_ERR_CUDA; return -1.f; }
+      float t = 0.f;
+      cudaEventElapsedTime(&t, e0, e1);
+      ms = std::min(ms, t / (2 * kPipe));
+    }
+    return ms;
+  };
   for (int l1 = lo; l1 <= hi && rc == FSTAT_OK; ++l1) {
     rc = set_split(p, l1);
     if (rc) break;
     rc = run_sky(p, 0.3, -0.5, st);
     if (rc) break;
-    launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, 0, kPipe, p->d_coef, st);
-    // isolated timings of every compiled shape of each pass
+    launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, 0, kPipe, spin_spacing(p),
+                     p->d.precision == FSTAT_FP64, p->d_coef, st);
+    // isolated timings of every distinct shape of each pass: for FP32 plans
+    // pass A with columns staged where that costs no occupancy (0) or never
+    // (2), pass B with 1 to 8 rows per tile; FP64 has one of each
     std::vector<std::pair<float, std::pair<int, int>>> ta, tb;
-    // schedules: radix-8 first (bit 0), one buffer (bit 1), for pass B tile
-    // loads by the tensor-memory-access engine (bit 2), for pass A three
-    // CTAs per SM (bit 3) and columns staged apart (16 at 8192 points, 18 at
-    // 4096), for pass B half of the next tile staged apart (8)
-    static const int kVa[] = {0, 1, 2, 3, 10, 16, 18};
-    for (int v : kVa) {
-      for (int c : kCa) {
-        float ms = time_pass(p, 0, c, v, p->d_coef, out, st, e0, e1);
-        if (ms > 0.f) ta.push_back({ms, {c, v}});
-      }
+    for (int v : {0, 2}) {
+      if (v && (!warp_passes(p) || !pass_a_shape(p->log2n2, 0, v))) continue;
+      const float ms = time_pass(p, 0, 0, v, p->d_coef, out, st, e0, e1);
+      if (ms > 0.f) ta.push_back({ms, {0, v}});
     }
-    for (int v = 0; v <= 8; ++v) {
-      for (int c : kCb) {
-        float ms = time_pass(p, 1, c, v, p->d_coef, out, st, e0, e1);
-        if (ms > 0.f) tb.push_back({ms, {c, v}});
-      }
+    for (int c : {0, 1, 2, 4, 8}) {
+      if (c && (!warp_passes(p) || !pass_b_shape(p->log2n1, c, 0) || wpass_b_rows(p->log2n1, c) != c ||
+                c == wpass_b_rows(p->log2n1, 0)))
+        continue;
+      const float ms = time_pass(p, 1, c, 0, p->d_coef, out, st, e0, e1);
+      if (ms > 0.f) tb.push_back({ms, {c, 0}});
     }
     std::sort(ta.begin(), ta.end());
     std::sort(tb.begin(), tb.end());
     // the best few of each, paired in the overlapped template pipeline
-    for (size_t ia = 0; ia < std::min<size_t>(3, ta.size()); ++ia) {
+    for (size_t ia = 0; ia < ta.size(); ++ia) {
       for (size_t ib = 0; ib < std::min<size_t>(3, tb.size()); ++ib) {
         p->ca = ta[ia].second.first;
         p->va = ta[ia].second.second;
         p->cb = tb[ib].second.first;
         p->vb = tb[ib].second.second;
-        int r = enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, 1, st,
-                                false, false);
-        if (r) { cudaGetLastError(); continue; }
-        // best of three trials of two pipelines each: the pairs differ by a
-        // few percent, about the spread of a single short trial
-        float ms = 1e30f;
-        for (int trial = 0; trial < 3 && rc == FSTAT_OK; ++trial) {
-          cudaEventRecord(e0, st);
-          for (int rep = 0; rep < 2; ++rep)
-            enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, 1, st, false,
-                            false);
-          cudaEventRecord(e1, st);
-          if (cudaEventSynchronize(e1) != cudaSuccess) { rc = FSTAT_ERR_CUDA; break; }
-          float t = 0.f;
-          cudaEventElapsedTime(&t, e0, e1);
-          ms = std::min(ms, t / (2 * kPipe));
-        }
+        const float ms = pipeline(nullptr);
         if (rc) break;
-        if (ms < best_ms) { best_ms = ms; best = Choice{l1, p->ca, p->va, p->cb, p->vb, 0}; }
+        if (ms > 0.f && ms < best_ms) { best_ms = ms; best = Choice{l1, p->ca, p->va, p->cb, p->vb, 0}; }
       }
       if (rc) break;
     }
     // the persistent launch of both passes over the same templates
     if (rc == FSTAT_OK && fused_ok(p)) {
       p->fused = true;
-      int r = enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, 1, st, false,
-                              false);
-      if (r == FSTAT_OK && cudaStreamSynchronize(st) == cudaSuccess) {
-        float ms = 1e30f;
-        for (int trial = 0; trial < 3 && rc == FSTAT_OK; ++trial) {
-          cudaEventRecord(e0, st);
-          for (int rep = 0; rep < 2; ++rep)
-            enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, 1, st, false,
-                            false);
-          cudaEventRecord(e1, st);
-          if (cudaEventSynchronize(e1) != cudaSuccess) { rc = FSTAT_ERR_CUDA; break; }
-          float t = 0.f;
-          cudaEventElapsedTime(&t, e0, e1);
-          ms = std::min(ms, t / (2 * kPipe));
-        }
-        if (rc == FSTAT_OK && ms < best_ms) { best_ms = ms; best = Choice{l1, p->ca, p->va, p->cb, p->vb, 1}; }
-      } else {
-        cudaGetLastError();
+      const float ms = pipeline(nullptr);
+      if (rc == FSTAT_OK && ms > 0.f && ms < best_ms) {
+        best_ms = ms;
+        best = Choice{l1, p->ca, p->va, p->cb, p->vb, 1};
       }
       p->fused = false;
     }
   }
-  cudaFree(out);
   if (rc == FSTAT_OK) rc = set_split(p, best.l1);
   if (rc == FSTAT_OK) {
     p->ca = best.ca;
@@ -1467,10 +1477,16 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
     p->cb = best.cb;
     p->vb = best.vb;
     p->fused = best.fused != 0 && fused_ok(p);
-    tune_peaks(p, st, e0, e1, &best.cbp, &best.vbp);
+    rc = run_sky(p, 0.3, -0.5, st);
+    if (rc == FSTAT_OK) {
+      launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, 0, kPipe, spin_spacing(p),
+                     p->d.precision == FSTAT_FP64, p->d_coef, st);
+      tune_peaks(p, st, pipeline, &best.cbp, &best.vbp);
+    }
     p->cb_pk = best.cbp;
     p->vb_pk = best.vbp;
   }
+  cudaFree(out);
   p->prof = saved_prof;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -74,7 +74,7 @@ namespace {
 // Radix-16 DFT stage two ways, for the choice between CUDA cores and tensor
 // cores in the FFT passes (X_m = sum_s x_s exp(-2 pi i m s / 16), the first
 // radix-16 stage of every column and row transform):
-//   method 0: the FFT passes' own butterflies (fft::dft16 on Fa/Fb pairs in
+//   method 0: the FFT passes' own butterflies (fft::dft on Fa/Fb pairs in
 //             registers, CUDA cores);
 //   method 1: the same stage as a matrix product on the tensor cores: the
 //             real 32 x 32 form of the 16-point DFT matrix times 32 x 8
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) k_dft16_simt(const float4* __restrict__ i
     Pair<float> v[16];
 #pragma unroll
     for (int s = 0; s < 16; ++s) v[s] = pload(buf + s * 256 + t);
-    fft::dft16(v);
+    fft::dft<float, 16>(v);
 #pragma unroll
     for (int s = 0; s < 16; ++s) pstore(buf + s * 256 + t, v[s]);
   }

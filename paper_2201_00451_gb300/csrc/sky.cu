@@ -1,8 +1,7 @@
 // Per-sky kernels: Sec. 3 steps (iii), (iv), (v) of the resampling method,
 // antenna weighting, the noise-weighted detector sum, and the antenna-pattern
 // integrals A, B, C, D of eq. (Fstat).  The result G = (G_a, G_b) is stored
-// in the column-major layout the FFT pass A reads: element j goes to
-// G[(j mod n1) * lc + j / n1].
+// in the column-major layout the FFT pass A reads (GCol).
 //
 // Timing (t_m, the inversion T + t_m(T) = t_b, u = (T - t0)/dt) is FP64 in
 // both precisions; f_h t_m is reduced mod 1 in FP64 before the sincos.
@@ -354,7 +353,7 @@ static_assert(kWin % 2 == 0, "whole 16-byte loads of complex64 samples");
 template <typename T, typename TZ>
 __global__ void __launch_bounds__(kSkyBlock)
 k_resample(Geo g, const SkyConst* __restrict__ skyp, const TZ* __restrict__ z,
-           typename PairMem<T>::type* __restrict__ G, int n1, int64_t lc, double* __restrict__ partials) {
+           typename PairMem<T>::type* __restrict__ G, int n1, GCol gc, double* __restrict__ partials) {
   (void)skyp;  // the sky position enters through the timing nodes
   __shared__ __align__(16) TZ win[kWin];
   __shared__ TapK<T> tk[2 * kMaxD + 1];
@@ -544,8 +543,8 @@ k_resample(Geo g, const SkyConst* __restrict__ skyp, const TZ* __restrict__ z,
     acc.bi += wb * zi;
   }
   if (j < g.n) {
-    int64_t n1i = j % n1, n2i = j / n1;
-    pstore(G + n1i * lc + n2i, acc);
+    const int n2i = (int)(j / n1);
+    pstore(G + (j % n1) * gc.lc + gc.at(n2i), acc);
   }
   // the fully valid segments' A, B, C: sum_r a(r)^2 over a segment = a^T M a
   // in the four node values (likewise b^T M b, a^T M b), one thread per
@@ -648,13 +647,14 @@ k_sky_finalize(const double* __restrict__ partials, int nblocks, SkyConst* sky, 
 }
 
 // Per-template spindown polynomial in s = j - J (see TmplCoef).
+template <bool F64>
 __global__ void k_tmpl_coef(const SkyConst* __restrict__ sky, double dt, int64_t n,
                             const fstat_template* __restrict__ tmpl, const int* __restrict__ order,
-                            int first, int count, TmplCoef* __restrict__ out) {
+                            int first, int count, double spacing, TmplCoef* __restrict__ out) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const fstat_template tp = tmpl[order[first + i]];
-  out[first + i] = spin_coef(sky->j_ref, n, dt, tp.f1dot, tp.f2dot);
+  out[first + i] = spin_coef<F64>(sky->j_ref, n, dt, tp.f1dot, tp.f2dot, spacing);
 }
 
 // (after k_sky_table on the same stream: the phase uses this sky's t_m)
@@ -678,7 +678,7 @@ cudaError_t launch_time_table(const Geo& g, TimeTab* tab, cudaStream_t st) {
 }
 
 void launch_sky(const Geo& g, int precision, double alpha, double delta, const void* const* xh,
-                const int* xh_dtype, void* z, void* G, int n1, int64_t lc, double* partials,
+                const int* xh_dtype, void* z, void* G, int n1, GCol gc, double* partials,
                 int n_blocks, SkyConst* sky, int* err, cudaStream_t st) {
   k_sky_setup<<<1, 32, 0, st>>>(g, alpha, delta, sky);
   k_sky_table<<<(g.tab_n + 255) / 256, 256, 0, st>>>(g, sky);
@@ -699,18 +699,20 @@ void launch_sky(const Geo& g, int precision, double alpha, double delta, const v
   }
   if (precision == FSTAT_FP64) {
     k_resample<double, double2><<<n_blocks, kSkyBlock, 0, st>>>(
-        g, sky, (const double2*)z, (PairMem<double>::type*)G, n1, lc, partials);
+        g, sky, (const double2*)z, (PairMem<double>::type*)G, n1, gc, partials);
   } else {
     k_resample<float, float2><<<n_blocks, kSkyBlock, 0, st>>>(
-        g, sky, (const float2*)z, (float4*)G, n1, lc, partials);
+        g, sky, (const float2*)z, (float4*)G, n1, gc, partials);
   }
   k_sky_finalize<<<1, 1024, 0, st>>>(partials, n_blocks, sky, err);
 }
 
 void launch_tmpl_coef(const SkyConst* sky, double dt, int64_t n, const fstat_template* tmpl,
-                      const int* order, int first, int count, TmplCoef* out, cudaStream_t st) {
+                      const int* order, int first, int count, double spacing, bool f64, TmplCoef* out,
+                      cudaStream_t st) {
   if (count <= 0) return;
-  k_tmpl_coef<<<(count + 127) / 128, 128, 0, st>>>(sky, dt, n, tmpl, order, first, count, out);
+  const auto k = f64 ? k_tmpl_coef<true> : k_tmpl_coef<false>;
+  k<<<(count + 127) / 128, 128, 0, st>>>(sky, dt, n, tmpl, order, first, count, spacing, out);
 }
 
 // Scan an input series for NaN/Inf.

@@ -16,20 +16,40 @@ constexpr int kMinLog2 = 5;         // FFT pass lengths 32 .. 4096 (pass B rows)
 constexpr int kMaxLog2 = 12;
 constexpr int kMaxLog2A = 13;       // pass A columns up to 8192 (FP32 plans)
 
-// Per-sky constants, written by k_sky_setup / k_sky_finalize (device memory).
+// Per-sky results in device memory (k_sky_finalize): the antenna-pattern
+// integrals and the weights of eq. (Fstat), 2A/D, 2B/D, 4C/D
+// (2F = kB|Fa|^2 + kA|Fb|^2 - kC Re FaFb*).
 struct SkyConst {
-  double alpha, delta;
-  double cos_alpha, sin_alpha;
-  double nx, ny, nz;          // unit vector to the source
+  double A, B, C, D;
+  double kA, kB, kC;
+  float kAf, kBf, kCf;
+};
+
+// What the per-sky kernels take from the sky position alone, formed on the
+// host (kernel argument, by value).
+struct SkyPos {
   double t_b0;                // start of the SSB grid
   double j_ref;               // (t_ref - t_b0) / dt
-  // antenna patterns a = sum_i ca[X][i] h_i, b = sum_i cb[X][i] h_i with
-  // h = (1, cos 2H, sin 2H, cos H, sin H), H = alpha - (lon + ph0 + W_rot t)
+  // t_m,X = ox cos(orbit) + oy sin(orbit) + rx cos(rotation) + ry sin(rotation) + rz
+  double ox, oy;
+  double rx[kMaxDet], ry[kMaxDet], rz[kMaxDet];
+  // antenna patterns a = c0 + c1 cH^2 + c2 sH cH + c3 cH + c4 sH, likewise b, with
+  // cH, sH = cos, sin(H), H = (alpha - lon) - rotation; cos, sin(alpha - lon)
+  double cx[kMaxDet], sx[kMaxDet];
   double ca[kMaxDet][5];
   double cb[kMaxDet][5];
-  double A, B, C, D;
-  double kA, kB, kC;          // 2A/D, 2B/D, 4C/D  (2F = kB|Fa|^2 + kA|Fb|^2 - kC Re FaFb*)
-  float kAf, kBf, kCf;
+};
+
+struct TmplCoef;
+
+// Templates whose spindown coefficients a per-sky group needs: entries
+// [first, first + count) of order, into out at the same places.
+struct CoefJob {
+  const fstat_template* tmpl;
+  const int* order;
+  int first, count;
+  double spacing;  // TmplCoef's D
+  TmplCoef* out;
 };
 
 // Per-template spindown phase polynomial in x = j - J (J = rint(j_ref)):
@@ -107,6 +127,14 @@ int device_sm_count();
 struct alignas(32) TimeTab {
   double co, so, cq, sq;
 };
+// Between two entries: c0 + c1 f + c2 f^2 + c3 f^3 at the fraction f of the
+// way, the cubic through the four nearest entries.
+struct alignas(32) Cubic {
+  double c0, c1, c2, c3;
+};
+struct RotCell {
+  Cubic c, s;  // cos, sin of the rotation angle
+};
 
 // Per-sky timing at one node (see Geo::nodes).
 struct alignas(32) SkyNode {
@@ -116,25 +144,38 @@ struct alignas(32) SkyNode {
 };
 // The same nodes for the FP32 (mixed-precision) path: v = vi + vf with
 // vi = rint(v) exact and |vf| <= 1/2 in FP32, dv = v(next node) - v (small:
-// the delay's change over kNodeStep samples), a, b in FP32; and the step-iii
+// the delay's change over a node step), a, b in FP32; and the step-iii
 // phase f_h t_m at the detector-time node as its fraction phf (|phf| <= 1/2)
-// and its change to the next node dph (below a cycle), both formed in FP64.
+// and its change to the next node dph (about a cycle at most), both formed in
+// FP64.
+// inner: every sample of the step that starts at this node is certainly valid
+// (k0 inside the data), from the delays of the cubic's four nodes with room for
+// its overshoot.
 struct alignas(32) NodeF32 {
   float a, b, vf, dv;
-  int vi;
+  int vi, inner;
   float phf, dph;
-  int pad_;
 };
-constexpr int kNodeStep = 16;  // samples between timing nodes
-inline int sky_nodes(int64_t n) { return (int)((n + kNodeStep - 1) / kNodeStep) + 3; }
+// Samples between timing nodes, 4 .. 64 (a resampling block holds whole steps):
+// the most for which a step lasts at most 32 s of the Earth's rotation, over
+// which the cubics below are exact to ~1e-14 s and ~5e-12 in a, b.
+inline int node_step_log2(double dt, double w_rot) {
+  int l = 2;
+  while (l < 6 && (2 << l) * dt <= 32.0 && fabs(w_rot) * (2 << l) * dt <= 2.4e-3) ++l;
+  return l;
+}
+inline int sky_nodes(int64_t n, int step_log2) { return (int)((n + (1 << step_log2) - 1) >> step_log2) + 3; }
 
 // Geometry constants for one plan (kernel argument, by value).
 struct Geo {
   double c, au, r_earth, w_rot, w_orb, cos_obl, sin_obl, orb_ph0, sid_ph0;
   double lat[kMaxDet], lon[kMaxDet], gam[kMaxDet];
+  double s2g[kMaxDet], c2g[kMaxDet], sl[kMaxDet], cl[kMaxDet], s2l[kMaxDet], c2l[kMaxDet];  // of 2 gam, lat, 2 lat
   double rcl[kMaxDet], rsl[kMaxDet];   // r_earth cos(lat), r_earth sin(lat)
   double w[kMaxDet];                   // noise weights of the rescaled series, sigma_ref^2 / (2 sigma_X^2)
-  double inv_sigma_ref;                // z is stored divided by sigma_ref (smallest sigma_X)
+  double inv_sigma_ref;                // z is formed divided by sigma_ref (smallest sigma_X)
+  float isf, wf[kMaxDet];              // inv_sigma_ref and w in FP32
+  float tap_c2;                        // (pi / N)^2 / 6, series form of the tap weights (sky.cu)
   double t0, dt, f_het, t_ref;
   int64_t n;                           // samples per detector
   int n_det, dterms;
@@ -143,17 +184,18 @@ struct Geo {
   // Sky-independent timing table (sky.cu): cos, sin of the orbital phase and
   // of the sidereal rotation angle at t = tab_t0 + i / tab_inv_h.
   const TimeTab* tab;
-  double tab_t0, tab_inv_h;
+  const RotCell* rot;                  // cubics of the rotation's cos, sin, same grid
+  double tab_t0, tab_inv_h, inv_dt;
   int tab_n;
-  // Roemer delay t_m of the current sky position for each detector on the
-  // same grid, [X * tab_n + i] (rewritten by every per-sky run)
-  double* tm_tab;
-  // Per-sky timing nodes every kNodeStep samples (sky.cu), [X * n_nodes + m]
-  // for sample j = (m - 1) kNodeStep: t_m at the detector time, and at the
+  // Roemer delay t_m of the current sky position for each detector as cubics on
+  // the same grid, [X * tab_n + i] (rewritten by every per-sky run)
+  Cubic* tm_tab;
+  // Per-sky timing nodes every 2^node_log2 samples (sky.cu), [X * n_nodes + m]
+  // for sample j = (m - 1) 2^node_log2: t_m at the detector time, and at the
   // SSB epoch the delay correction v = u - j and the antenna patterns a, b
   SkyNode* nodes;
   NodeF32* nodes32;                    // the same nodes in FP32 (mixed path)
-  int n_nodes;
+  int n_nodes, node_log2;
 };
 
 // ---------------------------------------------------- pair of complex values
@@ -212,6 +254,8 @@ __device__ __forceinline__ Pair<double> pload_g(const PairMem<double>::type* __r
   double2 a = __ldg(&p->a), b = __ldg(&p->b); return {a.x, a.y, b.x, b.y};
 }
 
+__device__ __forceinline__ float sinpi_t(float x) { return sinpif(x); }
+__device__ __forceinline__ double sinpi_t(double x) { return sinpi(x); }
 __device__ __forceinline__ void sincospi_t(float x, float* s, float* c) { sincospif(x, s, c); }
 __device__ __forceinline__ void sincospi_t(double x, double* s, double* c) { sincospi(x, s, c); }
 
@@ -230,16 +274,18 @@ inline GCol g_columns(int64_t n, int64_t n1, int rl) {
 }
 
 // ------------------------------------------------------------ host helpers
-void launch_sky(const Geo& g, int precision, double alpha, double delta, const void* const* xh,
-                const int* xh_dtype, void* z, void* G, int n1, GCol gc, double* partials,
-                int n_blocks, SkyConst* sky, int* err, cudaStream_t st);
+SkyPos sky_position(const Geo& g, double alpha, double delta);
+// Blocks of the resampling kernel for n samples (its A, B, C partial sums).
+int sky_blocks(int64_t n);
+// Steps (iii)-(v) for one sky position, and the spindown coefficients of job's
+// templates (count 0: none).  Four launches.
+void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* const* xh, const int* xh_dtype, void* G,
+                int n1, GCol gc, double* partials, SkyConst* sky, int* err, const CoefJob& job, cudaStream_t st);
 // Timing table: entries needed to cover [t_lo, t_hi] at spacing h, and the
 // kernel that fills them (FP64 sincos, once per plan).
 int time_table_entries(double t_lo, double t_hi, double h);
-cudaError_t launch_time_table(const Geo& g, TimeTab* tab, cudaStream_t st);
-void launch_tmpl_coef(const SkyConst* sky, double dt, int64_t n, const fstat_template* tmpl,
-                      const int* order, int first, int count, double spacing, bool f64, TmplCoef* out,
-                      cudaStream_t st);
+cudaError_t launch_time_table(const Geo& g, TimeTab* tab, RotCell* rot, cudaStream_t st);
+void launch_tmpl_coef(const SkyPos& pos, const Geo& g, int precision, const CoefJob& job, cudaStream_t st);
 // samples between the inputs of one of pass A's first butterflies
 int64_t pass_a_spacing(int log2n, int log2_n2);
 void launch_check_finite(const void* x, int dtype, int64_t n, int* err, cudaStream_t st);

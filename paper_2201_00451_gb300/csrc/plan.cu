@@ -51,7 +51,6 @@ struct fstat_plan {
   bool have[kMaxDet] = {};
   double sigma[kMaxDet] = {};
   double sigma_ref = 1.0;        // common rescaling of the series (see sky.cu)
-  void* z = nullptr;
   void* G = nullptr;
   void* Z = nullptr;
   // templates rotate over nstream streams (the caller's + plan-owned side
@@ -64,9 +63,8 @@ struct fstat_plan {
   cudaEvent_t fork = nullptr;
   cudaEvent_t join[kMaxStreams] = {};
   double* partials = nullptr;
-  int nblk = 0;
-  TimeTab* tab = nullptr;        // timing table (geo.tab)
-  double* tm_tab = nullptr;      // per-sky Roemer delay table (geo.tm_tab)
+  TimeTab* tab = nullptr;        // timing table and rotation cubics (geo.tab, geo.rot)
+  Cubic* tm_tab = nullptr;       // per-sky Roemer delay cubics (geo.tm_tab)
   SkyNode* nodes = nullptr;      // per-sky timing nodes (geo.nodes)
   NodeF32* nodes32 = nullptr;  // the same nodes in FP32 (geo.nodes32)
   SkyConst* sky = nullptr;
@@ -90,6 +88,7 @@ struct fstat_plan {
   bool staged_pending = false;
   bool sky_valid = false;
   double sky_alpha = 0, sky_delta = 0;
+  SkyPos pos{};                  // of that sky position
   // refinement: sample tables (built lazily), candidate staging, scratch
   void* gtab = nullptr;
   bool gtab_valid = false;
@@ -160,7 +159,6 @@ int ilog2_exact(int64_t v) {
 
 void free_all(fstat_plan* p) {
   for (int X = 0; X < kMaxDet; ++X) if (p->xh[X]) cudaFree(p->xh[X]);
-  if (p->z) cudaFree(p->z);
   if (p->G) cudaFree(p->G);
   if (p->Z) cudaFree(p->Z);
   for (int k = 1; k < fstat_plan::kMaxStreams; ++k) {
@@ -227,19 +225,34 @@ EventPair get_events(fstat_plan* p) {
   return e;
 }
 
-int run_sky(fstat_plan* p, double alpha, double delta, cudaStream_t st) {
+double spin_spacing(const fstat_plan* p) { return (double)pass_a_spacing(p->log2n, p->log2n2); }
+
+// Per-sky work and the spindown coefficients of sorted templates
+// [first, first + count) (none for count 0).
+int run_sky(fstat_plan* p, double alpha, double delta, const CoefJob& job, cudaStream_t st) {
   EventPair e{};
   if (p->prof) { e = get_events(p); cudaEventRecord(e.a, st); }
   const void* xh[kMaxDet];
   for (int X = 0; X < kMaxDet; ++X) xh[X] = p->xh[X];
-  launch_sky(p->geo, p->d.precision, alpha, delta, xh, p->dtype, p->z, p->G, (int)p->n1, p->gc,
-             p->partials, p->nblk, p->sky, p->d_err, st);
+  p->pos = sky_position(p->geo, alpha, delta);
+  launch_sky(p->geo, p->d.precision, p->pos, xh, p->dtype, p->G, (int)p->n1, p->gc, p->partials, p->sky, p->d_err, job,
+             st);
   CK(cudaGetLastError());
-  p->n_launches += 4 + p->d.n_det;  // setup, delay table, step iii per detector, resampling, finalize
+  p->n_launches += 4;  // delay table, nodes, resampling, final sums and coefficients
   if (p->prof) { cudaEventRecord(e.b, st); p->ev[2].push_back(e); p->launches[2]++; }
   p->sky_valid = true;
   p->sky_alpha = alpha;
   p->sky_delta = delta;
+  return FSTAT_OK;
+}
+
+// The same where the plan may hold this sky position's series already.
+int run_group(fstat_plan* p, const fstat_template& t, bool force, const CoefJob& job, cudaStream_t st) {
+  if (force || !(p->sky_valid && p->sky_alpha == t.alpha && p->sky_delta == t.delta))
+    return run_sky(p, t.alpha, t.delta, job, st);
+  launch_tmpl_coef(p->pos, p->geo, p->d.precision, job, st);
+  ++p->n_launches;
+  CK(cudaGetLastError());
   return FSTAT_OK;
 }
 
@@ -297,8 +310,6 @@ cudaError_t launch_b(fstat_plan* p, int cb, int vb, float* out, cudaStream_t st,
   }
   return launch_pass_b_f64(p->log2n1, cb, vb, Z, (int)p->n2, p->tt.b, p->sky, out, st, pk, res);
 }
-
-double spin_spacing(const fstat_plan* p) { return (double)pass_a_spacing(p->log2n, p->log2n2); }
 
 cudaError_t launch_b_acc(fstat_plan* p, float* out, int shift, bool first, cudaStream_t st, void* Z) {
   ++p->n_launches;
@@ -367,6 +378,12 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
     g.lat[X] = d.det[X].lat_rad;
     g.lon[X] = d.det[X].lon_rad;
     g.gam[X] = d.det[X].gamma_rad;
+    g.s2g[X] = std::sin(2.0 * g.gam[X]);
+    g.c2g[X] = std::cos(2.0 * g.gam[X]);
+    g.sl[X] = std::sin(g.lat[X]);
+    g.cl[X] = std::cos(g.lat[X]);
+    g.s2l[X] = std::sin(2.0 * g.lat[X]);
+    g.c2l[X] = std::cos(2.0 * g.lat[X]);
     g.rcl[X] = d.ephem.r_earth * std::cos(d.det[X].lat_rad);
     g.rsl[X] = d.ephem.r_earth * std::sin(d.det[X].lat_rad);
     g.clon[X] = std::cos(d.det[X].lon_rad);
@@ -378,15 +395,13 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   g.f_het = d.f_het;
   g.t_ref = std::isnan(d.t_ref) ? d.t0 + (double)(d.n_samples / 2) * d.dt : d.t_ref;
   g.n = d.n_samples;
+  g.tap_c2 = (float)(9.8696044010893586 / 6.0 / ((double)g.n * (double)g.n));
   g.n_det = d.n_det;
   g.dterms = d.dterms;
   g.interp = d.interp;
 
   const int64_t N = d.n_samples;
-  const size_t zb = d.precision == FSTAT_FP64 ? 16 : 8;
-  p->nblk = (int)((N + kSkyBlock - 1) / kSkyBlock);
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = palloc(p, &p->z, (size_t)d.n_det * N * zb);
   // whole columns of whole residues: up to N1 RL <= 2^12 x 16 pairs of padding
   if (e == cudaSuccess)
     e = palloc(p, &p->G, (size_t)(N + (int64_t(1) << (kMaxLog2 + (d.precision == FSTAT_FP64 ? 0 : 4)))) * p->pair_bytes);
@@ -405,28 +420,33 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   // timing table over every epoch the timing can reach: the data span
   // widened by the largest delay (|t_m| <= (au + r_earth)/c) plus margin
   {
-    // (and the timing nodes, which extend kNodeStep samples before the data
+    // (and the timing nodes, which extend one node step before the data
     // and up to three node steps past it)
+    g.node_log2 = node_step_log2(d.dt, d.ephem.omega_rot);
+    const double step = (double)(1 << g.node_log2);
     const double reach = (d.ephem.au + d.ephem.r_earth) / d.ephem.c + 100.0;
-    const double lo = d.t0 - 2.0 * reach - 2.0 * kTabStep - 2.0 * kNodeStep * d.dt;
-    const double hi = d.t0 + (double)N * d.dt + 2.0 * reach + 2.0 * kTabStep + 4.0 * kNodeStep * d.dt;
+    const double lo = d.t0 - 2.0 * reach - 2.0 * kTabStep - 2.0 * step * d.dt;
+    const double hi = d.t0 + (double)N * d.dt + 2.0 * reach + 2.0 * kTabStep + 4.0 * step * d.dt;
     g.tab_n = time_table_entries(lo, hi, kTabStep);
     g.tab_t0 = lo;
     g.tab_inv_h = 1.0 / kTabStep;
     TimeTab* tab = nullptr;
-    if (e == cudaSuccess) e = palloc(p, &tab, (size_t)g.tab_n * sizeof(TimeTab));
+    if (e == cudaSuccess) e = palloc(p, &tab, (size_t)g.tab_n * (sizeof(TimeTab) + sizeof(RotCell)));
+    RotCell* rot = reinterpret_cast<RotCell*>(tab + g.tab_n);
     p->tab = tab;
     g.tab = tab;
-    if (e == cudaSuccess) e = palloc(p, &p->tm_tab, (size_t)g.tab_n * kMaxDet * sizeof(double));
+    g.rot = rot;
+    g.inv_dt = 1.0 / d.dt;
+    if (e == cudaSuccess) e = palloc(p, &p->tm_tab, (size_t)g.tab_n * d.n_det * sizeof(Cubic));
     g.tm_tab = p->tm_tab;
-    g.n_nodes = sky_nodes(N);
+    g.n_nodes = sky_nodes(N, g.node_log2);
     if (e == cudaSuccess) e = palloc(p, &p->nodes, (size_t)g.n_nodes * d.n_det * sizeof(SkyNode));
     if (e == cudaSuccess) e = palloc(p, &p->nodes32, (size_t)g.n_nodes * d.n_det * sizeof(NodeF32));
     g.nodes = p->nodes;
     g.nodes32 = p->nodes32;
-    if (e == cudaSuccess) e = launch_time_table(g, tab, 0);
+    if (e == cudaSuccess) e = launch_time_table(g, tab, rot, 0);
   }
-  if (e == cudaSuccess) e = palloc(p, &p->partials, (size_t)3 * p->nblk * sizeof(double));
+  if (e == cudaSuccess) e = palloc(p, &p->partials, (size_t)3 * sky_blocks(N) * sizeof(double));
   if (e == cudaSuccess) e = palloc(p, &p->sky, sizeof(SkyConst));
   if (e == cudaSuccess && d.precision == FSTAT_FP64) e = palloc(p, &p->tw, (size_t)6 * (size_t(1) << kMaxLog2) * 16);
   if (e == cudaSuccess) e = palloc(p, &p->d_err, 2 * sizeof(int));
@@ -494,8 +514,12 @@ int finish_series(fstat_plan* p, int det, double sigma, cudaStream_t st) {
     if (p->have[X] && (ref == 0.0 || p->sigma[X] < ref)) ref = p->sigma[X];
   p->sigma_ref = ref;
   p->geo.inv_sigma_ref = 1.0 / ref;
+  p->geo.isf = (float)p->geo.inv_sigma_ref;
   for (int X = 0; X < p->d.n_det; ++X)
+    {
     p->geo.w[X] = p->have[X] ? ref * ref / (2.0 * p->sigma[X] * p->sigma[X]) : 0.0;
+    p->geo.wf[X] = (float)p->geo.w[X];
+  }
   return FSTAT_OK;
 }
 
@@ -650,16 +674,10 @@ int enqueue_compute(fstat_plan* p, const fstat_template* h_tmpl, const int* h_or
     const fstat_template& t0 = h_tmpl[h_ord[i]];
     int64_t j = i + 1;
     while (j < n && h_tmpl[h_ord[j]].alpha == t0.alpha && h_tmpl[h_ord[j]].delta == t0.delta) ++j;
-    if (force_sky || !(p->sky_valid && p->sky_alpha == t0.alpha && p->sky_delta == t0.delta)) {
-      int rc = run_sky(p, t0.alpha, t0.delta, st);
-      if (rc) return rc;
-    }
-    launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, d_tmpl, d_ord, (int)i, (int)(j - i), spin_spacing(p),
-                     p->d.precision == FSTAT_FP64, d_coef, st);
-    ++p->n_launches;
-    CK(cudaGetLastError());
+    int rc = run_group(p, t0, force_sky, CoefJob{d_tmpl, d_ord, (int)i, (int)(j - i), spin_spacing(p), d_coef}, st);
+    if (rc) return rc;
     if (!po && p->fused && fused_ok(p)) {
-      int rc = enqueue_fused(p, i, j, d_ord, d_coef, twoF, out_rows, st, prof);
+      rc = enqueue_fused(p, i, j, d_ord, d_coef, twoF, out_rows, st, prof);
       if (rc) return rc;
       i = j;
       continue;
@@ -829,14 +847,9 @@ int fstat_semicoherent(fstat_plan* const* seg, int n_seg, const fstat_template* 
     while (j < n && tmpl[ord[j]].alpha == t0.alpha && tmpl[ord[j]].delta == t0.delta) ++j;
     for (int s = 0; s < n_seg; ++s) {
       fstat_plan* p = seg[s];
-      if (!(p->sky_valid && p->sky_alpha == t0.alpha && p->sky_delta == t0.delta)) {
-        int rc = run_sky(p, t0.alpha, t0.delta, st);
-        if (rc) return rc;
-      }
-      launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, (int)i, (int)(j - i), spin_spacing(p),
-                       p->d.precision == FSTAT_FP64, p->d_coef, st);
-      ++p->n_launches;
-      CK(cudaGetLastError());
+      const int rc = run_group(p, t0, false,
+                               CoefJob{p->d_tmpl, p->d_order, (int)i, (int)(j - i), spin_spacing(p), p->d_coef}, st);
+      if (rc) return rc;
     }
     const int nq = (int)std::min<int64_t>(ns, j - i);
     if (nq > 1) {
@@ -1092,7 +1105,7 @@ int fstat_export_sky(fstat_plan* p, double alpha, double delta, double* ga, doub
   for (int X = 0; X < p->d.n_det; ++X)
     if (!p->have[X]) return FSTAT_ERR_NOT_READY;
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = run_sky(p, alpha, delta, st);
+  int rc = run_sky(p, alpha, delta, CoefJob{}, st);
   if (rc) return rc;
   const int64_t N = p->d.n_samples;
   std::vector<unsigned char> buf((size_t)(p->n1 * p->gc.lc) * p->pair_bytes);
@@ -1424,10 +1437,8 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
   for (int l1 = lo; l1 <= hi && rc == FSTAT_OK; ++l1) {
     rc = set_split(p, l1);
     if (rc) break;
-    rc = run_sky(p, 0.3, -0.5, st);
+    rc = run_sky(p, 0.3, -0.5, CoefJob{p->d_tmpl, p->d_order, 0, kPipe, spin_spacing(p), p->d_coef}, st);
     if (rc) break;
-    launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, 0, kPipe, spin_spacing(p),
-                     p->d.precision == FSTAT_FP64, p->d_coef, st);
     // isolated timings of every distinct shape of each pass: for FP32 plans
     // pass A with columns staged where that costs no occupancy (0) or never
     // (2), pass B with 1 to 8 rows per tile; FP64 has one of each
@@ -1477,12 +1488,8 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
     p->cb = best.cb;
     p->vb = best.vb;
     p->fused = best.fused != 0 && fused_ok(p);
-    rc = run_sky(p, 0.3, -0.5, st);
-    if (rc == FSTAT_OK) {
-      launch_tmpl_coef(p->sky, p->d.dt, p->d.n_samples, p->d_tmpl, p->d_order, 0, kPipe, spin_spacing(p),
-                     p->d.precision == FSTAT_FP64, p->d_coef, st);
-      tune_peaks(p, st, pipeline, &best.cbp, &best.vbp);
-    }
+    rc = run_sky(p, 0.3, -0.5, CoefJob{p->d_tmpl, p->d_order, 0, kPipe, spin_spacing(p), p->d_coef}, st);
+    if (rc == FSTAT_OK) tune_peaks(p, st, pipeline, &best.cbp, &best.vbp);
     p->cb_pk = best.cbp;
     p->vb_pk = best.vbp;
   }

@@ -51,3 +51,33 @@ def test_interpolator_variants_match_oracle(interp, dterms):
     want = resamp.fstat(t, x, tm)
     excess = np.abs(got - want) - (REL * np.abs(want) + ABS)
     assert excess.max() <= 0, excess.max()
+
+
+# FP64: the nodes' cubics are exact to ~1e-11 of a, b (32 s), f_h t_m to ~1e-10
+# radians; FP32 as above
+@pytest.mark.parametrize("precision,tol", [(pkg.MIXED, 2e-5), (pkg.FP64, 1e-9)])
+@pytest.mark.parametrize("dtype", ["c64", "c128", "both"])
+@pytest.mark.parametrize("n,dt,dterms", [
+    (17, 2.0, 2), (700, 4.0, 8), (1025, 1.0, 5), (4096, 0.5, 8), (40000, 1.0, 20), (600001, 0.5, 8)])
+def test_series_lengths_and_node_steps_match_oracle(n, dt, dterms, dtype, precision, tol):
+    # a node every 16, 32 and 64 samples; tap weights in the short- and the
+    # long-series form, unrolled (D = 8) or not; one and several tiles per
+    # block; whole steps of nodes and a cut one at the end
+    t = small_target(n_samples=n, dt=dt, n_fft=1 << max(10, (n - 1).bit_length()), n_det=2, seed=n, dtype="c128",
+                     dterms=dterms)
+    rng = np.random.default_rng(n)
+    x = [rng.standard_normal(n) + 1j * rng.standard_normal(n) for _ in range(2)]
+    for X in range(2):
+        if dtype == "c64" or (dtype == "both" and X == 0):
+            x[X] = x[X].astype(np.complex64)
+    a, d = t.skies[0]
+    ref = resamp.sky_prep(t, [v.astype(np.complex128) for v in x], a, d)
+    with pkg.FstatPlan.from_target(t, precision) as plan:
+        for X in range(2):
+            plan.set_data(X, x[X], t.sigmas[X])
+        ga, gb, abcd = plan.export_sky(a, d)
+    scale = max(np.abs(ref["Ga"]).max(), np.abs(ref["Gb"]).max())
+    assert np.abs(ga - ref["Ga"]).max() <= tol * scale
+    assert np.abs(gb - ref["Gb"]).max() <= tol * scale
+    for k, v in zip("ABCD", abcd):
+        assert abs(v - ref[k]) <= 1e-10 * abs(ref[k]) + 1e-12

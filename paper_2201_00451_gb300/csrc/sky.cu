@@ -221,7 +221,8 @@ k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
   if (m >= 1 && m + 2 < g.n_nodes) {
     const int lo = min(min(s_vi[t - 1], vi), min(s_vi[t + 1], s_vi[t + 2]));
     const int hi = max(max(s_vi[t - 1], vi), max(s_vi[t + 1], s_vi[t + 2]));
-    f.inner = hi - lo <= 4 && ji + lo >= 3 && ji + (step - 1) + hi <= (int)g.n - 4;
+    // (a whole step of SSB samples, and all of their positions in the data)
+    f.inner = hi - lo <= 4 && ji + step <= (int)g.n && ji + lo >= 3 && ji + (step - 1) + hi <= (int)g.n - 4;
   }
   g.nodes32[i] = f;
 }

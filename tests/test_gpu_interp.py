@@ -70,14 +70,15 @@ def test_series_lengths_and_node_steps_match_oracle(n, dt, dterms, dtype, precis
     for X in range(2):
         if dtype == "c64" or (dtype == "both" and X == 0):
             x[X] = x[X].astype(np.complex64)
-    a, d = t.skies[0]
-    ref = resamp.sky_prep(t, [v.astype(np.complex128) for v in x], a, d)
+    # (delays of both signs at both ends: which samples of the last, cut step count)
     with pkg.FstatPlan.from_target(t, precision) as plan:
         for X in range(2):
             plan.set_data(X, x[X], t.sigmas[X])
-        ga, gb, abcd = plan.export_sky(a, d)
-    scale = max(np.abs(ref["Ga"]).max(), np.abs(ref["Gb"]).max())
-    assert np.abs(ga - ref["Ga"]).max() <= tol * scale
-    assert np.abs(gb - ref["Gb"]).max() <= tol * scale
-    for k, v in zip("ABCD", abcd):
-        assert abs(v - ref[k]) <= 1e-10 * abs(ref[k]) + 1e-12
+        for a, d in (t.skies[0], (0.3, -0.6), (2.0, 0.4), (3.6, 0.2), (5.2, -0.1)):
+            ref = resamp.sky_prep(t, [v.astype(np.complex128) for v in x], a, d)
+            ga, gb, abcd = plan.export_sky(a, d)
+            scale = max(np.abs(ref["Ga"]).max(), np.abs(ref["Gb"]).max())
+            assert np.abs(ga - ref["Ga"]).max() <= tol * scale
+            assert np.abs(gb - ref["Gb"]).max() <= tol * scale
+            for k, v in zip("ABCD", abcd):
+                assert abs(v - ref[k]) <= 1e-10 * abs(ref[k]) + 1e-12

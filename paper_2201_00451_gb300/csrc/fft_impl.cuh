@@ -208,10 +208,16 @@ __device__ __forceinline__ int pad_idx(int pos, int ps) { return pos + (pos >> p
 
 template <typename TW> __device__ __forceinline__ TW tw_ld(const TW* p) { return __ldg(p); }
 
-// (cos, sin) of 2 pi x for x in turns, |x| <= 1/2: the hardware sine/cosine,
-// accurate to ~4e-7 absolute on [-pi, pi].
+// (cos, sin) of 2 pi x for x in turns, |x| <= 1/2: the hardware sine/cosine
+// (accurate to ~4e-7 absolute on [-pi, pi]) brought to unit length.  The
+// hardware's pair is short by ~7e-8 on average, which a transform's nine factors
+// per sample add up: 2F came out 1.3e-6 low throughout at 2^22 points.
 __device__ __forceinline__ void turn_sincos(float x, float* s, float* c) {
-  __sincosf(6.28318530717958647692f * x, s, c);
+  float sv, cv;
+  __sincosf(6.28318530717958647692f * x, &sv, &cv);
+  const float h = 0.5f * __fmaf_rn(-sv, sv, __fmaf_rn(-cv, cv, 1.f));
+  *s = __fmaf_rn(sv, h, sv);
+  *c = __fmaf_rn(cv, h, cv);
 }
 
 // ------------------------------------------------------------- small DFTs
@@ -242,26 +248,32 @@ template <typename T, int R> struct Twiddles {
       s[o + m] = fmadd(c[o], sm, s[o] * cm);
     }
   }
-  template <int M> __device__ __forceinline__ void level(float theta) {
-    turn_sincos(-theta * (float)(R / M), &s[tw_off(M)], &c[tw_off(M)]);
-    spread<M>();
-    if constexpr (M < R) level<2 * M>(theta);
-  }
-  // theta in [0, 1/R)
-  __device__ __forceinline__ explicit Twiddles(float theta) { level<2>(theta); }
   template <int M> __device__ __forceinline__ void square() {  // level M from level 2M
     const T x = c[tw_off(2 * M)], y = s[tw_off(2 * M)];
     c[tw_off(M)] = fmadd(x, x, -(y * y));
     s[tw_off(M)] = (x + x) * y;
     spread<M>();
-    if constexpr (M > 2) square<M / 2>();
   }
+  template <int M> __device__ __forceinline__ void squares() {
+    square<M>();
+    if constexpr (M > 2) squares<M / 2>();
+  }
+  // every other level by its angle, the one below it by squaring: the rounding
+  // of a factor doubles once only
+  template <int M> __device__ __forceinline__ void level(float theta) {
+    turn_sincos(-theta * (float)(R / M), &s[tw_off(M)], &c[tw_off(M)]);
+    spread<M>();
+    if constexpr (M > 2) square<M / 2>();
+    if constexpr (M > 4) level<M / 4>(theta);
+  }
+  // theta in [0, 1/R)
+  __device__ __forceinline__ explicit Twiddles(float theta) { level<R>(theta); }
   // from the angle's own factor exp(-2 pi i theta)
   __device__ __forceinline__ Twiddles(T cw, T sw) {
     c[tw_off(R)] = cw;
     s[tw_off(R)] = sw;
     spread<R>();
-    if constexpr (R > 2) square<R / 2>();
+    if constexpr (R > 2) squares<R / 2>();
   }
 };
 

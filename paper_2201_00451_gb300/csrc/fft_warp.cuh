@@ -138,10 +138,6 @@ template <int L, int CB, int SUBMAX> __device__ __forceinline__ int out_index(in
   return u + (e / S::RE) * S::GW + (e % S::RE) * (S::SUB / S::RE);
 }
 
-// Templates of one launch: their intermediates, and for pass B their output
-// rows (row ord[k] mod out_rows of `out`, or `out` itself without ord).
-struct ZList { float4* z[kMaxBatch]; };
-
 // ------------------------------------------------------------- pass A
 // G holds column n1's samples residue by residue: sample n2 = r + RL j at
 // [(n1 RL + r) lcs + j].  STAGED: the next column (RL lcs pairs) is copied by
@@ -153,7 +149,7 @@ template <int L> using WA = WShape<L, 1, kSubA>;
 template <int L, bool STAGED>
 __global__ void __launch_bounds__(WA<L>::NT, WA<L>::MINB)
 k_wpass_a(const float4* __restrict__ G, int lcs, int n, int n1, const TmplCoef* __restrict__ coef,
-          const __grid_constant__ ZList zl, ZLayout zy, int n_tmpl, int* __restrict__ err, int wait_limit) {
+          float4* __restrict__ z0, ZLayout zy, int n_tmpl, int* __restrict__ err, int wait_limit) {
   using S = WA<L>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float4* smem = reinterpret_cast<float4*>(smem_raw);
@@ -236,7 +232,7 @@ k_wpass_a(const float4* __restrict__ G, int lcs, int n, int n1, const TmplCoef* 
         },
         [] {});
     const int zp = (col & ((1 << zy.rl) - 1)) * zy.sub + (col >> zy.rl);  // [r][j]
-    float4* z = zl.z[k];
+    float4* z = z0 + (int64_t)k * L * n1;
     auto zat = [&](int k2) {
       return (((int64_t)(k2 >> zy.cb) * n1 + zp) << zy.cb) + (k2 & ((1 << zy.cb) - 1));
     };
@@ -289,7 +285,7 @@ template <int L, int CB, int MODE> struct WSmemB {
 template <int L, int CB, int MODE>
 __global__ void __launch_bounds__(WB<L, CB>::NT, WB<L, CB>::MINB)
 k_wpass_b(int n2, const SkyConst* __restrict__ sky, float* __restrict__ out, const int* __restrict__ ord,
-          int64_t out_rows, int n_tmpl, int n_bands, const PeakArgs pk0, const __grid_constant__ ZList zl) {
+          int64_t out_rows, int n_tmpl, int n_bands, const PeakArgs pk0, const float4* __restrict__ z0) {
   using S = WB<L, CB>;
   using M = WSmemB<L, CB, MODE>;
   static_assert(S::COLS == 1, "pass B tiles fill at least a warp");
@@ -317,9 +313,8 @@ k_wpass_b(int n2, const SkyConst* __restrict__ sky, float* __restrict__ out, con
       const int it = issued / M::NQ, q = issued % M::NQ, slot = issued % M::NSLOT;
       const int64_t tile = blockIdx.x + (int64_t)it * gridDim.x;
       if (tile >= n_tiles) break;
-      const int k = (int)tile / tpt;
       mbar_expect_tx(&bar[slot], (unsigned)M::PART);
-      bulk_load(smem_raw + slot * M::PART, zl.z[k] + (int64_t)((int)tile - k * tpt) * (L * CB) + q * PP,
+      bulk_load(smem_raw + slot * M::PART, z0 + tile * (L * CB) + q * PP,
                 (unsigned)M::PART, &bar[slot]);
     }
   };
@@ -461,7 +456,7 @@ k_wpass_b(int n2, const SkyConst* __restrict__ sky, float* __restrict__ out, con
 // Pass A.  staging: 0 = where the staged columns leave room for as many CTAs
 // as registers allow, 1 = required, 2 = none.
 template <int L>
-cudaError_t run_wa(const float4* G, int lcs, int64_t n, int n1, const TmplCoef* coef, const ZList& z, ZLayout zy, int n_tmpl,
+cudaError_t run_wa(const float4* G, int lcs, int64_t n, int n1, const TmplCoef* coef, float4* z, ZLayout zy, int n_tmpl,
                    int staging, int* err, int wait_limit, cudaStream_t st, int res) {
   using S = WA<L>;
   if (n1 % S::COLS) return cudaErrorInvalidConfiguration;
@@ -497,7 +492,7 @@ template <int L, int CB> constexpr bool wb_ok() {
 }
 
 template <int L, int CB, int MODE>
-cudaError_t run_wb(const ZList& z, int n2, const WBArgs& a, cudaStream_t st, int res) {
+cudaError_t run_wb(float4* z, int n2, const WBArgs& a, cudaStream_t st, int res) {
   using S = WB<L, CB>;
   if constexpr (!wb_ok<L, CB>()) {
     return cudaErrorInvalidConfiguration;
@@ -527,7 +522,7 @@ template <int L> constexpr int wb_rows(int cb) {
 }
 
 template <int L, int MODE>
-cudaError_t pick_wb(int cb, const ZList& z, int n2, const WBArgs& a, cudaStream_t st, int res) {
+cudaError_t pick_wb(int cb, float4* z, int n2, const WBArgs& a, cudaStream_t st, int res) {
   switch (wb_rows<L>(cb)) {
     case 1: return run_wb<L, 1, MODE>(z, n2, a, st, res);
     case 2: return run_wb<L, 2, MODE>(z, n2, a, st, res);
@@ -537,7 +532,7 @@ cudaError_t pick_wb(int cb, const ZList& z, int n2, const WBArgs& a, cudaStream_
   }
 }
 template <int MODE>
-cudaError_t dispatch_wb(int log2_n1, int cb, const ZList& z, int n2, const WBArgs& a, cudaStream_t st, int res) {
+cudaError_t dispatch_wb(int log2_n1, int cb, float4* z, int n2, const WBArgs& a, cudaStream_t st, int res) {
   switch (log2_n1) {
     case 5: return pick_wb<32, MODE>(cb, z, n2, a, st, res);
     case 6: return pick_wb<64, MODE>(cb, z, n2, a, st, res);

@@ -4,10 +4,8 @@
 namespace fstat {
 
 cudaError_t launch_wpass_a(int log2_n2, int staging, const void* G, GCol gc, int64_t n, int n1, const TmplCoef* coef,
-                           void* const* Z, ZLayout zy, int n_tmpl, int* err, int wait_limit, cudaStream_t st, int res) {
-  fft::ZList z{};
-  if (n_tmpl < 1 || n_tmpl > kMaxBatch) return cudaErrorInvalidValue;
-  for (int k = 0; k < n_tmpl; ++k) z.z[k] = (float4*)Z[k];
+                           void* Z, ZLayout zy, int n_tmpl, int* err, int wait_limit, cudaStream_t st, int res) {
+  float4* z = (float4*)Z;
   const float4* g = (const float4*)G;
   switch (log2_n2) {
 #define FSTAT_WA(B) \

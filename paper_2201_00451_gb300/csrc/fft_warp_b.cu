@@ -4,14 +4,6 @@
 namespace fstat {
 
 namespace {
-bool zlist(fft::ZList* z, void* const* Z, int n_tmpl) {
-  if (n_tmpl < 1 || n_tmpl > kMaxBatch) return false;
-  for (int k = 0; k < n_tmpl; ++k) z->z[k] = (float4*)Z[k];
-  return true;
-}
-}  // namespace
-
-namespace {
 template <int L, int CB> ZLayout layout_of() {
   using S = fft::WB<L, CB>;
   return ZLayout{fft::log2c(CB), fft::log2c(S::RL), S::SUB};
@@ -41,26 +33,22 @@ ZLayout wpass_z_layout(int log2_n1, int cb) {
 }
 int wpass_b_rows(int log2_n1, int cb) { return 1 << wpass_z_layout(log2_n1, cb).cb; }
 
-cudaError_t launch_wpass_b(int log2_n1, int cb, void* const* Z, int n_tmpl, int n2, const SkyConst* sky, float* out,
+cudaError_t launch_wpass_b(int log2_n1, int cb, void* Z, int n_tmpl, int n2, const SkyConst* sky, float* out,
                            const int* ord, int64_t out_rows, int* err, int wait_limit, cudaStream_t st, int res) {
-  fft::ZList z{};
-  if (!zlist(&z, Z, n_tmpl)) return cudaErrorInvalidValue;
   fft::WBArgs a{sky, out, ord, out_rows, n_tmpl, 0, PeakArgs{}};
   a.pk.err = err;
   set_wait(a.pk, wait_limit);
-  return fft::dispatch_wb<fft::kStore>(log2_n1, cb, z, n2, a, st, res);
+  return fft::dispatch_wb<fft::kStore>(log2_n1, cb, (float4*)Z, n2, a, st, res);
 }
 
 cudaError_t launch_wpass_b_acc(int log2_n1, int cb, void* Z, int n2, const SkyConst* sky, float* out, int shift,
                                bool first, int* err, int wait_limit, cudaStream_t st, int res) {
-  fft::ZList z{};
-  zlist(&z, &Z, 1);
   fft::WBArgs a{sky, out, nullptr, 1, 1, 0, PeakArgs{}};
   a.pk.err = err;
   a.pk.shift = shift;
   a.pk.first = first;
   set_wait(a.pk, wait_limit);
-  return fft::dispatch_wb<fft::kAccumulate>(log2_n1, cb, z, n2, a, st, res);
+  return fft::dispatch_wb<fft::kAccumulate>(log2_n1, cb, (float4*)Z, n2, a, st, res);
 }
 
 }  // namespace fstat

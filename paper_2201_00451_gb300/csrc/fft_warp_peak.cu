@@ -6,16 +6,13 @@ namespace fstat {
 // pk: the call's request; template k of the launch is the call's template
 // ord[k] (added to pk.tmpl, its band keys at pk.band_key + ord[k] n_bands),
 // or the only one without ord.
-cudaError_t launch_wpass_b_peak(int log2_n1, int cb, void* const* Z, int n_tmpl, int n2, const SkyConst* sky,
+cudaError_t launch_wpass_b_peak(int log2_n1, int cb, void* Z, int n_tmpl, int n2, const SkyConst* sky,
                                 const int* ord, int n_bands, const PeakArgs& pk, int* err, int wait_limit,
                                 cudaStream_t st, int res) {
-  fft::ZList z{};
-  if (n_tmpl < 1 || n_tmpl > kMaxBatch) return cudaErrorInvalidValue;
-  for (int k = 0; k < n_tmpl; ++k) z.z[k] = (float4*)Z[k];
   fft::WBArgs a{sky, nullptr, ord, 1, n_tmpl, n_bands, pk};
   if (!a.pk.err) a.pk.err = err;
   set_wait(a.pk, wait_limit);
-  return fft::dispatch_wb<fft::kPeaks>(log2_n1, cb, z, n2, a, st, res);
+  return fft::dispatch_wb<fft::kPeaks>(log2_n1, cb, (float4*)Z, n2, a, st, res);
 }
 
 }  // namespace fstat

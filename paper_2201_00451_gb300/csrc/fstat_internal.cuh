@@ -148,9 +148,9 @@ struct alignas(32) SkyNode {
 // phase f_h t_m at the detector-time node as its fraction phf (|phf| <= 1/2)
 // and its change to the next node dph (about a cycle at most), both formed in
 // FP64.
-// inner: every sample of the step that starts at this node is certainly valid
-// (k0 inside the data), from the delays of the cubic's four nodes with room for
-// its overshoot.
+// inner: the step that starts at this node is a whole one and every sample of it
+// certainly valid (k0 inside the data), from the delays of the cubic's four
+// nodes with room for its overshoot.
 struct alignas(32) NodeF32 {
   float a, b, vf, dv;
   int vi, inner;
@@ -355,12 +355,11 @@ inline void set_wait(PeakArgs& a, int wait_limit) {
   a.wait_limit = wait_limit >= 0 ? wait_limit : 0;
 }
 // The warp-local FP32 passes (fft_warp.cuh).  Z: the intermediates of the
-// launch's n_tmpl <= kMaxBatch templates, whose coefficients are coef[0..];
+// launch's n_tmpl templates, one behind the other; coef[0..]: their coefficients;
 // pass B writes template k to row ord[k] mod out_rows of out (ord == nullptr:
 // one template, to out).  staging: pass A's columns staged in shared memory
 // where that costs no occupancy (0), always (1; an error where they do not
 // fit) or never (2).
-constexpr int kMaxBatch = 8;
 // whether (ca, va) / (cb, vb) names a shape of the length
 bool pass_a_shape(int log2_n2, int ca, int va);
 bool pass_b_shape(int log2_n1, int cb, int vb);
@@ -370,13 +369,13 @@ struct ZLayout { int cb, rl, sub; };
 ZLayout wpass_z_layout(int log2_n1, int cb);  // cb: rows per tile asked of pass B (0 = default)
 int wpass_b_rows(int log2_n1, int cb);        // and what it runs with
 cudaError_t launch_wpass_a(int log2_n2, int staging, const void* G, GCol gc, int64_t n, int n1, const TmplCoef* coef,
-                           void* const* Z, ZLayout zy, int n_tmpl, int* err, int wait_limit, cudaStream_t st, int res);
+                           void* Z, ZLayout zy, int n_tmpl, int* err, int wait_limit, cudaStream_t st, int res);
 int wpass_a_residues_log2(int log2_n2);  // GCol::rl for pass A of this length
-cudaError_t launch_wpass_b(int log2_n1, int cb, void* const* Z, int n_tmpl, int n2, const SkyConst* sky, float* out,
+cudaError_t launch_wpass_b(int log2_n1, int cb, void* Z, int n_tmpl, int n2, const SkyConst* sky, float* out,
                            const int* ord, int64_t out_rows, int* err, int wait_limit, cudaStream_t st, int res);
 cudaError_t launch_wpass_b_acc(int log2_n1, int cb, void* Z, int n2, const SkyConst* sky, float* out, int shift,
                                bool first, int* err, int wait_limit, cudaStream_t st, int res);
-cudaError_t launch_wpass_b_peak(int log2_n1, int cb, void* const* Z, int n_tmpl, int n2, const SkyConst* sky,
+cudaError_t launch_wpass_b_peak(int log2_n1, int cb, void* Z, int n_tmpl, int n2, const SkyConst* sky,
                                 const int* ord, int n_bands, const PeakArgs& pk, int* err, int wait_limit,
                                 cudaStream_t st, int res);
 

@@ -129,10 +129,10 @@ extern "C" int fstat_twoF_noalloc(const void* g_pairs, int64_t n_samples, int64_
       NoallocArgs{A, B, C, tau0, dt, f1dot, f2dot, (double)pass_a_spacing(log2n, log2n2)});
   if (cudaGetLastError() != cudaSuccess) return FSTAT_ERR_CUDA;
   void* Z = p.Z;
-  cudaError_t e = launch_wpass_a(log2n2, 0, p.G, gc, n_samples, n1, p.coef, &Z, wpass_z_layout(log2n1, 0), 1, nullptr, -1,
+  cudaError_t e = launch_wpass_a(log2n2, 0, p.G, gc, n_samples, n1, p.coef, Z, wpass_z_layout(log2n1, 0), 1, nullptr, -1,
                                  st, 0);
   if (e != cudaSuccess) return FSTAT_ERR_CUDA;
-  e = launch_wpass_b(log2n1, 0, &Z, 1, n2, p.sky, twoF, nullptr, 1, nullptr, -1, st, 0);
+  e = launch_wpass_b(log2n1, 0, Z, 1, n2, p.sky, twoF, nullptr, 1, nullptr, -1, st, 0);
   if (e != cudaSuccess) return FSTAT_ERR_CUDA;
   return FSTAT_OK;
 }

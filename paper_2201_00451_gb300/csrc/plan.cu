@@ -58,7 +58,11 @@ struct fstat_plan {
   // templates overlap
   static constexpr int kMaxStreams = 8;
   int nstream = 2;
-  void* Zs[kMaxStreams] = {};      // Zs[0] aliases Z
+  // FP32 plans: templates share launches, over up to n_z intermediates one
+  // behind the other from Z on (see template_batch); 1: as many as streams
+  int n_z = 1;
+  bool batched = false;
+  void* Zs[kMaxStreams] = {};      // Zs[0] aliases Z, Zs[k < n_z] lie in its block
   cudaStream_t side[kMaxStreams] = {};
   cudaEvent_t fork = nullptr;
   cudaEvent_t join[kMaxStreams] = {};
@@ -162,7 +166,7 @@ void free_all(fstat_plan* p) {
   if (p->G) cudaFree(p->G);
   if (p->Z) cudaFree(p->Z);
   for (int k = 1; k < fstat_plan::kMaxStreams; ++k) {
-    if (p->Zs[k]) cudaFree(p->Zs[k]);
+    if (p->Zs[k] && k >= p->n_z) cudaFree(p->Zs[k]);
     if (p->side[k]) cudaStreamDestroy(p->side[k]);
     if (p->join[k]) cudaEventDestroy(p->join[k]);
   }
@@ -225,6 +229,67 @@ EventPair get_events(fstat_plan* p) {
   return e;
 }
 
+// Intermediates.  One pass of one short transform leaves most of the GPU idle and
+// lasts as long as its chain of loads, barriers and stores (~8 us), so FP32
+// plans give one launch several templates where their intermediates stay in
+// L2 (64 MB; 128 MB at 2^21, where the block is one of two per stream).  Above
+// 2^21 a template fills the GPU, and two streams overlap consecutive passes.
+int z_wanted(int64_t n_fft) {
+  if (n_fft > (int64_t(1) << 21)) return 2;
+  return (int)std::min<int64_t>(32, std::max<int64_t>(4, (int64_t(1) << 22) / n_fft));
+}
+
+cudaError_t alloc_z(fstat_plan* p) {
+  const size_t one = (size_t)p->d.n_fft * p->pair_bytes;
+  cudaError_t e = cudaErrorMemoryAllocation;
+  // (a plan with a cap on its memory keeps what one template per stream takes)
+  if (p->d.precision != FSTAT_FP64 && !p->alloc_cap) {
+    const int n = z_wanted(p->d.n_fft);
+    e = palloc(p, &p->Z, n * one);
+    if (e == cudaSuccess) {
+      p->n_z = n;
+      p->batched = true;
+    } else {
+      cudaGetLastError();
+    }
+  }
+  if (e != cudaSuccess) e = palloc(p, &p->Z, one);
+  for (int k = 0; k < p->n_z && k < fstat_plan::kMaxStreams && e == cudaSuccess; ++k) p->Zs[k] = (char*)p->Z + k * one;
+  return e;
+}
+
+// Templates per launch of a group of n, and the streams that the launches rotate
+// over.  Up to 2^16 one stream: a launch of many templates fills the GPU, and
+// the fork and join would cost more than the overlap of the two passes gives.
+// us per call of 16 templates, one per launch over four streams (two from 2^20
+// on) -> so: 2^13 117 -> 56, 2^16 115 -> 66, 2^18 134 -> 101, 2^19 164 -> 150,
+// 2^20 254 -> 236, 2^21 447 -> 441; of 4 templates: 2^13 62 -> 55, 2^18 82 -> 77.
+//
+// ring: fewer output rows than templates, 0 = a row each.  Later templates replace
+// earlier ones there, so a launch's rows differ and a row stays with one stream:
+// rows in order (ord ascending by one), and the streams' launches together
+// divide the ring; otherwise one template after the other.
+int template_batch(const fstat_plan* p, const int* ord, int64_t n, int64_t ring, int* streams) {
+  *streams = (int)std::min<int64_t>(p->nstream, n);
+  if (ring) {
+    while (ring % *streams) --*streams;
+    for (int64_t k = 1; k < n && *streams > 1; ++k)
+      if (ord[k] != ord[k - 1] + 1) *streams = 1;
+  }
+  if (!p->batched) return 1;
+  const int ns = p->d.n_fft <= (int64_t(1) << 16) ? 1 : 2;
+  int T = (int)std::min<int64_t>(p->n_z / ns, (n + ns - 1) / ns);
+  if (ring) {
+    while (T & (T - 1)) T &= T - 1;
+    while (T > 1 && ring % (T * ns)) T >>= 1;
+    for (int64_t k = 1; k < n && T > 1; ++k)
+      if (ord[k] != ord[k - 1] + 1) T = 1;
+    if (T == 1) return 1;
+  }
+  *streams = (int)std::min<int64_t>(ns, n);
+  return T;
+}
+
 double spin_spacing(const fstat_plan* p) { return (double)pass_a_spacing(p->log2n, p->log2n2); }
 
 // Per-sky work and the spindown coefficients of sorted templates
@@ -281,32 +346,36 @@ int set_split(fstat_plan* p, int log2n1) {
 bool warp_passes(const fstat_plan* p) { return p->d.precision != FSTAT_FP64; }
 
 // cb: rows per tile of the pass B that follows
-cudaError_t launch_a(fstat_plan* p, int ca, int va, int cb, const TmplCoef* coef, cudaStream_t st, void* Z = nullptr,
-                     int res = -1) {
+// T > 1 (FP32 plans): templates coef[0 .. T) in one launch, intermediates from Z on.
+cudaError_t launch_a(fstat_plan* p, int ca, int va, int cb, const TmplCoef* coef, cudaStream_t st,
+                     void* Z = nullptr, int res = -1, int T = 1) {
   if (!Z) Z = p->Z;
   if (res < 0) res = p->ra;
   ++p->n_launches;
   if (warp_passes(p)) {
     if (!pass_a_shape(p->log2n2, ca, va)) return cudaErrorInvalidConfiguration;
     const int staging = va >= 16 ? 1 : va == 2 ? 2 : 0;  // staged columns asked for; none asked for
-    return launch_wpass_a(p->log2n2, staging, p->G, p->gc, p->d.n_samples, (int)p->n1, coef, &Z,
-                          wpass_z_layout(p->log2n1, cb), 1, p->d_err, p->wait_limit, st, res);
+    return launch_wpass_a(p->log2n2, staging, p->G, p->gc, p->d.n_samples, (int)p->n1, coef, Z,
+                          wpass_z_layout(p->log2n1, cb), T, p->d_err, p->wait_limit, st, res);
   }
   return launch_pass_a_f64(p->log2n2, ca, va, p->G, p->gc, p->d.n_samples, (int)p->n1, p->tt.a, coef, Z, st, res);
 }
 
+// T > 1: rows ord[0 .. T) mod out_rows of out (their band keys from
+// pk->band_key + ord n_bands, pk->tmpl + ord; see launch_wpass_b*).
 cudaError_t launch_b(fstat_plan* p, int cb, int vb, float* out, cudaStream_t st, void* Z = nullptr,
-                     const PeakArgs* pk = nullptr, int res = -1) {
+                     const PeakArgs* pk = nullptr, int res = -1, int T = 1, const int* ord = nullptr,
+                     int64_t out_rows = 1) {
   if (!Z) Z = p->Z;
   if (res < 0) res = p->rb;
   ++p->n_launches;
   if (warp_passes(p)) {
     if (!pass_b_shape(p->log2n1, cb, vb)) return cudaErrorInvalidConfiguration;
     if (pk)
-      return launch_wpass_b_peak(p->log2n1, cb, &Z, 1, (int)p->n2, p->sky, nullptr,
+      return launch_wpass_b_peak(p->log2n1, cb, Z, T, (int)p->n2, p->sky, ord,
                                  pk->band_key ? (int)(p->d.n_fft >> pk->log2_band) : 0, *pk, p->d_err, p->wait_limit, st,
                                  res);
-    return launch_wpass_b(p->log2n1, cb, &Z, 1, (int)p->n2, p->sky, out, nullptr, 1, p->d_err, p->wait_limit, st, res);
+    return launch_wpass_b(p->log2n1, cb, Z, T, (int)p->n2, p->sky, out, ord, out_rows, p->d_err, p->wait_limit, st, res);
   }
   return launch_pass_b_f64(p->log2n1, cb, vb, Z, (int)p->n2, p->tt.b, p->sky, out, st, pk, res);
 }
@@ -405,15 +474,14 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   // whole columns of whole residues: up to N1 RL <= 2^12 x 16 pairs of padding
   if (e == cudaSuccess)
     e = palloc(p, &p->G, (size_t)(N + (int64_t(1) << (kMaxLog2 + (d.precision == FSTAT_FP64 ? 0 : 4)))) * p->pair_bytes);
-  if (e == cudaSuccess) e = palloc(p, &p->Z, (size_t)d.n_fft * p->pair_bytes);
+  if (e == cudaSuccess) e = alloc_z(p);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
   // short transforms leave most of the GPU idle between launches: four
   // template streams up to n_fft = 2^19 (measured on GB300: 2^18 runs 1.6x
   // faster with four than with two), two above (2^21: four are 8% slower)
   p->nstream = d.n_fft <= (int64_t(1) << 19) ? 4 : 2;
-  p->Zs[0] = p->Z;
   for (int k = 1; k < p->nstream && e == cudaSuccess; ++k) {
-    e = palloc(p, &p->Zs[k], (size_t)d.n_fft * p->pair_bytes);
+    if (!p->Zs[k]) e = palloc(p, &p->Zs[k], (size_t)d.n_fft * p->pair_bytes);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side[k], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join[k], cudaEventDisableTiming);
   }
@@ -682,42 +750,46 @@ int enqueue_compute(fstat_plan* p, const fstat_template* h_tmpl, const int* h_or
       i = j;
       continue;
     }
-    // Templates rotate over `st` and the plan's side streams, each with its
-    // own intermediate, so the passes of consecutive templates overlap; the
+    // Launches of tmax templates rotate over `st` and the plan's side streams, each
+    // with its own intermediates, so that consecutive passes overlap; the
     // side streams join back before the next sky position overwrites the
     // per-sky series.
-    const int ns = (int)std::min<int64_t>(p->nstream, j - i);
+    int ns = 0;
+    const int tmax = template_batch(p, h_ord + i, j - i, po || out_rows >= n ? 0 : out_rows, &ns);
     if (ns > 1) {
       CK(cudaEventRecord(p->fork, st));
       for (int q = 1; q < ns; ++q) CK(cudaStreamWaitEvent(p->side[q], p->fork, 0));
     }
-    for (int64_t k = i; k < j; ++k) {
-      float* out = po ? nullptr : twoF + ((int64_t)h_ord[k] % out_rows) * nfft;
+    for (int64_t k = i, b = 0; k < j; k += tmax, ++b) {
+      const int T = (int)std::min<int64_t>(tmax, j - k), q = (int)(b % ns);
+      // one template: its own row; more: the rows of the device's order
+      float* out = po ? nullptr : T > 1 ? twoF : twoF + ((int64_t)h_ord[k] % out_rows) * nfft;
+      const int* ord = T > 1 ? d_ord + k : nullptr;
       PeakArgs pk{};
       if (po) {
-        pk.band_key = po->n_bands > 0 ? p->keys + (int64_t)h_ord[k] * po->n_bands : nullptr;
+        const int64_t own = T > 1 ? 0 : h_ord[k];
+        pk.band_key = po->n_bands > 0 ? p->keys + own * po->n_bands : nullptr;
         pk.peaks = po->peaks;
         pk.count = po->n_peaks;
         pk.cap = po->n_peaks ? po->capacity : 0;
-        pk.tmpl = po->tmpl_offset + h_ord[k];
+        pk.tmpl = (int)(po->tmpl_offset + own);
         pk.thr = po->threshold;
         pk.log2_band = log2_band;
       }
       const TmplCoef* coef = d_coef + k;
-      const int q = (int)((k - i) % ns);
       cudaStream_t s = q ? p->side[q] : st;
-      void* Zb = p->Zs[q];
+      void* Zb = tmax > 1 ? (char*)p->Z + (size_t)q * tmax * nfft * p->pair_bytes : p->Zs[q];
       EventPair ea{}, eb{};
       if (prof) { ea = get_events(p); cudaEventRecord(ea.a, s); }
       const bool own = po && p->cb_pk >= 0;  // the peaks mode's own pass-B shape
       const int cb = own ? p->cb_pk : p->cb, vb = own ? p->vb_pk : p->vb;
-      cudaError_t e = launch_a(p, p->ca, p->va, cb, coef, s, Zb);
+      cudaError_t e = launch_a(p, p->ca, p->va, cb, coef, s, Zb, -1, T);
       if (e != cudaSuccess) return cuda_status(e);
       if (prof) {
         cudaEventRecord(ea.b, s); p->ev[0].push_back(ea); p->launches[0]++;
         eb = get_events(p); cudaEventRecord(eb.a, s);
       }
-      e = launch_b(p, cb, vb, out, s, Zb, po ? &pk : nullptr);
+      e = launch_b(p, cb, vb, out, s, Zb, po ? &pk : nullptr, -1, T, ord, out_rows);
       if (e != cudaSuccess) return cuda_status(e);
       if (prof) { cudaEventRecord(eb.b, s); p->ev[1].push_back(eb); p->launches[1]++; }
     }
@@ -1183,6 +1255,7 @@ int fstat_set_streams(fstat_plan* p, int n) {
     if (!p->join[k]) CK(cudaEventCreateWithFlags(&p->join[k], cudaEventDisableTiming));
   }
   p->nstream = n;
+  p->batched = false;  // one template per launch, over these streams
   return FSTAT_OK;
 }
 
@@ -1272,8 +1345,8 @@ std::string tune_key(const fstat_plan* p) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, p->device) != cudaSuccess) prop.name[0] = 0;
   char buf[400];
-  std::snprintf(buf, sizeof buf, "v6|%s|N=%lld|nfft=%lld|prec=%d|ndet=%d|ns=%d", prop.name,
-                (long long)p->d.n_samples, (long long)p->d.n_fft, p->d.precision, p->d.n_det, p->nstream);
+  std::snprintf(buf, sizeof buf, "v6|%s|N=%lld|nfft=%lld|prec=%d|ndet=%d|ns=%d%s", prop.name,
+                (long long)p->d.n_samples, (long long)p->d.n_fft, p->d.precision, p->d.n_det, p->nstream, p->batched ? "b" : "");
   for (char* c = buf; *c; ++c)
     if (*c == ' ' || *c == '\t') *c = '_';
   return buf;
@@ -1400,7 +1473,12 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
   std::vector<fstat_template> ht(p->h_tmpl, p->h_tmpl + kPipe);
   std::vector<int> ho(p->h_order, p->h_order + kPipe);
   float* out = nullptr;
-  CK(cudaMalloc(&out, (size_t)p->d.n_fft * sizeof(float)));
+  int64_t rows = p->batched ? p->n_z : p->nstream;  // a row per template in flight
+  if (cudaMalloc(&out, (size_t)rows * p->d.n_fft * sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    rows = 1;
+    CK(cudaMalloc(&out, (size_t)p->d.n_fft * sizeof(float)));
+  }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -1418,7 +1496,7 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
   // percent, about the spread of a single short trial.
   auto pipeline = [&](const fstat_peak_out* po) -> float {
     auto once = [&] {
-      return enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, 1, st, false, false,
+      return enqueue_compute(p, ht.data(), ho.data(), kPipe, p->d_tmpl, p->d_order, p->d_coef, out, rows, st, false, false,
                              po);
     };
     if (once()) { cudaGetLastError(); return -1.f; }

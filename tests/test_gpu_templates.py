@@ -1,0 +1,85 @@
+"""Templates that share launches give what each gives alone.
+
+A plan of up to 2^21 bins hands several templates of one sky position to one
+launch of each transform pass; fstat_set_streams(1) makes it one per launch.
+The arithmetic of a template is the same, so 2F, the band maxima and the
+crossings have to be equal bit for bit, in every count of templates (one, fewer
+than a launch holds, a launch and a rest), with sky positions interleaved.
+"""
+
+import numpy as np
+import pytest
+
+import paper_2201_00451_gb300 as pkg
+from workloads import small_target
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2201_00451_gb300 import build as fbuild
+
+    fbuild.build()
+    pkg.load()
+
+
+def bank(n, n_skies, span):
+    tm = np.zeros(n, dtype=pkg.TEMPLATE_DTYPE)
+    tm["alpha"] = np.array((0.4, 2.9, 5.0))[np.arange(n) % n_skies]
+    tm["delta"] = np.array((0.2, -0.7, 1.1))[np.arange(n) % n_skies]
+    tm["f1dot"] = np.linspace(-1.0, 1.0, n) * 40.0 / span ** 2
+    return tm
+
+
+@pytest.mark.parametrize("log2_n", [10, 13, 16, 17, 19, 21, 22])
+@pytest.mark.parametrize("n_tmpl,n_skies", [(1, 1), (2, 1), (5, 1), (7, 3), (37, 1), (70, 2)])
+def test_shared_launches_equal_single_ones(log2_n, n_tmpl, n_skies):
+    if log2_n > 19 and n_tmpl > 37:
+        pytest.skip("covered by the smaller lengths")
+    n = (1 << log2_n) * 5 // 7
+    t = small_target(n_samples=n, dt=2.0, n_fft=1 << log2_n, n_det=2, seed=log2_n, dtype="c64")
+    rng = np.random.default_rng(n_tmpl)
+    tm = bank(n_tmpl, n_skies, n * 2.0)
+    got = []
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            x = rng.standard_normal((n, 2)).astype(np.float32).view(np.complex64)[:, 0]
+            plan.set_data(X, x, t.sigmas[X])
+        for streams in (0, 1):
+            if streams:
+                plan.set_streams(streams)
+            two_f = plan.compute(tm)
+            pk = plan.compute_peaks(tm, threshold=14.0, n_bands=4, capacity=n_tmpl << (log2_n - 2))
+            assert int(pk["count"].item()) <= n_tmpl << (log2_n - 2)
+            plan.sync()
+            lst = np.sort(pkg.peaks_to_numpy(pk), order=("tmpl", "bin"))
+            got.append((two_f.cpu().numpy(), lst, pk["band_max"].cpu().numpy(), pk["band_bin"].cpu().numpy()))
+    assert np.all(np.isfinite(got[0][0]))
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("log2_n", [13, 18, 20])
+@pytest.mark.parametrize("rows", [1, 2, 3, 4, 8, 12])
+def test_ring_of_rows_keeps_the_last(log2_n, rows):
+    import torch
+
+    n = (1 << log2_n) * 5 // 7
+    t = small_target(n_samples=n, dt=2.0, n_fft=1 << log2_n, n_det=2, seed=1, dtype="c64")
+    rng = np.random.default_rng(rows)
+    tm = bank(24, 1, n * 2.0)
+    with pkg.FstatPlan.from_target(t) as plan, pkg.FstatBatch() as batch:
+        for X in range(2):
+            x = rng.standard_normal((n, 2)).astype(np.float32).view(np.complex64)[:, 0]
+            plan.set_data(X, x, t.sigmas[X])
+        want = plan.compute(tm)
+        if rows in (1, 3):  # not shared among launches: in order over one stream
+            plan.set_streams(1)
+        out = torch.zeros((rows, t.n_fft), dtype=torch.float32, device="cuda")
+        batch.add(plan, tm, out, out_rows=rows)
+        batch.instantiate()
+        batch.launch()
+        torch.cuda.synchronize()
+        for i in range(24 - rows, 24):
+            assert torch.equal(out[i % rows], want[i])

@@ -196,6 +196,7 @@ struct Geo {
   SkyNode* nodes;
   NodeF32* nodes32;                    // the same nodes in FP32 (mixed path)
   int n_nodes, node_log2;
+  const struct ResTab* rtab;           // the resampling's constants (sky.cu)
 };
 
 // ---------------------------------------------------- pair of complex values
@@ -276,11 +277,13 @@ inline GCol g_columns(int64_t n, int64_t n1, int rl) {
 // ------------------------------------------------------------ host helpers
 SkyPos sky_position(const Geo& g, double alpha, double delta);
 // Blocks of the resampling kernel for n samples (its A, B, C partial sums).
-int sky_blocks(int64_t n);
+size_t sky_partials_bytes(int64_t n);  // (zeroed once)
+size_t resample_table_bytes();
+cudaError_t launch_resample_table(const Geo& g, struct ResTab* t, cudaStream_t st);
 // Steps (iii)-(v) for one sky position, and the spindown coefficients of job's
 // templates (count 0: none).  Four launches.
 void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* const* xh, const int* xh_dtype, void* G,
-                int n1, GCol gc, double* partials, SkyConst* sky, int* err, const CoefJob& job, cudaStream_t st);
+                int n1, GCol gc, void* partials, SkyConst* sky, int* err, const CoefJob& job, cudaStream_t st);
 // Timing table: entries needed to cover [t_lo, t_hi] at spacing h, and the
 // kernel that fills them (FP64 sincos, once per plan).
 int time_table_entries(double t_lo, double t_hi, double h);

@@ -66,7 +66,8 @@ struct fstat_plan {
   cudaStream_t side[kMaxStreams] = {};
   cudaEvent_t fork = nullptr;
   cudaEvent_t join[kMaxStreams] = {};
-  double* partials = nullptr;
+  void* partials = nullptr;      // sums of the resampling's blocks (sky.cu)
+  ResTab* rtab = nullptr;        // its constants (geo.rtab)
   TimeTab* tab = nullptr;        // timing table and rotation cubics (geo.tab, geo.rot)
   Cubic* tm_tab = nullptr;       // per-sky Roemer delay cubics (geo.tm_tab)
   SkyNode* nodes = nullptr;      // per-sky timing nodes (geo.nodes)
@@ -172,6 +173,7 @@ void free_all(fstat_plan* p) {
   }
   if (p->fork) cudaEventDestroy(p->fork);
   if (p->partials) cudaFree(p->partials);
+  if (p->rtab) cudaFree(p->rtab);
   if (p->tab) cudaFree(p->tab);
   if (p->tm_tab) cudaFree(p->tm_tab);
   if (p->nodes) cudaFree(p->nodes);
@@ -303,7 +305,7 @@ int run_sky(fstat_plan* p, double alpha, double delta, const CoefJob& job, cudaS
   launch_sky(p->geo, p->d.precision, p->pos, xh, p->dtype, p->G, (int)p->n1, p->gc, p->partials, p->sky, p->d_err, job,
              st);
   CK(cudaGetLastError());
-  p->n_launches += 4;  // delay table, nodes, resampling, final sums and coefficients
+  p->n_launches += 3;  // delay table; nodes; resampling, sums and coefficients
   if (p->prof) { cudaEventRecord(e.b, st); p->ev[2].push_back(e); p->launches[2]++; }
   p->sky_valid = true;
   p->sky_alpha = alpha;
@@ -513,8 +515,12 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
     g.nodes = p->nodes;
     g.nodes32 = p->nodes32;
     if (e == cudaSuccess) e = launch_time_table(g, tab, rot, 0);
+    if (e == cudaSuccess) e = palloc(p, &p->rtab, resample_table_bytes());
+    if (e == cudaSuccess) e = launch_resample_table(g, p->rtab, 0);
+    g.rtab = p->rtab;
   }
-  if (e == cudaSuccess) e = palloc(p, &p->partials, (size_t)3 * sky_blocks(N) * sizeof(double));
+  if (e == cudaSuccess) e = palloc(p, &p->partials, sky_partials_bytes(N));
+  if (e == cudaSuccess) e = cudaMemset(p->partials, 0, sky_partials_bytes(N));
   if (e == cudaSuccess) e = palloc(p, &p->sky, sizeof(SkyConst));
   if (e == cudaSuccess && d.precision == FSTAT_FP64) e = palloc(p, &p->tw, (size_t)6 * (size_t(1) << kMaxLog2) * 16);
   if (e == cudaSuccess) e = palloc(p, &p->d_err, 2 * sizeof(int));

@@ -3,10 +3,10 @@
 // integrals A, B, C, D of eq. (Fstat).  The result G = (G_a, G_b) is stored
 // in the column-major layout the FFT pass A reads (GCol).
 //
-// Four launches per sky position: the delay table, the timing nodes, the
-// resampling (step iii applied as the detector samples are staged), the final
-// sums together with the templates' spindown coefficients.  Trigonometry of the
-// sky position alone is done on the host.
+// Three launches per sky position: the delay table; the timing nodes; the
+// resampling (step iii applied as the detector samples are staged), beside it
+// A, B, C, D and the templates' spindown coefficients.  Trigonometry of the sky
+// position alone is done on the host.
 //
 // Timing (t_m, the inversion T + t_m(T) = t_b, u = (T - t0)/dt) is FP64 in
 // both precisions; f_h t_m is reduced mod 1 in FP64 before the sincos.
@@ -137,7 +137,72 @@ __device__ __forceinline__ void node_weights(int r, int step_log2, double* w) {
   w[2] = -fp * f * f2 * 0.5;
   w[3] = fp * f * fm * (1.0 / 6.0);
 }
-constexpr int kMaxStep = 64;
+constexpr int kMaxStep = 64, kMaxD = 32;
+
+}  // namespace
+
+// What a resampling block would otherwise form again for every launch: node
+// weights by j mod step, the step matrix M of A, B, C, the taps' constants.
+struct ResTab {
+  double w[kMaxStep][4], m[4][4];
+  float wf[kMaxStep][4];
+  TapK<float> tf[2 * kMaxD + 1];
+  TapK<double> td[2 * kMaxD + 1];
+  float2 tt[kMaxD + 1];  // series form, see series_taps
+};
+
+namespace {
+
+__device__ __forceinline__ const TapK<float>* taps_of(const ResTab* t, float) { return t->tf; }
+__device__ __forceinline__ const TapK<double>* taps_of(const ResTab* t, double) { return t->td; }
+
+// Dirichlet kernel of the full series (length N) or of the 2D + 1 taps themselves
+template <typename T> __device__ __forceinline__ T kernel_len(const Geo& g) {
+  return g.interp == FSTAT_INTERP_PERIODIC ? (T)(2 * g.dterms + 1) : (T)g.n;
+}
+template <typename T> __device__ void form_tap(const Geo& g, int m, TapK<T>* out) {
+  T sn, cs;
+  TapK<T> q;
+  sincospi_t((T)m / kernel_len<T>(g), &sn, &cs);
+  q.c = cs;
+  q.s = sn;
+  sincospi_t((T)m * ((T)1 / (T)(g.dterms + 1)), &sn, &cs);
+  q.tc = cs;
+  q.ts = sn;
+  *out = q;
+}
+__global__ void k_resample_table(Geo g, ResTab* t) {
+  const int i = threadIdx.x, step = 1 << g.node_log2, D = g.dterms;
+  if (i < step) {
+    node_weights(i, g.node_log2, t->w[i]);
+    for (int q = 0; q < 4; ++q) t->wf[i][q] = (float)t->w[i][q];
+  }
+  if (i <= 2 * D) {
+    form_tap(g, i - D, &t->tf[i]);
+    form_tap(g, i - D, &t->td[i]);
+    const float h = g.interp == FSTAT_INTERP_TAPERED ? (i - D) & 1 ? -0.46f : 0.46f : 0.f;
+    if (i >= D) t->tt[i - D] = make_float2(h * t->tf[i].tc, h * t->tf[i].ts);
+  }
+  __syncthreads();
+  if (i < 16) {
+    double m = 0.0;
+    for (int r = 0; r < step; ++r) m += t->w[r][i >> 2] * t->w[r][i & 3];
+    t->m[i >> 2][i & 3] = m;
+  }
+}
+
+// Spindown polynomial of template i of the job (see TmplCoef).
+template <bool F64>
+__device__ __forceinline__ void tmpl_coef(const CoefJob& c, double j_ref, double dt, int64_t n, int i) {
+  if (i >= c.count) return;
+  const fstat_template tp = c.tmpl[c.order[c.first + i]];
+  c.out[c.first + i] = spin_coef<F64>(j_ref, n, dt, tp.f1dot, tp.f2dot, c.spacing);
+}
+template <bool F64>
+__global__ void __launch_bounds__(128)
+k_tmpl_coef(const __grid_constant__ CoefJob job, double j_ref, double dt, int64_t n) {
+  tmpl_coef<F64>(job, j_ref, dt, n, (int)blockIdx.x * 128 + (int)threadIdx.x);
+}
 
 // Timing nodes of the current sky position (FP64, every 2^node_log2 samples,
 // from one step before sample 0 on): the Roemer delay at the detector time, and
@@ -257,15 +322,15 @@ k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
 // sum_r a(r)^2 is the quadratic form a^T M a with M = sum_r W_r W_r^T
 // (and likewise b^T M b, a^T M b), exact algebra in FP64, one thread per
 // detector and step, in blocks of their own of the same launch, so that the
-// FP64 work runs beside the others' FP32 work.  Steps near the data's edges
-// (those not marked inner) sum their valid samples in the
-// sample blocks.
+// FP64 work runs beside the others' FP32 work.  A launch of its own to add the
+// sums and form the coefficients took 7 to 12 us; sums of the edges' samples by
+// the sample blocks, 4 us more for a fence in every block.
 //
 // Bound by instruction issue (55 % of the slots; half of the warps resident) and the
-// wait for a tile's samples.  Two detectors, D = 8, 10 days at 0.5 s: 76 us, where
+// wait for a tile's samples.  Two detectors, D = 8, 10 days at 0.5 s: 69 us, where
 // step (iii) as a pass of its own over memory and 25 instructions a tap took
-// 17 + 17 + 122; 120 days at 1 s: 482 us (42 + 42 + 683).
-constexpr int kMaxD = 32;
+// 17 + 17 + 122; 120 days at 1 s: 390 us (42 + 42 + 683).  D = 16, 400 001 samples:
+// 24 us (45 with the constants of ResTab formed by every block).
 constexpr int kWin = kSkyBlock + 2 * kMaxD + 8;  // staged window, samples (covers the drift)
 
 template <typename T> struct C2;
@@ -364,137 +429,218 @@ __device__ __forceinline__ void series_taps(int D, const TZ* wp, float d, float 
   *zi = i;
 }
 
+// Step (iv): the sample position u = k0 + dlt of SSB sample j at detector X,
+// interpolated between the timing nodes (node: the step's, m its index within the
+// detector).  FP32 path: u = j + v with v = vi + vf at the step's node plus the
+// weighted node-to-node changes (the interpolating cubic written about that node),
+// so the integer part is exact and only the fraction, |f| <~ 1/2, is rounded to
+// FP32.  FP64 plans (and the FP32-timing negative control) form u in FP64.
+// (k0 is held within 2^29: far outside the data, and invalid all the same.)
+template <typename T> constexpr bool kWide = sizeof(T) == sizeof(double) || kNegCtrlFp32;
+__device__ __forceinline__ int far_out(int k0) { return max(-(1 << 29), min(1 << 29, k0)); }
+__device__ __forceinline__ int position(int j, float vf, float dvm, float dv, float dvp, int vi, const float* wf, float* dlt) {
+  // (explicit operations: sample blocks and sums decide alike which samples are valid)
+  const float f = __fadd_rn(vf, __fmaf_rn(wf[2], dv, __fmaf_rn(wf[3], __fadd_rn(dv, dvp), __fmul_rn(-wf[0], dvm))));
+  const float big = __fadd_rn(f, 12582912.f);  // 1.5 2^23 + rint(f)
+  *dlt = __fsub_rn(f, __fsub_rn(big, 12582912.f));
+  return far_out(j + vi + (__float_as_int(big) - 0x4b400000));
+}
+template <typename T>
+__device__ __forceinline__ int position(int j, const SkyNode* nd, const double* wn, T* dlt) {
+  double u = (double)j + (wn[0] * nd[-1].v + wn[1] * nd[0].v + wn[2] * nd[1].v + wn[3] * nd[2].v);
+  if constexpr (kNegCtrlFp32) u = (double)((float)j + (float)(u - (double)j));
+  const int k0 = __double2int_rn(u);
+  *dlt = (T)(u - (double)k0);
+  return far_out(k0);
+}
+
+// Sums of the blocks that form A, B, C; done counts those that have left theirs.
+struct Partials {
+  unsigned* done;
+  double* sum;  // [blocks][3]
+};
+
+// A, B, C over the node steps, block b of nb: a whole step of valid samples
+// (inner) by its quadratic form, the samples of any other step one by one, a
+// quarter of them per thread (a short series is mostly such steps: 3000 samples
+// took 21 us with a step per thread).  The block that ends last adds the sums in
+// a fixed order and forms D and eq. (Fstat)'s weights.
+constexpr int kStepParts = 4;  // divides the shortest step
+template <typename T>
+__device__ __noinline__ void sum_abc(const Geo& g, int b, int nb, const Partials& left, SkyConst* sky, int* err) {
+  __shared__ double red[3][kSkyBlock / 32];
+  __shared__ bool last;
+  const ResTab* tab = g.rtab;
+  const int step = 1 << g.node_log2, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int steps = (int)((g.n + step - 1) >> g.node_log2), total = steps * g.n_det;
+  double v[3] = {0.0, 0.0, 0.0};
+  for (int i = b * kSkyBlock + t; i < kStepParts * total; i += nb * kSkyBlock) {
+    const int part = i / total, is = i - part * total;
+    const int X = is / steps, sg = is - X * steps;
+    const SkyNode* nd = g.nodes + X * g.n_nodes + sg + 1;
+    const NodeF32* nf = g.nodes32 + X * g.n_nodes + sg + 1;
+    const bool inner = nf[0].inner;
+    if (inner && part > 0) continue;
+    const double av[4] = {nd[-1].a, nd[0].a, nd[1].a, nd[2].a};
+    const double bv[4] = {nd[-1].b, nd[0].b, nd[1].b, nd[2].b};
+    double aa = 0.0, bb = 0.0, ab = 0.0;
+    if (inner) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        double ma = 0.0, mb = 0.0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          ma += tab->m[q][r] * av[r];
+          mb += tab->m[q][r] * bv[r];
+        }
+        aa += av[q] * ma;
+        bb += bv[q] * mb;
+        ab += av[q] * mb;
+      }
+    } else {
+      const int per = step / kStepParts;
+#pragma unroll 2
+      for (int r = part * per; r < (part + 1) * per; ++r) {
+        const int j = (sg << g.node_log2) + r;
+        const double* wn = tab->w[r];
+        int k0;
+        T dlt;
+        if constexpr (kWide<T>) k0 = position<T>(j, nd, wn, &dlt);
+        else k0 = position(j, nf[0].vf, nf[-1].dv, nf[0].dv, nf[1].dv, nf[0].vi, tab->wf[r], &dlt);
+        if (j >= g.n || k0 < 0 || k0 > g.n - 1) continue;
+        const double a = wn[0] * av[0] + wn[1] * av[1] + wn[2] * av[2] + wn[3] * av[3];
+        const double c = wn[0] * bv[0] + wn[1] * bv[1] + wn[2] * bv[2] + wn[3] * bv[3];
+        aa += a * a;
+        bb += c * c;
+        ab += a * c;
+      }
+    }
+    const double w = g.w[X];
+    v[0] += w * aa;
+    v[1] += w * bb;
+    v[2] += w * ab;
+  }
+  // over the block; result in thread 0
+  auto reduce = [&] {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+      if (lane == 0) red[q][wid] = v[q];
+    }
+    __syncthreads();
+    if (wid == 0)
+      for (int q = 0; q < 3; ++q) {
+        v[q] = lane < kSkyBlock / 32 ? red[q][lane] : 0.0;
+        for (int o = kSkyBlock / 64; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+      }
+  };
+  reduce();
+  if (nb > 1) {
+    if (t == 0) {
+      for (int q = 0; q < 3; ++q) left.sum[3 * b + q] = v[q];
+      __threadfence();
+      last = atomicAdd(left.done, 1u) == (unsigned)nb - 1;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int q = 0; q < 3; ++q) v[q] = t < nb ? __ldcg(left.sum + 3 * t + q) : 0.0;  // nb <= kSkyBlock
+    reduce();
+    if (t == 0) *left.done = 0;  // for the next launch
+  }
+  if (t > 0) return;
+  double A = v[0], B = v[1], C = v[2];
+  double D = A * B - C * C;
+  sky->A = A;
+  sky->B = B;
+  sky->C = C;
+  sky->D = D;
+  const bool ok = isfinite(D) && D > 1e-12 * A * B && A > 0.0 && B > 0.0;
+  if (!ok) {
+    atomicCAS(err, 0, FSTAT_ERR_DEGENERATE);
+    D = 1.0;
+    A = B = C = 0.0;
+  }
+  const double inv = 1.0 / D;
+  sky->kA = 2.0 * A * inv;
+  sky->kB = 2.0 * B * inv;
+  sky->kC = 4.0 * C * inv;
+  sky->kAf = (float)sky->kA;
+  sky->kBf = (float)sky->kB;
+  sky->kCf = (float)sky->kC;
+}
+
 template <typename T, bool C128>
 __global__ void __launch_bounds__(kSkyBlock, sizeof(T) == 4 ? 4 : 2)
 k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typename PairMem<T>::type* __restrict__ G,
-           int n1_log2, GCol gc, int tiles, int sample_blocks, double* __restrict__ partials) {
+           int n1_log2, GCol gc, int tiles, int sample_blocks, const Partials part, int sum_blocks, SkyConst* __restrict__ sky,
+           int* __restrict__ err, const __grid_constant__ CoefJob job, double j_ref) {
   using TZ = typename C2<T>::type;
+  // the sums and the coefficients, by the launch's first blocks: both are chains of
+  // FP64 operations that the others' time hides
+  const int block = (int)blockIdx.x - ((int)gridDim.x - sample_blocks);
+  if (block < 0) {
+    if ((int)blockIdx.x < sum_blocks) sum_abc<T>(g, (int)blockIdx.x, sum_blocks, part, sky, err);
+    else
+      tmpl_coef<sizeof(T) == sizeof(double)>(job, j_ref, g.dt, g.n, ((int)blockIdx.x - sum_blocks) * kSkyBlock + (int)threadIdx.x);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TZ* win_all = reinterpret_cast<TZ*>(smem_raw);  // [n_det][kWin]
   __shared__ TapK<T> tk[2 * kMaxD + 1];
   __shared__ float2 s_tt[kMaxD + 1];
   __shared__ int s_span[kMaxDet][2];
-  __shared__ double s_w[kMaxStep][4], s_m[4][4];  // node weights by j mod step; step matrix M
-  __shared__ float s_wf[kMaxStep][4];
+  __shared__ double s_w[kWide<T> ? kMaxStep : 1][4];  // node weights by j mod step
+  __shared__ __align__(16) float s_wf[kMaxStep][4];
   const int step_log2 = g.node_log2, step = 1 << step_log2;
   const int D = g.dterms;
-  const T nT = (T)g.n;
-  // Dirichlet kernel of the full series (length N) or of the 2D + 1 taps
-  // themselves; the Hamming taper only for the default kernel
-  const T len = g.interp == FSTAT_INTERP_PERIODIC ? (T)(2 * D + 1) : nT;
-  const bool taper = g.interp == FSTAT_INTERP_TAPERED;
+  const T len = kernel_len<T>(g);
+  const bool taper = g.interp == FSTAT_INTERP_TAPERED;  // the Hamming taper only for the default kernel
   const T inv_taper = (T)1 / (T)(D + 1);
   // (pi (D + 1/2) / N)^4 7/360 < 3e-9
   const bool series = sizeof(T) == sizeof(float) && g.interp != FSTAT_INTERP_PERIODIC &&
                       3.14159265f * ((float)D + 0.5f) < 0.0198f * (float)g.n;
-  for (int m = threadIdx.x; m <= 2 * D; m += blockDim.x) {
-    T sn, cs;
-    TapK<T> q;
-    sincospi_t((T)(m - D) / len, &sn, &cs);
-    q.c = cs;
-    q.s = sn;
-    sincospi_t((T)(m - D) * inv_taper, &sn, &cs);
-    q.tc = cs;
-    q.ts = sn;
-    tk[m] = q;
-    if (m >= D) {
-      const float h = taper ? ((m - D) & 1 ? -0.46f : 0.46f) : 0.f;
-      s_tt[m - D] = make_float2(h * (float)cs, h * (float)sn);
-    }
-  }
+  const ResTab* tab = g.rtab;
+  // (taps outside a staged window and short series take the general form)
+  for (int m = threadIdx.x; m <= 2 * D; m += blockDim.x) tk[m] = taps_of(tab, T())[m];
+  if (threadIdx.x >= 128 && threadIdx.x - 128 <= D) s_tt[threadIdx.x - 128] = tab->tt[threadIdx.x - 128];
   if (threadIdx.x < step) {
-    node_weights(threadIdx.x, step_log2, s_w[threadIdx.x]);
+    *reinterpret_cast<float4*>(s_wf[threadIdx.x]) = *reinterpret_cast<const float4*>(tab->wf[threadIdx.x]);
+    if (kWide<T>)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) s_wf[threadIdx.x][q] = (float)s_w[threadIdx.x][q];
+      for (int q = 0; q < 4; ++q) s_w[threadIdx.x][q] = tab->w[threadIdx.x][q];
   }
   __syncthreads();
-  const double* wn = s_w[threadIdx.x & (step - 1)];
+  const double* wn = s_w[kWide<T> ? threadIdx.x & (step - 1) : 0];
   const float* wf = s_wf[threadIdx.x & (step - 1)];
-  double sa = 0.0, sb = 0.0, sab = 0.0;
-  bool summed = false;  // this thread added to sa, sb, sab
-  const int abc = (int)blockIdx.x - sample_blocks;
-  if (abc >= 0) {  // A, B, C of the inner steps, a grid of the launch's last blocks
-    if (threadIdx.x < 16) {
-      const int q = threadIdx.x >> 2, r2 = threadIdx.x & 3;
-      double m = 0.0;
-      for (int r = 0; r < step; ++r) m += s_w[r][q] * s_w[r][r2];
-      s_m[q][r2] = m;
-    }
-    __syncthreads();
-    const int steps = (int)((g.n + step - 1) >> step_log2), total = steps * g.n_det;
-    for (int i = abc * kSkyBlock + (int)threadIdx.x; i < total; i += ((int)gridDim.x - sample_blocks) * kSkyBlock) {
-      const int X = i / steps, sg = i - X * steps;
-      const int node0 = X * g.n_nodes + sg + 1;
-      if (!g.nodes32[node0].inner) continue;
-      const SkyNode* nd = g.nodes + node0;
-      const double av[4] = {nd[-1].a, nd[0].a, nd[1].a, nd[2].a};
-      const double bv[4] = {nd[-1].b, nd[0].b, nd[1].b, nd[2].b};
-      double aMa = 0.0, bMb = 0.0, aMb = 0.0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double ma = 0.0, mb = 0.0;
-#pragma unroll
-        for (int r2 = 0; r2 < 4; ++r2) {
-          ma += s_m[q][r2] * av[r2];
-          mb += s_m[q][r2] * bv[r2];
-        }
-        aMa += av[q] * ma;
-        bMb += bv[q] * mb;
-        aMb += av[q] * mb;
-      }
-      const double w = g.w[X];
-      sa += w * aMa;
-      sb += w * bMb;
-      sab += w * aMb;
-    }
-    summed = true;
-  }
-  for (int tile = blockIdx.x; abc < 0 && tile < tiles; tile += sample_blocks) {
+  for (int tile = block; tile < tiles; tile += sample_blocks) {
     const int j0 = tile * kSkyBlock;
     const int j = j0 + (int)threadIdx.x;
     const int j_last = min(j0 + kSkyBlock, (int)g.n) - 1;
-    // steps (iv)-(v): the sample position u of T (T + t_m(T) = t_b^j),
-    // interpolated between the timing nodes, as k0 = rint(u) and dlt = u - k0
-    // for u = j + v.  FP32 path: v = vi + vf at this step's node, plus the
-    // weighted node-to-node changes (the interpolating cubic written about that
-    // node), so the integer part is exact and only the fraction, |f| <~ 1/2, is
-    // rounded to FP32.  FP64 plans (and the FP32-timing negative control) form
-    // u in FP64.
     const int node_j = (min(j, j_last) >> step_log2) + 1;
     int k0s[kMaxDet];
     T dlts[kMaxDet], was[kMaxDet], wbs[kMaxDet];
-    unsigned inner = 0;  // detector X's step is an inner one
 #pragma unroll
     for (int X = 0; X < kMaxDet; ++X) {
       if (X >= g.n_det) break;
       int k0;
       T dlt;
-      if constexpr (sizeof(T) == sizeof(float) && !kNegCtrlFp32) {
+      if constexpr (!kWide<T>) {
         const NodeF32* nf = g.nodes32 + X * g.n_nodes + node_j;
         auto abvd = [&](int q) { return *reinterpret_cast<const float4*>(&nf[q]); };  // a, b, vf, dv
         const float4 m1 = abvd(-1), z0 = abvd(0), p1 = abvd(1), p2 = abvd(2);
-        const int2 vi = *reinterpret_cast<const int2*>(&nf[0].vi);
-        const float f = z0.z + ((wf[2] * z0.w + wf[3] * (z0.w + p1.w)) - wf[0] * m1.w);
-        const float big = __fadd_rn(f, 12582912.f);  // 1.5 2^23 + rint(f)
-        k0 = j + vi.x + (__float_as_int(big) - 0x4b400000);
-        dlt = __fsub_rn(f, __fsub_rn(big, 12582912.f));
+        k0 = position(j, z0.z, m1.w, z0.w, p1.w, nf[0].vi, wf, &dlt);
         // the antenna patterns at T, weighted
         const float wx = g.wf[X];
         was[X] = wx * (wf[0] * m1.x + wf[1] * z0.x + wf[2] * p1.x + wf[3] * p2.x);
         wbs[X] = wx * (wf[0] * m1.y + wf[1] * z0.y + wf[2] * p1.y + wf[3] * p2.y);
-        inner |= (vi.y ? 1u : 0u) << X;
       } else {
         const SkyNode* nd = g.nodes + X * g.n_nodes + node_j;
-        double u = (double)j + (wn[0] * nd[-1].v + wn[1] * nd[0].v + wn[2] * nd[1].v + wn[3] * nd[2].v);
-        if constexpr (kNegCtrlFp32) u = (double)((float)j + (float)(u - (double)j));
-        k0 = __double2int_rn(u);
-        dlt = (T)(u - (double)k0);
+        k0 = position<T>(j, nd, wn, &dlt);
         const double w = g.w[X];
         was[X] = (T)(w * (wn[0] * nd[-1].a + wn[1] * nd[0].a + wn[2] * nd[1].a + wn[3] * nd[2].a));
         wbs[X] = (T)(w * (wn[0] * nd[-1].b + wn[1] * nd[0].b + wn[2] * nd[1].b + wn[3] * nd[2].b));
-        inner |= (g.nodes32[X * g.n_nodes + node_j].inner ? 1u : 0u) << X;
       }
-      k0 = max(-(1 << 29), min(1 << 29, k0));  // far outside the data: invalid all the same
       if (j == j0) s_span[X][0] = k0;
       if (j == j_last) s_span[X][1] = k0;
       k0s[X] = k0;
@@ -521,7 +667,6 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
     }
     __syncthreads();
     Pair<T> acc = pzero<T>();
-    unsigned edge = 0;  // detectors with a valid sample in a step that is not inner
 #pragma unroll
     for (int X = 0; X < kMaxDet; ++X) {
       if (X >= g.n_det) break;
@@ -577,7 +722,6 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
           }
         }
       }
-      edge |= (~inner >> X & 1u) << X;
       // the antenna-weighted detector sum G (FP32 a, b in the mixed path)
       const T wa = was[X], wb = wbs[X];
       acc.ar += wa * zr;
@@ -585,102 +729,10 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
       acc.br += wb * zr;
       acc.bi += wb * zi;
     }
-    // (a loop of its own: predicated into the one above, its FP64 instructions
-    // would take their issue slots of that pipe for every sample)
-    for (; edge; edge &= edge - 1) {
-      const int X = __ffs(edge) - 1;
-      const SkyNode* nd = g.nodes + X * g.n_nodes + node_j;
-      const double w = g.w[X];
-      const double a = wn[0] * nd[-1].a + wn[1] * nd[0].a + wn[2] * nd[1].a + wn[3] * nd[2].a;
-      const double b = wn[0] * nd[-1].b + wn[1] * nd[0].b + wn[2] * nd[1].b + wn[3] * nd[2].b;
-      summed = true;
-      sa += w * a * a;
-      sb += w * b * b;
-      sab += w * a * b;
-    }
     if (j < g.n) {
       const int n2i = j >> n1_log2;
       pstore(G + (int64_t)(j - (n2i << n1_log2)) * gc.lc + gc.at(n2i), acc);
     }
-  }
-  // block reduction of the A, B, C partial sums (fixed order).  Only the
-  // warps that summed anything reduce (per-sample sums arise only at the data's
-  // edges): the others' zeros would not change a bit of the result.
-  __shared__ double red[3][kSkyBlock / 32];
-  if (__any_sync(0xffffffffu, summed)) {
-    for (int o = 16; o > 0; o >>= 1) {
-      sa += __shfl_down_sync(0xffffffffu, sa, o);
-      sb += __shfl_down_sync(0xffffffffu, sb, o);
-      sab += __shfl_down_sync(0xffffffffu, sab, o);
-    }
-  }
-  const int wid = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { red[0][wid] = sa; red[1][wid] = sb; red[2][wid] = sab; }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double t = 0;
-    for (int i = 0; i < kSkyBlock / 32; ++i) t += red[threadIdx.x][i];
-    partials[3 * blockIdx.x + threadIdx.x] = t;
-  }
-}
-
-// Spindown polynomial of template i of the job (see TmplCoef).
-template <bool F64>
-__device__ __forceinline__ void tmpl_coef(const CoefJob& c, double j_ref, double dt, int64_t n, int i) {
-  if (i >= c.count) return;
-  const fstat_template tp = c.tmpl[c.order[c.first + i]];
-  c.out[c.first + i] = spin_coef<F64>(j_ref, n, dt, tp.f1dot, tp.f2dot, c.spacing);
-}
-constexpr int kFinal = 512;
-
-// Block 0: A, B, C from the blocks' partial sums (fixed order), eq. (Fstat)'s
-// weights.  The other blocks (all of them for n_partials < 0): the job's
-// spindown coefficients, kFinal templates each.
-template <bool F64>
-__global__ void __launch_bounds__(kFinal)
-k_sky_finalize(const double* __restrict__ partials, int n_partials, SkyConst* sky, int* err,
-               const __grid_constant__ CoefJob job, double j_ref, double dt, int64_t n) {
-  const int sums = n_partials >= 0;
-  if ((int)blockIdx.x >= sums) {
-    tmpl_coef<F64>(job, j_ref, dt, n, ((int)blockIdx.x - sums) * kFinal + (int)threadIdx.x);
-    return;
-  }
-  __shared__ double red[3][kFinal / 32];
-  double v[3] = {0.0, 0.0, 0.0};
-#pragma unroll 4
-  for (int i = threadIdx.x; i < n_partials; i += kFinal)
-#pragma unroll
-    for (int q = 0; q < 3; ++q) v[q] += partials[3 * i + q];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
-    if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = v[q];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double A = 0.0, B = 0.0, C = 0.0;
-    for (int i = 0; i < kFinal / 32; ++i) {
-      A += red[0][i];
-      B += red[1][i];
-      C += red[2][i];
-    }
-    double D = A * B - C * C;
-    sky->A = A;
-    sky->B = B;
-    sky->C = C;
-    sky->D = D;
-    bool ok = isfinite(D) && D > 1e-12 * A * B && A > 0.0 && B > 0.0;
-    if (!ok) {
-      atomicCAS(err, 0, FSTAT_ERR_DEGENERATE);
-      D = 1.0;
-      A = B = C = 0.0;
-    }
-    sky->kA = 2.0 * A / D;
-    sky->kB = 2.0 * B / D;
-    sky->kC = 4.0 * C / D;
-    sky->kAf = (float)sky->kA;
-    sky->kBf = (float)sky->kB;
-    sky->kCf = (float)sky->kC;
   }
 }
 
@@ -741,24 +793,20 @@ int sample_blocks(int64_t n) {
   const int64_t per = std::min<int64_t>(8, std::max<int64_t>(1, tiles / full));
   return (int)((tiles + per - 1) / per);
 }
-// blocks for the step sums: at least four steps per thread for long data
-int step_blocks(int64_t n) { return (int)std::min<int64_t>(device_sm_count(), n / (16 * 4 * kSkyBlock) + 1); }
+// blocks for the step sums, at most as many as the last one has threads to add
+int step_blocks(int64_t n) { return (int)std::min<int64_t>(std::min(device_sm_count(), kSkyBlock), n / (16 / kStepParts * kSkyBlock) + 1); }
 }  // namespace
 
-int sky_blocks(int64_t n) { return sample_blocks(n) + step_blocks(n); }
+size_t sky_partials_bytes(int64_t n) { return 16 + (size_t)step_blocks(n) * 3 * sizeof(double); }
 
-namespace {
-void finalize(const SkyPos& pos, const Geo& g, int precision, const double* partials, int n_partials, SkyConst* sky,
-              int* err, const CoefJob& job, cudaStream_t st) {
-  const int blocks = (n_partials >= 0) + (job.count + kFinal - 1) / kFinal;
-  if (blocks == 0) return;
-  const auto k = precision == FSTAT_FP64 ? k_sky_finalize<true> : k_sky_finalize<false>;
-  k<<<blocks, kFinal, 0, st>>>(partials, n_partials, sky, err, job, pos.j_ref, g.dt, g.n);
+size_t resample_table_bytes() { return sizeof(ResTab); }
+cudaError_t launch_resample_table(const Geo& g, ResTab* t, cudaStream_t st) {
+  k_resample_table<<<1, 2 * kMaxD + 1, 0, st>>>(g, t);
+  return cudaGetLastError();
 }
-}  // namespace
 
 void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* const* xh, const int* xh_dtype, void* G,
-                int n1, GCol gc, double* partials, SkyConst* sky, int* err, const CoefJob& job, cudaStream_t st) {
+                int n1, GCol gc, void* partials, SkyConst* sky, int* err, const CoefJob& job, cudaStream_t st) {
   k_sky_table<<<(g.tab_n + kTabOut - 1) / kTabOut, kTabThreads, 0, st>>>(g, pos);
   const dim3 nodes((unsigned)((g.n_nodes + kNodeOut - 1) / kNodeOut), (unsigned)g.n_det);
   k_sky_nodes<<<nodes, kNodeThreads, 0, st>>>(g, pos);
@@ -769,21 +817,27 @@ void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* cons
     x.c128[X] = xh_dtype[X] == FSTAT_C128;
     c128 = c128 || x.c128[X];
   }
-  const int samples = sample_blocks(g.n), blocks = sky_blocks(g.n), tiles = (int)((g.n + kSkyBlock - 1) / kSkyBlock);
+  const int samples = sample_blocks(g.n), sums = step_blocks(g.n), tiles = (int)((g.n + kSkyBlock - 1) / kSkyBlock);
   int l1 = 0;
   while ((1 << l1) < n1) ++l1;
+  const int blocks = samples + sums + (job.count + kSkyBlock - 1) / kSkyBlock;
+  const Partials part{(unsigned*)partials, (double*)((char*)partials + 16)};
   const size_t smem = (size_t)g.n_det * kWin * (precision == FSTAT_FP64 ? 16 : 8);  // at most 21 KB
   if (precision == FSTAT_FP64)
-    k_resample<double, true><<<blocks, kSkyBlock, smem, st>>>(g, x, (PairMem<double>::type*)G, l1, gc, tiles, samples, partials);
+    k_resample<double, true><<<blocks, kSkyBlock, smem, st>>>(g, x, (PairMem<double>::type*)G, l1, gc, tiles, samples, part, sums, sky, err,
+                                                              job, pos.j_ref);
   else if (c128)
-    k_resample<float, true><<<blocks, kSkyBlock, smem, st>>>(g, x, (float4*)G, l1, gc, tiles, samples, partials);
+    k_resample<float, true><<<blocks, kSkyBlock, smem, st>>>(g, x, (float4*)G, l1, gc, tiles, samples, part, sums, sky, err,
+                                                              job, pos.j_ref);
   else
-    k_resample<float, false><<<blocks, kSkyBlock, smem, st>>>(g, x, (float4*)G, l1, gc, tiles, samples, partials);
-  finalize(pos, g, precision, partials, blocks, sky, err, job, st);
+    k_resample<float, false><<<blocks, kSkyBlock, smem, st>>>(g, x, (float4*)G, l1, gc, tiles, samples, part, sums, sky, err,
+                                                              job, pos.j_ref);
 }
 
 void launch_tmpl_coef(const SkyPos& pos, const Geo& g, int precision, const CoefJob& job, cudaStream_t st) {
-  finalize(pos, g, precision, nullptr, -1, nullptr, nullptr, job, st);
+  if (job.count == 0) return;
+  const auto k = precision == FSTAT_FP64 ? k_tmpl_coef<true> : k_tmpl_coef<false>;
+  k<<<(job.count + 127) / 128, 128, 0, st>>>(job, pos.j_ref, g.dt, g.n);
 }
 
 // Scan an input series for NaN/Inf.

@@ -203,14 +203,9 @@ struct CandConst {
 // Antenna patterns (JKS 1998 eqs. 12-13) as harmonics of phi for one
 // detector: with H = alpha - phi and u = (1, cos 2H, sin 2H, cos H, sin H),
 // a = sum ka_i u_i, b = sum kb_i u_i, and their sky derivatives.
-__device__ void patterns(double lam, double gam, double alpha, double delta, double (*p)[5]) {
-  double sl, cl, sg, cg, sd, cd, s2d, c2d;
-  sincos(lam, &sl, &cl);
-  sincos(2.0 * gam, &sg, &cg);
-  sincos(delta, &sd, &cd);
-  s2d = 2.0 * sd * cd;
-  c2d = cd * cd - sd * sd;
-  const double s2l = 2.0 * sl * cl, c2l = cl * cl - sl * sl;
+__device__ void patterns(const Geo& g, int X, double sa, double ca, double sd, double cd, double (*p)[5]) {
+  const double sl = g.sl[X], cl = g.cl[X], sg = g.s2g[X], cg = g.c2g[X], s2l = g.s2l[X], c2l = g.c2l[X];
+  const double s2d = 2.0 * sd * cd, c2d = cd * cd - sd * sd;
   // value and d/ddelta of the coefficients
   const double k[4][5] = {
       {0.75 * sg * cl * cl * cd * cd, sg * (3.0 - c2l) * (3.0 - c2d) / 16.0, -0.25 * cg * sl * (3.0 - c2d),
@@ -219,8 +214,6 @@ __device__ void patterns(double lam, double gam, double alpha, double delta, dou
       {-1.5 * sg * cl * cl * cd * sd, sg * (3.0 - c2l) * s2d / 8.0, -0.5 * cg * sl * s2d, 0.5 * sg * s2l * c2d,
        -cg * cl * c2d},
       {0.0, cg * sl * cd, 0.25 * sg * (3.0 - c2l) * cd, -cg * cl * sd, -0.5 * sg * s2l * sd}};
-  double sa, ca;
-  sincos(alpha, &sa, &ca);
   const double s2a = 2.0 * sa * ca, c2a = ca * ca - sa * sa;
   auto turn = [&](const double* u, double* o) {
     o[0] = u[0];
@@ -237,32 +230,59 @@ __device__ void patterns(double lam, double gam, double alpha, double delta, dou
   }
 }
 
-// sums over the sample grid of cos(m phi), sin(m phi), m = 0..4, per detector
-struct Harmonics { double c[kMaxDet][5], s[kMaxDet][5]; };
+// sums over the sample grid of the products of two harmonics 1, cos 2phi, sin 2phi,
+// cos phi, sin phi, per detector
+struct Harmonics { double m[kMaxDet][5][5]; };
 
 // sum_k w u(phi_k) v(phi_k) for two patterns u, v over the grid
-__device__ double pat_sum(const double* u, const double* v, const double* C, const double* S) {
-  // products of the harmonics: 1, cos 2phi, sin 2phi, cos phi, sin phi
-  const double m[5][5] = {{C[0], C[2], S[2], C[1], S[1]},
-                          {C[2], 0.5 * (C[0] + C[4]), 0.5 * S[4], 0.5 * (C[3] + C[1]), 0.5 * (S[3] - S[1])},
-                          {S[2], 0.5 * S[4], 0.5 * (C[0] - C[4]), 0.5 * (S[3] + S[1]), 0.5 * (C[1] - C[3])},
-                          {C[1], 0.5 * (C[3] + C[1]), 0.5 * (S[3] + S[1]), 0.5 * (C[0] + C[2]), 0.5 * S[2]},
-                          {S[1], 0.5 * (S[3] - S[1]), 0.5 * (C[1] - C[3]), 0.5 * S[2], 0.5 * (C[0] - C[2])}};
+__device__ __forceinline__ double pat_sum(const double* u, const double* v, const double (*m)[5]) {
   double t = 0.0;
   for (int i = 0; i < 5; ++i)
     for (int j = 0; j < 5; ++j) t += u[i] * m[i][j] * v[j];
   return t;
 }
 
-__global__ void k_cand_consts(Geo g, Harmonics h, const fstat_candidate* __restrict__ cand, int n,
-                              CandConst* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const fstat_candidate c = cand[i];
-  CandConst& k = out[i];
+// A warp per candidate.  The chain of FP64 operations is what this kernel lasts (64 us
+// with a thread per candidate, whatever their number), so the eleven sums of each
+// detector go to lanes of their own.  With k_finalize's CTA per candidate a call for
+// one candidate over 10 days takes 82 us instead of 137, for 256 of them 1183
+// instead of 1246.
+constexpr int kSums = 11;
+__global__ void __launch_bounds__(32)
+k_cand_consts(const __grid_constant__ Geo g, const __grid_constant__ Harmonics h, const fstat_candidate* __restrict__ cand,
+              CandConst* __restrict__ out) {
+  __shared__ double s_sum[kMaxDet * kSums];
+  const int lane = threadIdx.x;
+  const fstat_candidate c = cand[blockIdx.x];
+  CandConst& k = out[blockIdx.x];
   double sa, ca, sd, cd;
   sincos(c.alpha, &sa, &ca);
   sincos(c.delta, &sd, &cd);
+  for (int i = lane; i < g.n_det * kSums; i += 32) {
+    const int X = i / kSums, q = i - X * kSums;
+    double p[kPat][5];
+    patterns(g, X, sa, ca, sd, cd, p);
+    if (q < kPat)
+      for (int m = 0; m < 5; ++m) k.pat[X][q][m] = (float)p[q][m];
+    // 0-2: aa, bb, ab; then a da, b db, da b, a db by alpha and by delta
+    const int d = q < 3 ? 0 : q < 7 ? 1 : 2, e = q < 3 ? q : (q - 3) & 3;
+    const double *da = p[2 * d], *db = p[2 * d + 1];
+    const double* u = e == 1 ? p[1] : d && e == 2 ? da : p[0];
+    const double* v = e == 0 ? da : d && e == 2 ? p[1] : db;
+    s_sum[i] = pat_sum(u, v, h.m[X]);
+  }
+  __syncwarp();
+  if (lane < 9) {
+    const int d = lane / 3, e = lane - 3 * d;
+    double t = 0.0;
+    for (int X = 0; X < g.n_det; ++X) {
+      const double* r = s_sum + X * kSums + (d ? 4 * d - 1 : 0);
+      const double w = d ? 2.0 * g.w[X] : g.w[X];
+      t += d && e == 2 ? g.w[X] * (r[2] + r[3]) : w * r[e];
+    }
+    k.abc[lane] = t;
+  }
+  if (lane > 0) return;
   k.nx = df_from(cd * ca);
   k.ny = df_from(cd * sa);
   k.nz = df_from(sd);
@@ -283,23 +303,6 @@ __global__ void k_cand_consts(Geo g, Harmonics h, const fstat_candidate* __restr
   k.f2 = (float)c.f2dot;
   k.dt = df_from(g.dt);
   k.pad_ = 0.f;
-  double abc[9] = {};
-  for (int X = 0; X < g.n_det; ++X) {
-    double p[kPat][5];
-    patterns(g.lat[X], g.gam[X], c.alpha, c.delta, p);
-    for (int q = 0; q < kPat; ++q)
-      for (int m = 0; m < 5; ++m) k.pat[X][q][m] = (float)p[q][m];
-    for (int d = 0; d < 3; ++d) {
-      // d = 0: the values; 1, 2: the alpha and delta derivatives
-      const double *a = p[0], *b = p[1], *da = p[2 * d], *db = p[2 * d + 1];
-      const double w = d ? 2.0 * g.w[X] : g.w[X];
-      abc[3 * d] += w * pat_sum(a, da, h.c[X], h.s[X]);
-      abc[3 * d + 1] += w * pat_sum(b, db, h.c[X], h.s[X]);
-      abc[3 * d + 2] += d ? g.w[X] * (pat_sum(da, b, h.c[X], h.s[X]) + pat_sum(a, db, h.c[X], h.s[X]))
-                          : w * pat_sum(a, b, h.c[X], h.s[X]);
-    }
-  }
-  for (int q = 0; q < 9; ++q) k.abc[q] = abc[q];
 }
 
 // ------------------------------------------------------------ the sums
@@ -534,24 +537,33 @@ k_moments(int n_det, int64_t tiles, const float2* __restrict__ xt, const float* 
 
 // sum the chunk partials (fixed order) and apply the chain rule in FP64, one
 // warp per candidate; partial[chunk][cand][kAcc]
-__global__ void k_finalize(const double* __restrict__ partial, const CandConst* __restrict__ cc, int n_cand,
-                           int n_chunks, float* __restrict__ twoF, float* __restrict__ grad) {
+// (a CTA per candidate: a warp alone took 30 us for the 211 chunks of 10 days)
+__global__ void __launch_bounds__(kWarps * 32)
+k_finalize(const double* __restrict__ partial, const CandConst* __restrict__ cc, int n_cand, int n_chunks,
+           float* __restrict__ twoF, float* __restrict__ grad) {
   __shared__ double s_sum[kWarps][kAcc];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kWarps + warp;
-  if (i >= n_cand) return;
+  const int i = blockIdx.x;
   if (lane < kAcc) {
     double t[4] = {0.0, 0.0, 0.0, 0.0};
-    int c = 0;
-    for (; c + 4 <= n_chunks; c += 4)
+    int c = warp;
+    for (; c + 3 * kWarps < n_chunks; c += 4 * kWarps)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) t[q] += partial[((int64_t)(c + q) * n_cand + i) * kAcc + lane];
-    for (; c < n_chunks; ++c) t[0] += partial[((int64_t)c * n_cand + i) * kAcc + lane];
+      for (int q = 0; q < 4; ++q) t[q] += partial[((int64_t)(c + q * kWarps) * n_cand + i) * kAcc + lane];
+    for (; c < n_chunks; c += kWarps) t[0] += partial[((int64_t)c * n_cand + i) * kAcc + lane];
     s_sum[warp][lane] = (t[0] + t[1]) + (t[2] + t[3]);
+  }
+  __syncthreads();
+  if (warp > 0) return;
+  if (lane < kAcc) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) t += s_sum[w][lane];
+    s_sum[0][lane] = t;
   }
   __syncwarp();
   if (lane >= 4) return;
-  const double* s = s_sum[warp];
+  const double* s = s_sum[0];
   const double* m = cc[i].abc;
   const double A = m[0], B = m[1], C = m[2];
   const double D = A * B - C * C;
@@ -579,15 +591,23 @@ __global__ void k_finalize(const double* __restrict__ partial, const CandConst* 
 // exp(i m (phi_0 + (n-1) step / 2)) sin(n x) / sin(x), x = m step / 2
 Harmonics harmonics(const Geo& g) {
   Harmonics h{};
-  for (int X = 0; X < g.n_det; ++X)
+  for (int X = 0; X < g.n_det; ++X) {
+    double C[5], S[5];
     for (int m = 0; m <= 4; ++m) {
       const double step = g.w_rot * g.dt, x = 0.5 * m * step, n = (double)g.n, sx = sin(x);
       // at a multiple of pi the quotient's limit, n cos(n x) / cos(x)
       const double amp = fabs(sx) < 1e-14 ? n * cos(n * x) / cos(x) : sin(n * x) / sx;
       const double mid = m * (g.lon[X] + g.sid_ph0 + g.w_rot * g.t0 + 0.5 * (n - 1.0) * step);
-      h.c[X][m] = amp * cos(mid);
-      h.s[X][m] = amp * sin(mid);
+      C[m] = amp * cos(mid);
+      S[m] = amp * sin(mid);
     }
+    const double m[5][5] = {{C[0], C[2], S[2], C[1], S[1]},
+                            {C[2], 0.5 * (C[0] + C[4]), 0.5 * S[4], 0.5 * (C[3] + C[1]), 0.5 * (S[3] - S[1])},
+                            {S[2], 0.5 * S[4], 0.5 * (C[0] - C[4]), 0.5 * (S[3] + S[1]), 0.5 * (C[1] - C[3])},
+                            {C[1], 0.5 * (C[3] + C[1]), 0.5 * (S[3] + S[1]), 0.5 * (C[0] + C[2]), 0.5 * S[2]},
+                            {S[1], 0.5 * (S[3] - S[1]), 0.5 * (C[1] - C[3]), 0.5 * S[2], 0.5 * (C[0] - C[2])}};
+    for (int i = 0; i < 25; ++i) h.m[X][i / 5][i % 5] = m[i / 5][i % 5];
+  }
   return h;
 }
 
@@ -649,7 +669,7 @@ cudaError_t launch_grad(const Geo& g, const void* tables, const fstat_candidate*
   const float w_step = (float)(g.w_rot * g.dt);
   for (int c0 = 0; c0 < n_cand; c0 += batch) {
     const int n = std::min(batch, n_cand - c0);
-    k_cand_consts<<<(n + 31) / 32, 32, 0, st>>>(g, h, cand_dev + c0, n, cc);
+    k_cand_consts<<<n, 32, 0, st>>>(g, h, cand_dev + c0, cc);
     const unsigned grid = (unsigned)(((int64_t)n * chunks + kWarps - 1) / kWarps);
     auto run = [&](auto kernel) {
       kernel<<<grid, kWarps * 32, 0, st>>>(g.n_det, l.tiles, x, nodes, w_step, cc, n, chunks, partial);
@@ -660,7 +680,7 @@ cudaError_t launch_grad(const Geo& g, const void* tables, const fstat_candidate*
       case 8: run(k_moments<8>); break;
       default: run(k_moments<1>); break;
     }
-    k_finalize<<<(n + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(partial, cc, n, chunks, twoF + c0, grad + 4 * (int64_t)c0);
+    k_finalize<<<n, kWarps * 32, 0, st>>>(partial, cc, n, chunks, twoF + c0, grad + 4 * (int64_t)c0);
   }
   return cudaGetLastError();
 }

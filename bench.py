@@ -146,7 +146,7 @@ def peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for name in ("fft_impl.cuh", "fstat_internal.cuh"):
+    for name in ("fft_impl.cuh", "fft_warp.cuh", "fstat_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2201_00451_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

@@ -16,7 +16,7 @@ constexpr int kMinLog2 = 5;         // FFT pass lengths 32 .. 4096 (pass B rows)
 constexpr int kMaxLog2 = 12;
 constexpr int kMaxLog2A = 13;       // pass A columns up to 8192 (FP32 plans)
 
-// Per-sky results in device memory (k_sky_finalize): the antenna-pattern
+// Per-sky results in device memory (k_resample's sums): the antenna-pattern
 // integrals and the weights of eq. (Fstat), 2A/D, 2B/D, 4C/D
 // (2F = kB|Fa|^2 + kA|Fb|^2 - kC Re FaFb*).
 struct SkyConst {

@@ -701,7 +701,18 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
         if (!done) {
           T sdl, cdl;
           sincospi_t(d / len, &sdl, &cdl);
-          for (int m = -D; m <= D; ++m) {
+          if (inside) {  // no bounds per tap (samples outside the data are staged as 0)
+            const TZ* wp = win + i0;
+#pragma unroll 4
+            for (int m = -D; m <= D; ++m) {
+              const TapK<T> q = tk[m + D];
+              const T sx = sdl * q.c - cdl * q.s;
+              T wgt = tap_div((m & 1) ? -sd : sd, len * sx);
+              if (taper) wgt *= (T)0.54 + (T)0.46 * (cdt * q.tc + sdt * q.ts);
+              zr += (T)wp[m].x * wgt;
+              zi += (T)wp[m].y * wgt;
+            }
+          } else for (int m = -D; m <= D; ++m) {
             const int k = k0 + m;
             if (k < 0 || k >= g.n) continue;
             // sin(pi (d - m)) = (-1)^m sin(pi d); sin(pi (d - m)/len) by angle addition

@@ -52,7 +52,7 @@ NARROW = ("narrowband single target: H1+L1, 10 d, dt=0.5 s, 1,728,000 c64 sample
 
 
 def headline_config(world: int) -> dict:
-    """The ``config`` object both arms print (the driver compares them)."""
+    """The ``config`` object both arms print, equal in both."""
     return {"workload": WORKLOAD, "templates_per_step": 16384, "sky_positions_in_job": 64,
             "n_fft": 1 << 24, "n_samples": 10_368_000,
             "l2": "flushed between steps (256 MB write, untimed); inputs (2 x 83 MB x_h, 166 MB "

@@ -333,10 +333,12 @@ int fstat_set_cta(fstat_plan* plan, int ca, int va, int cb, int vb);
 int fstat_set_residency(fstat_plan* plan, int ra, int rb);
 int fstat_get_residency(const fstat_plan* plan, int* ra, int* rb);
 
-/* Number of streams (1..8; default 4 for n_fft <= 2^19, else 2) over which consecutive templates
- * rotate inside fstat_compute; each stream owns an n_fft-point intermediate
- * (16 B per point in FP32), so the FFT passes of consecutive templates
- * overlap.  Synchronises. */
+/* Number of streams (1..8) over which consecutive templates rotate inside
+ * fstat_compute, one template per launch; each stream owns an n_fft-point
+ * intermediate (16 B per point in FP32), so the FFT passes of consecutive
+ * templates overlap.  Without this call: two above n_fft = 2^21; FP32 plans up
+ * to there hand several templates to one launch, on one stream up to 2^16 and
+ * two above; FP64 plans use four up to 2^19, else two.  Synchronises. */
 int fstat_set_streams(fstat_plan* plan, int n);
 
 /* Persistent launch of the template loop (Sec. 3 template loop; the paper

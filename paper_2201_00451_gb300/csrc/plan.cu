@@ -478,9 +478,9 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
     e = palloc(p, &p->G, (size_t)(N + (int64_t(1) << (kMaxLog2 + (d.precision == FSTAT_FP64 ? 0 : 4)))) * p->pair_bytes);
   if (e == cudaSuccess) e = alloc_z(p);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
-  // short transforms leave most of the GPU idle between launches: four
-  // template streams up to n_fft = 2^19 (measured on GB300: 2^18 runs 1.6x
-  // faster with four than with two), two above (2^21: four are 8% slower)
+  // where templates do not share launches (FP64, segment sums): four template
+  // streams up to n_fft = 2^19 (2^18 runs 1.6x faster with four than with two),
+  // two above (2^21: four are 8% slower)
   p->nstream = d.n_fft <= (int64_t(1) << 19) ? 4 : 2;
   for (int k = 1; k < p->nstream && e == cudaSuccess; ++k) {
     if (!p->Zs[k]) e = palloc(p, &p->Zs[k], (size_t)d.n_fft * p->pair_bytes);

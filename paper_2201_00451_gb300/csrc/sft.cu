@@ -287,7 +287,10 @@ cudaError_t run_sft(const void* bins, int64_t n_sft, int B, double f_het, double
   size_t smem = (size_t)(plan.np > 1 ? 2 : 1) * B * sizeof(V);
   const bool in_smem = smem + (size_t)B * sizeof(V) <= kSftSmemMax;
   if (in_smem) smem += (size_t)B * sizeof(V);
-  cudaError_t e = cudaFuncSetAttribute(k_sft_to_xh<T, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the limit belongs to the kernel, not to this call: every call sets the same
+  // value, so that none lowers it between another thread's setting and launch)
+  cudaError_t e =
+      cudaFuncSetAttribute(k_sft_to_xh<T, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSftSmemMax);
   if (e != cudaSuccess) return e;
   k_sft_roots<T><<<(B + 255) / 256, 256, 0, st>>>(B, (V*)roots);
   const bool direct = plan.np == 1 && plan.r[0] > max_radix<T>();

@@ -139,42 +139,46 @@ def test_every_kind_of_band_length(nb, precision, tol):
 
 def test_two_threads_with_different_band_lengths():
     # distinct plans may be used at the same time: bands of 3600 bins (three
-    # buffers of shared memory, 86 KB) and of 30 from two host threads, every
-    # series equal to what the same call gives alone
+    # buffers of shared memory, 86 KB) from one host thread and short ones from
+    # three others for 1.5 s, bins on the device so that the calls follow each
+    # other closely; every call succeeds, and the last gives what it gave alone
     import threading
+    import time
 
-    t_sft, calls = 1800.0, 400
-    plans, bands, alone = [], [], []
-    for nb in (3600, 30):
+    t_sft = 1800.0
+    jobs = []
+    for nb in (3600, 30, 30, 60):
         t = small_target(n_samples=2 * nb, dt=t_sft / nb, n_fft=1 << max(10, (2 * nb - 1).bit_length()), n_det=1,
                          f_het=100.0, seed=126, dtype="c64")
         rng = np.random.default_rng(nb)
-        bands.append((rng.standard_normal((2, nb)) + 1j * rng.standard_normal((2, nb))).astype(np.complex64))
-        plans.append(pkg.FstatPlan.from_target(t))
+        b = (rng.standard_normal((2, nb)) + 1j * rng.standard_normal((2, nb))).astype(np.complex64)
+        jobs.append((pkg.FstatPlan.from_target(t), torch.from_numpy(b).cuda(), nb))
 
-    def load(i, stream=None):
-        nb = bands[i].shape[1]
-        plans[i].set_sfts(0, bands[i], int(100.0 * t_sft) - nb // 2, t_sft, 2 * nb, 1.0, stream=stream)
+    def load(job, stream=None):
+        plan, bins, nb = job
+        plan.set_sfts(0, bins, int(100.0 * t_sft) - nb // 2, t_sft, 2 * nb, 1.0, stream=stream)
 
-    for i in range(2):
-        load(i)
-        alone.append(plans[i].export_data(0))
-    failed = []
+    alone, failed = [], []
+    for job in jobs:
+        load(job)
+        alone.append(job[0].export_data(0))
+    stop = time.monotonic() + 1.5
 
-    def work(i):
+    def work(job):
         s = torch.cuda.Stream()
-        try:
-            for _ in range(calls):
-                load(i, s)
-        except pkg.FstatError as e:
-            failed.append((i, e.code))
+        while time.monotonic() < stop:
+            try:
+                load(job, s)
+            except pkg.FstatError as e:
+                failed.append((job[2], e.code))
+        load(job, s)
 
-    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    threads = [threading.Thread(target=work, args=(job,)) for job in jobs]
     for th in threads:
         th.start()
     for th in threads:
         th.join()
-    assert not failed, failed
-    for i in range(2):
-        assert np.array_equal(plans[i].export_data(0), alone[i])
-        plans[i].close()
+    assert not failed, (len(failed), failed[:3])
+    for job, want in zip(jobs, alone):
+        assert np.array_equal(job[0].export_data(0), want)
+        job[0].close()

@@ -125,7 +125,6 @@ struct fstat_plan {
   // templates (FP32 plans, splits with a compiled fused shape)
   bool fused = false;
   int* fq = nullptr;       // launch state of the fused kernel
-  int64_t fq_cap = 0;      // templates it has room for
 };
 
 namespace {
@@ -676,21 +675,13 @@ bool fused_ok(const fstat_plan* p) {
   return p->d.precision == FSTAT_MIXED && fused_supported(p->log2n1, p->log2n2);
 }
 
-// The fused launch's ring of intermediates and its launch state.
-int fused_buffers(fstat_plan* p, int64_t T) {
+// The fused launch's ring of intermediates and its launch state (256 KB, for the
+// most templates of one launch: a captured batch keeps its address, so a later
+// call with more templates must not replace it).
+int fused_buffers(fstat_plan* p) {
   for (int r = 0; r < kRing; ++r)
     if (!p->Zs[r]) CK(palloc(p, &p->Zs[r], (size_t)p->d.n_fft * p->pair_bytes));
-  if (T > p->fq_cap) {
-    const int64_t c = std::min<int64_t>(kFusedMaxT, std::max<int64_t>(T, 256));
-    if (p->fq) {
-      CK(cudaDeviceSynchronize());
-      cudaFree(p->fq);
-      p->fq = nullptr;
-      p->fq_cap = 0;
-    }
-    CK(palloc(p, &p->fq, queue_ints((int)c) * sizeof(int)));
-    p->fq_cap = c;
-  }
+  if (!p->fq) CK(palloc(p, &p->fq, queue_ints((int)kFusedMaxT) * sizeof(int)));
   return FSTAT_OK;
 }
 
@@ -698,7 +689,7 @@ int fused_buffers(fstat_plan* p, int64_t T) {
 // launches of up to kFusedMaxT templates each.
 int enqueue_fused(fstat_plan* p, int64_t i, int64_t j, const int* d_ord, const TmplCoef* d_coef, float* twoF,
                   int64_t out_rows, cudaStream_t st, bool prof) {
-  int rc = fused_buffers(p, std::min<int64_t>(kFusedMaxT, j - i));
+  int rc = fused_buffers(p);
   if (rc) return rc;
   for (int64_t k0 = i; k0 < j; k0 += kFusedMaxT) {
     const int T = (int)std::min<int64_t>(kFusedMaxT, j - k0);

@@ -170,3 +170,23 @@ def test_fused_unsupported_split_and_precision_are_refused():
         with pytest.raises(pkg.FstatError) as e:
             plan.set_fused(True)
         assert e.value.code == -7
+
+
+def test_a_captured_batch_outlives_a_larger_call():
+    # the graph holds the plan's launch state: a call with more templates than
+    # the batch's (past 256, where the state used to be replaced) leaves it valid
+    t, xs = _noise_target(18, 86_411, seed=340, n_f1=300)
+    tm = t.templates()
+    with pkg.FstatPlan.from_target(t) as plan, pkg.FstatBatch() as batch:
+        for X in range(2):
+            plan.set_data(X, xs[X], t.sigmas[X])
+        plan.set_split(512)
+        plan.set_fused(True)
+        out = torch.zeros((5, t.n_fft), dtype=torch.float32, device="cuda")
+        batch.add(plan, tm[:5], out)
+        batch.instantiate()
+        want = plan.compute(tm)
+        out.zero_()
+        batch.launch()
+        plan.sync()
+        assert torch.equal(out, want[:5])

@@ -362,8 +362,9 @@ int fstat_get_fused(const fstat_plan* plan, int* enabled);
 
 /* Polls of the first wait for each of pass B's tile loads and of the wait for
  * each staged column of pass A (FP32 plans): a kernel that waits longer records
- * FSTAT_ERR_TIMEOUT (returned by fstat_sync), lets its copies in flight land
- * under the full default limit, and returns.  polls < 0 restores the default
+ * FSTAT_ERR_TIMEOUT (returned by fstat_sync), sets the bins it leaves unformed
+ * to NaN (fstat_compute and fstat_semicoherent, not the persistent launch), lets
+ * its copies in flight land under the full default limit, and returns.  polls < 0 restores the default
  * (2^22 polls); 0 makes every first wait give up at once, which tests of the
  * timeout path use.  In the persistent launch (fstat_set_fused) the limit
  * also bounds each work item's wait for the items it depends on.  Takes
@@ -412,11 +413,22 @@ int fstat_get_peaks_cta(const fstat_plan* plan, int* cb, int* vb);
  * the GPU (different streams, or different host threads) race on it.  The
  * first call on each device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current; make that first call
- * before any stream capture.  Errors: INVALID_ARG, UNSUPPORTED, DEGENERATE,
- * CUDA. */
+ * before any stream capture.  The passes' waits for their own copies are
+ * bounded: bins that a wait which ran out leaves unformed are NaN.  Errors:
+ * INVALID_ARG, UNSUPPORTED, DEGENERATE, CUDA. */
 int fstat_twoF_noalloc(const void* g_pairs, int64_t n_samples, int64_t n_fft, double dt, double tau0,
                        double A, double B, double C, double f1dot, double f2dot, float* twoF,
                        void* stream);
+
+/* The same call, which also reports a wait that ran out: *status (DEVICE int,
+ * may be NULL; 0 before the first call) is set to FSTAT_ERR_TIMEOUT by then,
+ * and a status other than 0 stays until the caller clears it.  wait_polls:
+ * polls of the first wait for each staged column and tile (< 0: the default,
+ * 2^22; 0 makes every first wait give up at once, for tests of the timeout
+ * path).  Errors: as above. */
+int fstat_twoF_noalloc_status(const void* g_pairs, int64_t n_samples, int64_t n_fft, double dt, double tau0,
+                              double A, double B, double C, double f1dot, double f2dot, float* twoF,
+                              int* status, int wait_polls, void* stream);
 
 /* Batch: several plans' template banks (uneven targets: different sample
  * counts, spans and FFT lengths) captured once into one CUDA graph and

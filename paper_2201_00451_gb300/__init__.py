@@ -43,7 +43,7 @@ EXPORTS = (
     "fstat_plan_create", "fstat_set_data", "fstat_compute", "fstat_freq_axis",
     "fstat_invalidate_sky", "fstat_export_sky", "fstat_sync", "fstat_set_profiling",
     "fstat_kernel_stats", "fstat_get_split", "fstat_set_split", "fstat_plan_destroy",
-    "fstat_strerror", "fstat_twoF_noalloc", "fstat_get_cta", "fstat_set_cta", "fstat_autotune",
+    "fstat_strerror", "fstat_twoF_noalloc", "fstat_twoF_noalloc_status", "fstat_get_cta", "fstat_set_cta", "fstat_autotune",
     "fstat_grad", "fstat_batch_create", "fstat_batch_add", "fstat_batch_instantiate",
     "fstat_batch_launch", "fstat_batch_nodes", "fstat_batch_destroy", "fstat_set_streams",
     "fstat_compute_peaks", "fstat_semicoherent", "fstat_set_residency", "fstat_get_residency",
@@ -139,6 +139,7 @@ def open_library(path: str) -> ctypes.CDLL:
         "fstat_plan_destroy": (None, [P]),
         "fstat_strerror": (ctypes.c_char_p, [i32]),
         "fstat_twoF_noalloc": (i32, [P, i64, i64, dbl, dbl, dbl, dbl, dbl, dbl, dbl, P, P]),
+        "fstat_twoF_noalloc_status": (i32, [P, i64, i64, dbl, dbl, dbl, dbl, dbl, dbl, dbl, P, P, i32, P]),
         "fstat_get_cta": (i32, [P] + [ctypes.POINTER(i32)] * 4),
         "fstat_get_peaks_cta": (i32, [P] + [ctypes.POINTER(i32)] * 2),
         "fstat_set_cta": (i32, [P, i32, i32, i32, i32]),

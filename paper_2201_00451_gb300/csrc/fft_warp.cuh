@@ -138,6 +138,11 @@ template <int L, int CB, int SUBMAX> __device__ __forceinline__ int out_index(in
   return u + (e / S::RE) * S::GW + (e % S::RE) * (S::SUB / S::RE);
 }
 
+__device__ __forceinline__ Pair<float> nan_pair() {
+  const float q = __int_as_float(0x7fffffff);
+  return {q, q, q, q};
+}
+
 // ------------------------------------------------------------- pass A
 // G holds column n1's samples residue by residue: sample n2 = r + RL j at
 // [(n1 RL + r) lcs + j].  STAGED: the next column (RL lcs pairs) is copied by
@@ -180,6 +185,10 @@ k_wpass_a(const float4* __restrict__ G, int lcs, int n, int n1, const TmplCoef* 
     }
     __syncthreads();
   }
+  auto z_col = [&](int col) { return (col & ((1 << zy.rl) - 1)) * zy.sub + (col >> zy.rl); };  // [r][j]
+  auto z_at = [&](int zp, int k2) {
+    return (((int64_t)(k2 >> zy.cb) * n1 + zp) << zy.cb) + (k2 & ((1 << zy.cb) - 1));
+  };
   bool all_ok = true;
   for (; tile < n_tiles; tile += gridDim.x) {
     const int k = tile / tpt, col = (tile - k * tpt) * S::COLS + cc;
@@ -231,11 +240,9 @@ k_wpass_a(const float4* __restrict__ G, int lcs, int n, int n1, const TmplCoef* 
             if (threadIdx.x == 0 && tile + (int)gridDim.x < n_tiles) issue(tile + gridDim.x);
         },
         [] {});
-    const int zp = (col & ((1 << zy.rl) - 1)) * zy.sub + (col >> zy.rl);  // [r][j]
     float4* z = z0 + (int64_t)k * L * n1;
-    auto zat = [&](int k2) {
-      return (((int64_t)(k2 >> zy.cb) * n1 + zp) << zy.cb) + (k2 & ((1 << zy.cb) - 1));
-    };
+    const int zp = z_col(col);
+    auto zat = [&](int k2) { return z_at(zp, k2); };
     if constexpr (L >= 512) {  // the outputs' spacing is a multiple of any CB
       float4* z0 = z + zat(out_index<L, 1, kSubA>(0, u, threadIdx.x));
 #pragma unroll
@@ -245,11 +252,20 @@ k_wpass_a(const float4* __restrict__ G, int lcs, int n, int n1, const TmplCoef* 
       for (int e = 0; e < 16; ++e) pstore(z + zat(out_index<L, 1, kSubA>(e, u, threadIdx.x)), v[e]);
     }
   }
-  if (STAGED && !all_ok && threadIdx.x == 0) {
-    // a wait ran out: record it, then give the copy still in flight a
-    // bounded chance to land before the CTA's shared memory goes away
-    if (err) atomicCAS(err, 0, FSTAT_ERR_TIMEOUT);
-    for (unsigned q = waited; q < issued; ++q) mbar_wait(bar, q & 1u);
+  if (STAGED && !all_ok) {
+    // a wait ran out: the columns not formed become NaN (which pass B carries to
+    // every bin), so that nobody takes what was there before for a result;
+    // record it, then give the copy still in flight a bounded chance to land
+    // before the CTA's shared memory goes away
+    for (; tile < n_tiles; tile += gridDim.x) {
+      const int k = tile / tpt, c0 = (tile - k * tpt) * S::COLS;
+      for (int i = threadIdx.x; i < S::COLS * L; i += S::NT)
+        pstore(z0 + (int64_t)k * L * n1 + z_at(z_col(c0 + i / L), i & (L - 1)), nan_pair());
+    }
+    if (threadIdx.x == 0) {
+      if (err) atomicCAS(err, 0, FSTAT_ERR_TIMEOUT);
+      for (unsigned q = waited; q < issued; ++q) mbar_wait(bar, q & 1u);
+    }
   }
 }
 
@@ -440,8 +456,21 @@ k_wpass_b(int n2, const SkyConst* __restrict__ sky, float* __restrict__ out, con
     }
   }
   if (!all_ok) {
-    // a wait ran out: record it, then give the loads still in flight a
-    // bounded chance to land before the CTA's shared memory goes away
+    // a wait ran out: 2F of the rows not formed becomes NaN (as in pass A);
+    // record it, then give the loads still in flight a bounded chance to land
+    // before the CTA's shared memory goes away
+    if constexpr (MODE != kPeaks) {
+      for (int tile = blockIdx.x + it * gridDim.x; tile < n_tiles; tile += gridDim.x) {
+        const int k = tile / tpt, m0 = (tile - k * tpt) * CB;
+        if (ord) row = out + (int64_t)(ord[k] % out_rows) * ((int64_t)n2 * L);
+        for (int i = threadIdx.x; i < L * CB; i += S::NT) {
+          const int mg = m0 + (i & (CB - 1)) + n2 * (i / CB) - (MODE == kAccumulate ? pk.shift : 0);
+          const bool in = MODE == kStore || (unsigned)mg < (unsigned)(n2 * L);
+          if (in) row[mg] = nan_pair().ar;
+          else if (pk.first) row[mg & (n2 * L - 1)] = 0.f;
+        }
+      }
+    }
     if (threadIdx.x == 0) {
       if (pk.err) atomicCAS(pk.err, 0, FSTAT_ERR_TIMEOUT);
       for (int g = M::NQ * it; g < issued; ++g) mbar_wait(&bar[g % M::NSLOT], (unsigned)(g / M::NSLOT) & 1u);

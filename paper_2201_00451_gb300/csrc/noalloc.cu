@@ -98,6 +98,13 @@ using namespace fstat;
 extern "C" int fstat_twoF_noalloc(const void* g_pairs, int64_t n_samples, int64_t n_fft, double dt,
                                   double tau0, double A, double B, double C, double f1dot,
                                   double f2dot, float* twoF, void* stream) {
+  return fstat_twoF_noalloc_status(g_pairs, n_samples, n_fft, dt, tau0, A, B, C, f1dot, f2dot, twoF, nullptr, -1,
+                                   stream);
+}
+
+extern "C" int fstat_twoF_noalloc_status(const void* g_pairs, int64_t n_samples, int64_t n_fft, double dt,
+                                         double tau0, double A, double B, double C, double f1dot,
+                                         double f2dot, float* twoF, int* status, int wait_polls, void* stream) {
   if (!g_pairs || !twoF || n_samples < 1 || !(dt > 0.0) || !isfinite(tau0) || !isfinite(f1dot) ||
       !isfinite(f2dot) || !isfinite(A) || !isfinite(B) || !isfinite(C))
     return FSTAT_ERR_INVALID_ARG;
@@ -129,10 +136,10 @@ extern "C" int fstat_twoF_noalloc(const void* g_pairs, int64_t n_samples, int64_
       NoallocArgs{A, B, C, tau0, dt, f1dot, f2dot, (double)pass_a_spacing(log2n, log2n2)});
   if (cudaGetLastError() != cudaSuccess) return FSTAT_ERR_CUDA;
   void* Z = p.Z;
-  cudaError_t e = launch_wpass_a(log2n2, 0, p.G, gc, n_samples, n1, p.coef, Z, wpass_z_layout(log2n1, 0), 1, nullptr, -1,
-                                 st, 0);
+  cudaError_t e = launch_wpass_a(log2n2, 0, p.G, gc, n_samples, n1, p.coef, Z, wpass_z_layout(log2n1, 0), 1, status,
+                                 wait_polls, st, 0);
   if (e != cudaSuccess) return FSTAT_ERR_CUDA;
-  e = launch_wpass_b(log2n1, 0, Z, 1, n2, p.sky, twoF, nullptr, 1, nullptr, -1, st, 0);
+  e = launch_wpass_b(log2n1, 0, Z, 1, n2, p.sky, twoF, nullptr, 1, status, wait_polls, st, 0);
   if (e != cudaSuccess) return FSTAT_ERR_CUDA;
   return FSTAT_OK;
 }

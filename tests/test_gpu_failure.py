@@ -114,3 +114,64 @@ def test_device_memory_cap_gives_oom_and_leaves_plans_usable(monkeypatch):
         plan.sync()
     assert _ok(out, resamp.fstat(t, x, tm))
     assert os.environ.get("FSTAT_DEVICE_BYTES_CAP") is None
+
+
+@pytest.mark.parametrize("log2_n,split,va", [(10, 0, 0), (13, 0, 0), (18, 0, 2), (20, 1024, 0), (20, 256, 2), (21, 256, 16)])
+def test_a_pass_that_gave_up_leaves_no_stale_bins(log2_n, split, va):
+    # rows of an earlier call in the output: with every first wait given up at
+    # once (staged pass A and pass B, or pass B alone with va 2), no bin of it is left
+    import torch
+
+    n = (1 << log2_n) * 5 // 8
+    t = small_target(n_samples=n, dt=2.0, n_fft=1 << log2_n, n_det=2, seed=3, dtype="c64", f1dots=(0.0, 1e-16, 2e-16))
+    rng = np.random.default_rng(log2_n)
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            plan.set_data(X, (rng.standard_normal(n) + 1j * rng.standard_normal(n)).astype(np.complex64), t.sigmas[X])
+        if split:
+            plan.set_split(split)
+        plan.set_cta(0, 0, va, 0)
+        out = plan.compute(t.templates())
+        plan.sync()
+        want = out.clone()
+        plan.set_wait_limit(0)
+        plan.compute(t.templates(), out=out)
+        with pytest.raises(pkg.FstatError) as e:
+            plan.sync()
+        assert e.value.code == TIMEOUT
+        assert bool(torch.isnan(out).all())
+        plan.set_wait_limit(-1)
+        plan.compute(t.templates(), out=out)
+        plan.sync()
+        assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("log2_n", [10, 15, 18])
+def test_noalloc_call_that_gave_up_says_so(log2_n):
+    # no plan and no fstat_sync there: NaN in every bin, and the caller's status word
+    import ctypes
+
+    import torch
+
+    lib = pkg.load()
+    n = (1 << log2_n) * 5 // 8 + 1
+    g = torch.randn((n, 4), device="cuda", generator=torch.Generator(device="cuda").manual_seed(4))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.zeros(1 << log2_n, device="cuda")
+
+    def call(polls, word):
+        assert 0 == lib.fstat_twoF_noalloc_status(
+            ctypes.c_void_p(g.data_ptr()), n, 1 << log2_n, 1.0, -0.5 * n, 0.7, 0.6, 0.1, 1e-10, 0.0,
+            ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(word.data_ptr() if word is not None else 0), polls,
+            ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        torch.cuda.synchronize()
+
+    call(-1, status)
+    want = out.clone()
+    assert status.item() == 0 and bool(torch.isfinite(want).all())
+    call(0, status)
+    assert status.item() == TIMEOUT and bool(torch.isnan(out).all())
+    call(-1, status)
+    assert status.item() == TIMEOUT and torch.equal(out, want)   # kept until the caller clears it
+    call(0, None)
+    assert bool(torch.isnan(out).all())

@@ -144,17 +144,19 @@ struct alignas(32) SkyNode {
 };
 // The same nodes for the FP32 (mixed-precision) path: v = vi + vf with
 // vi = rint(v) exact and |vf| <= 1/2 in FP32, dv = v(next node) - v (small:
-// the delay's change over a node step), a, b in FP32; and the step-iii
-// phase f_h t_m at the detector-time node as its fraction phf (|phf| <= 1/2)
-// and its change to the next node dph (about a cycle at most), both formed in
-// FP64.
-// inner: the step that starts at this node is a whole one and every sample of it
-// certainly valid (k0 inside the data), from the delays of the cubic's four
-// nodes with room for its overshoot.
+// the delay's change over a node step), a, b in FP32; and the step-iii phase
+// f_h t_m at the detector-time node, formed in FP64: ph its fraction and rate its
+// change per sample up to the next node in units of 2^-32 cycles (both modulo a
+// cycle, so that a sample's multiple of rate is exact), curv the change from that
+// step's phase difference to the next step's, in half cycles (~1e-4).
+// vi_inner = 2 vi + inner; inner: the step that starts at this node is a whole
+// one and every sample of it certainly valid (k0 inside the data), from the
+// delays of the cubic's four nodes with room for its overshoot.
 struct alignas(32) NodeF32 {
   float a, b, vf, dv;
-  int vi, inner;
-  float phf, dph;
+  int vi_inner;
+  unsigned ph, rate;
+  float curv;
 };
 // Samples between timing nodes, 4 .. 64 (a resampling block holds whole steps):
 // the most for which a step lasts at most 32 s of the Earth's rotation, over

@@ -226,6 +226,9 @@ k_tmpl_coef(const __grid_constant__ CoefJob job, double j_ref, double dt, int64_
 // Each block computes three nodes more than it stores, for the changes to the
 // next node and the inner mark (NodeF32).
 constexpr int kNodeThreads = 128, kNodeOut = kNodeThreads - 3;
+// 1.5 2^20: added to a phase below 2^19 cycles it leaves the fraction in units of
+// 2^-32 cycles, modulo a cycle, in the low word
+constexpr double kTurns32 = 1572864.0;
 __global__ void __launch_bounds__(kNodeThreads)
 k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
   __shared__ double s_v[kNodeThreads], s_tm[kNodeThreads];
@@ -276,19 +279,21 @@ k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
   NodeF32 f;
   f.a = (float)nd.a;
   f.b = (float)nd.b;
-  f.vi = vi;
   f.vf = (float)(nd.v - (double)vi);
   f.dv = next ? (float)(s_v[t + 1] - nd.v) : 0.f;
   const double ph = g.f_het * nd.tm_det;
-  f.phf = (float)(ph - rint(ph));
-  f.dph = next ? (float)(g.f_het * (s_tm[t + 1] - nd.tm_det)) : 0.f;
-  f.inner = 0;
+  const double d0 = next ? g.f_het * (s_tm[t + 1] - nd.tm_det) : 0.0;
+  f.ph = (unsigned)__double2loint((ph - rint(ph)) + kTurns32);
+  f.rate = (unsigned)__double2loint(fma(d0, __hiloint2double((1023 - g.node_log2) << 20, 0), kTurns32));  // d0 / step
+  f.curv = m + 2 < g.n_nodes ? 2.f * (float)fma(g.f_het, s_tm[t + 2] - s_tm[t + 1], -d0) : 0.f;
+  bool inner = false;
   if (m >= 1 && m + 2 < g.n_nodes) {
     const int lo = min(min(s_vi[t - 1], vi), min(s_vi[t + 1], s_vi[t + 2]));
     const int hi = max(max(s_vi[t - 1], vi), max(s_vi[t + 1], s_vi[t + 2]));
     // (a whole step of SSB samples, and all of their positions in the data)
-    f.inner = hi - lo <= 4 && ji + step <= (int)g.n && ji + lo >= 3 && ji + (step - 1) + hi <= (int)g.n - 4;
+    inner = hi - lo <= 4 && ji + step <= (int)g.n && ji + lo >= 3 && ji + (step - 1) + hi <= (int)g.n - 4;
   }
+  f.vi_inner = 2 * vi + (inner ? 1 : 0);
   g.nodes32[i] = f;
 }
 
@@ -365,16 +370,19 @@ __device__ __forceinline__ typename C2<T>::type z_sample(const Geo& g, int X, co
     }
   }
   if constexpr (sizeof(T) == sizeof(float) && !kNegCtrlFp32) {
-    // the phase's fraction from the FP32 node image (the cubic written about
-    // the step's node)
+    // The cubic through the four nodes written about the step's own one: with the
+    // phase differences d of this step and of its neighbours, the weights sum to
+    // ph + (r / step) d + w3 (d_next - d) - w0 (d_prev - d).  The first two terms in
+    // integers modulo a cycle (exact but for rate's rounding, 63/2 units = 7e-9
+    // cycles), the rest is ~1e-4 cycles.  In FP32 throughout d's rounding alone was
+    // 3e-7 rad at 490 Hz and 64 samples a step, and grew with f_h.
     const float* wf = s_wf[r];
     const NodeF32* nf = g.nodes32 + m;
-    const float2 q = *reinterpret_cast<const float2*>(&nf[0].phf);
-    const float d0 = q.y;
-    float p = q.x + ((wf[2] * d0 + wf[3] * (d0 + nf[1].dph)) - wf[0] * nf[-1].dph);
-    p = __fsub_rn(p, __fsub_rn(__fadd_rn(p, 12582912.f), 12582912.f));  // p - rint(p)
+    const int4 q = *reinterpret_cast<const int4*>(&nf[0].vi_inner);  // vi_inner, ph, rate, curv
+    const float p = fmaf((float)(int)((unsigned)q.y + (unsigned)r * (unsigned)q.z), (float)(1.0 / 2147483648.0),
+                         fmaf(wf[3], __int_as_float(q.w), wf[0] * nf[-1].curv));  // half turns
     float sn, cs;
-    sincospif(2.0f * p, &sn, &cs);
+    sincospif(p, &sn, &cs);
     return make_float2(xrf * cs + xif * sn, xif * cs - xrf * sn);
   } else {
     const double* w = s_w[r];
@@ -438,12 +446,12 @@ __device__ __forceinline__ void series_taps(int D, const TZ* wp, float d, float 
 // (k0 is held within 2^29: far outside the data, and invalid all the same.)
 template <typename T> constexpr bool kWide = sizeof(T) == sizeof(double) || kNegCtrlFp32;
 __device__ __forceinline__ int far_out(int k0) { return max(-(1 << 29), min(1 << 29, k0)); }
-__device__ __forceinline__ int position(int j, float vf, float dvm, float dv, float dvp, int vi, const float* wf, float* dlt) {
+__device__ __forceinline__ int position(int j, float vf, float dvm, float dv, float dvp, int vi_inner, const float* wf, float* dlt) {
   // (explicit operations: sample blocks and sums decide alike which samples are valid)
   const float f = __fadd_rn(vf, __fmaf_rn(wf[2], dv, __fmaf_rn(wf[3], __fadd_rn(dv, dvp), __fmul_rn(-wf[0], dvm))));
   const float big = __fadd_rn(f, 12582912.f);  // 1.5 2^23 + rint(f)
   *dlt = __fsub_rn(f, __fsub_rn(big, 12582912.f));
-  return far_out(j + vi + (__float_as_int(big) - 0x4b400000));
+  return far_out(j + (vi_inner >> 1) + (__float_as_int(big) - 0x4b400000));
 }
 template <typename T>
 __device__ __forceinline__ int position(int j, const SkyNode* nd, const double* wn, T* dlt) {
@@ -479,7 +487,7 @@ __device__ __noinline__ void sum_abc(const Geo& g, int b, int nb, const Partials
     const int X = is / steps, sg = is - X * steps;
     const SkyNode* nd = g.nodes + X * g.n_nodes + sg + 1;
     const NodeF32* nf = g.nodes32 + X * g.n_nodes + sg + 1;
-    const bool inner = nf[0].inner;
+    const bool inner = nf[0].vi_inner & 1;
     if (inner && part > 0) continue;
     const double av[4] = {nd[-1].a, nd[0].a, nd[1].a, nd[2].a};
     const double bv[4] = {nd[-1].b, nd[0].b, nd[1].b, nd[2].b};
@@ -506,7 +514,7 @@ __device__ __noinline__ void sum_abc(const Geo& g, int b, int nb, const Partials
         int k0;
         T dlt;
         if constexpr (kWide<T>) k0 = position<T>(j, nd, wn, &dlt);
-        else k0 = position(j, nf[0].vf, nf[-1].dv, nf[0].dv, nf[1].dv, nf[0].vi, tab->wf[r], &dlt);
+        else k0 = position(j, nf[0].vf, nf[-1].dv, nf[0].dv, nf[1].dv, nf[0].vi_inner, tab->wf[r], &dlt);
         if (j >= g.n || k0 < 0 || k0 > g.n - 1) continue;
         const double a = wn[0] * av[0] + wn[1] * av[1] + wn[2] * av[2] + wn[3] * av[3];
         const double c = wn[0] * bv[0] + wn[1] * bv[1] + wn[2] * bv[2] + wn[3] * bv[3];
@@ -629,7 +637,7 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
         const NodeF32* nf = g.nodes32 + X * g.n_nodes + node_j;
         auto abvd = [&](int q) { return *reinterpret_cast<const float4*>(&nf[q]); };  // a, b, vf, dv
         const float4 m1 = abvd(-1), z0 = abvd(0), p1 = abvd(1), p2 = abvd(2);
-        k0 = position(j, z0.z, m1.w, z0.w, p1.w, nf[0].vi, wf, &dlt);
+        k0 = position(j, z0.z, m1.w, z0.w, p1.w, nf[0].vi_inner, wf, &dlt);
         // the antenna patterns at T, weighted
         const float wx = g.wf[X];
         was[X] = wx * (wf[0] * m1.x + wf[1] * z0.x + wf[2] * p1.x + wf[3] * p2.x);

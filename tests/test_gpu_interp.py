@@ -82,3 +82,28 @@ def test_series_lengths_and_node_steps_match_oracle(n, dt, dterms, dtype, precis
             assert np.abs(gb - ref["Gb"]).max() <= tol * scale
             for k, v in zip("ABCD", abcd):
                 assert abs(v - ref[k]) <= 1e-10 * abs(ref[k]) + 1e-12
+
+
+@pytest.mark.parametrize("f_het,dt", [(490.0, 0.25), (490.0, 0.5), (490.0, 2.0), (2000.0, 0.5), (2000.0, 2.0)])
+def test_heterodyne_phase_of_mixed_plans_at_high_frequencies(f_het, dt):
+    # Step (iii) in mixed plans against FP64 plans: what a non-zero f_h adds to the
+    # rms difference of G (at f_h = 0 only the taps' and the patterns' rounding is
+    # left).  The phase: two FP32 roundings of at most a half turn (6e-8 rad rms
+    # together) and node steps in units of 2^-32 cycles (at most 5e-8 rad); the
+    # sine and cosine 6e-8, the rotation's products and sum 6e-8 each: 1.3e-7 in
+    # all.  It must not grow with f_h or with the node spacing.
+    n = 60001
+    rng = np.random.default_rng(1)
+    x = [(rng.standard_normal(n) + 1j * rng.standard_normal(n)).astype(np.complex64) for _ in range(2)]
+    rms = []
+    for f in (0.0, f_het):
+        t = small_target(n_samples=n, dt=dt, n_fft=1 << 16, n_det=2, seed=5, dtype="c64", f_het=f)
+        g = []
+        for precision in (pkg.MIXED, pkg.FP64):
+            with pkg.FstatPlan.from_target(t, precision) as plan:
+                for X in range(2):
+                    plan.set_data(X, x[X], t.sigmas[X])
+                ga, gb, _ = plan.export_sky(*t.skies[0])
+                g.append(np.concatenate([ga, gb]))
+        rms.append((np.abs(g[0] - g[1]) ** 2).mean() / (np.abs(g[1]) ** 2).mean())
+    assert np.sqrt(max(0.0, rms[1] - rms[0])) <= 2e-7

@@ -769,7 +769,7 @@ int enqueue_compute(fstat_plan* p, const fstat_template* h_tmpl, const int* h_or
         pk.peaks = po->peaks;
         pk.count = po->n_peaks;
         pk.cap = po->n_peaks ? po->capacity : 0;
-        pk.tmpl = (int)(po->tmpl_offset + own);
+        pk.tmpl = po->tmpl_offset + own;
         pk.thr = po->threshold;
         pk.log2_band = log2_band;
       }

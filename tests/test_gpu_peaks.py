@@ -303,3 +303,20 @@ def test_empty_calls_return_without_work():
     assert int(out["count"].item()) == 0
     assert pkg.semicoherent([plan], empty, t.t_reference).shape == (0, t.n_fft)
     plan.close()
+
+
+@pytest.mark.parametrize("n_tmpl", [1, 5])
+def test_template_offsets_beyond_32_bits(n_tmpl):
+    # a search numbers its templates through all its calls: the offset is 64 bits
+    # wide in the request and in the list, whether launches share templates or not
+    t, x, plan = setup(57, n_fft=1 << 13, n=5000)
+    tm = np.repeat(t.templates()[:1], n_tmpl)
+    tm["f1dot"] = np.linspace(-1e-10, 0.0, n_tmpl)
+    off = (1 << 40) + 7
+    near = plan.compute_peaks(tm, threshold=12.0, capacity=1 << 16)
+    far = plan.compute_peaks(tm, threshold=12.0, capacity=1 << 16, tmpl_offset=off)
+    plan.sync()
+    a, b = (np.sort(pkg.peaks_to_numpy(v), order=("tmpl", "bin")) for v in (near, far))
+    assert len(a) > 0 and np.array_equal(a["tmpl"] + off, b["tmpl"])
+    assert np.array_equal(a["bin"], b["bin"]) and np.array_equal(a["twoF"], b["twoF"])
+    plan.close()

@@ -160,13 +160,18 @@ struct alignas(32) NodeF32 {
 };
 // Samples between timing nodes, 4 .. 64 (a resampling block holds whole steps):
 // the most for which a step lasts at most 32 s of the Earth's rotation, over
-// which the cubics below are exact to ~1e-14 s and ~5e-12 in a, b.
-inline int node_step_log2(double dt, double w_rot) {
+// which cubics are exact to ~1e-14 s and ~5e-12 in a, b (four samples, the fewest,
+// pass 32 s above dt = 8 s: the errors grow as the fourth power of the step, to
+// 2e-9 in a, b at 30 s).  FP64 plans, whose series keeps a, b in FP64: at most 16.
+inline int node_step_log2(double dt, double w_rot, int precision) {
+  const int most = precision == FSTAT_FP64 ? 4 : 6;
   int l = 2;
-  while (l < 6 && (2 << l) * dt <= 32.0 && fabs(w_rot) * (2 << l) * dt <= 2.4e-3) ++l;
+  while (l < most && (2 << l) * dt <= 32.0 && fabs(w_rot) * (2 << l) * dt <= 2.4e-3) ++l;
   return l;
 }
-inline int sky_nodes(int64_t n, int step_log2) { return (int)((n + (1 << step_log2) - 1) >> step_log2) + 3; }
+// A step's six nearest nodes begin two steps before it and end three after.
+constexpr int kNodeLead = 2;
+inline int sky_nodes(int64_t n, int step_log2) { return (int)((n + (1 << step_log2) - 1) >> step_log2) + 5; }
 
 // Geometry constants for one plan (kernel argument, by value).
 struct Geo {
@@ -193,7 +198,7 @@ struct Geo {
   // the same grid, [X * tab_n + i] (rewritten by every per-sky run)
   Cubic* tm_tab;
   // Per-sky timing nodes every 2^node_log2 samples (sky.cu), [X * n_nodes + m]
-  // for sample j = (m - 1) 2^node_log2: t_m at the detector time, and at the
+  // for sample j = (m - kNodeLead) 2^node_log2: t_m at the detector time, and at the
   // SSB epoch the delay correction v = u - j and the antenna patterns a, b
   SkyNode* nodes;
   NodeF32* nodes32;                    // the same nodes in FP32 (mixed path)

@@ -489,9 +489,9 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   // timing table over every epoch the timing can reach: the data span
   // widened by the largest delay (|t_m| <= (au + r_earth)/c) plus margin
   {
-    // (and the timing nodes, which extend one node step before the data
+    // (and the timing nodes, which extend two node steps before the data
     // and up to three node steps past it)
-    g.node_log2 = node_step_log2(d.dt, d.ephem.omega_rot);
+    g.node_log2 = node_step_log2(d.dt, d.ephem.omega_rot, d.precision);
     const double step = (double)(1 << g.node_log2);
     const double reach = (d.ephem.au + d.ephem.r_earth) / d.ephem.c + 100.0;
     const double lo = d.t0 - 2.0 * reach - 2.0 * kTabStep - 2.0 * step * d.dt;

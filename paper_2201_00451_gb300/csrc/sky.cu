@@ -82,11 +82,26 @@ __global__ void k_time_table(Geo g, TimeTab* __restrict__ tab) {
   }
 }
 
-__global__ void k_rot_cells(int tab_n, const TimeTab* __restrict__ tab, RotCell* __restrict__ rot) {
+// The rotation's cosine and sine by cubics of their own: about a cell's middle, y in
+// [-Y, Y], cos y = 1 - y^2/2 + y^4/24 and sin y = y - y^3/6 with y^4 replaced by
+// Y^2 y^2 - Y^4/8 (its best lower approximation): 8e-15 at 30 s, where the cubics
+// through four entries leave 5e-13 of one sign, and 1.4e-12 of A and B.
+__global__ void k_rot_cells(Geo g, RotCell* __restrict__ rot) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < 1 || i > tab_n - 3) return;
-  const TimeTab a = tab[i - 1], b = tab[i], c = tab[i + 1], d = tab[i + 2];
-  rot[i] = RotCell{cubic_through(a.cq, b.cq, c.cq, d.cq), cubic_through(a.sq, b.sq, c.sq, d.sq)};
+  if (i < 1 || i > g.tab_n - 3) return;
+  const double x = g.w_rot / g.tab_inv_h, Y = 0.5 * x, t = g.tab_t0 + ((double)i + 0.5) / g.tab_inv_h;
+  double S, C;
+  sincos(g.sid_ph0 + g.w_rot * t, &S, &C);
+  const double e0 = 1.0 - Y * Y * Y * Y / 192.0, e2 = Y * Y / 24.0 - 0.5;
+  auto cubic = [&](double k0, double k1, double k2, double k3) {  // in y = x f - Y
+    Cubic c;
+    c.c0 = k0 - Y * (k1 - Y * (k2 - Y * k3));
+    c.c1 = x * (k1 - Y * (2.0 * k2 - 3.0 * Y * k3));
+    c.c2 = x * x * (k2 - 3.0 * Y * k3);
+    c.c3 = x * x * x * k3;
+    return c;
+  };
+  rot[i] = RotCell{cubic(C * e0, -S, C * e2, S / 6.0), cubic(S * e0, C, S * e2, -C / 6.0)};
 }
 
 // t_m = (r_orb + r_rot) . n / c at every entry and the cubics between them, for
@@ -145,7 +160,8 @@ constexpr int kMaxStep = 64, kMaxD = 32;
 // weights by j mod step, the step matrix M of A, B, C, the taps' constants.
 struct ResTab {
   double w[kMaxStep][4], m[4][4];
-  float wf[kMaxStep][4];
+  double fourth;  // see sum_abc
+  alignas(16) float wf[kMaxStep][4];  // (read as float4)
   TapK<float> tf[2 * kMaxD + 1];
   TapK<double> td[2 * kMaxD + 1];
   float2 tt[kMaxD + 1];  // series form, see series_taps
@@ -188,6 +204,14 @@ __global__ void k_resample_table(Geo g, ResTab* t) {
     double m = 0.0;
     for (int r = 0; r < step; ++r) m += t->w[r][i >> 2] * t->w[r][i & 3];
     t->m[i >> 2][i & 3] = m;
+  } else if (i == 16) {
+    double q = 0.0, p = 0.0;
+    for (int r = 0; r < step; ++r) {
+      const double f = (double)r / (double)step;
+      q += (f + 1.0) * f * (f - 1.0) * (f - 2.0) * (1.0 / 24.0);
+      p += f * (1.0 - f);
+    }
+    t->fourth = -2.0 * q / p;
   }
 }
 
@@ -205,7 +229,7 @@ k_tmpl_coef(const __grid_constant__ CoefJob job, double j_ref, double dt, int64_
 }
 
 // Timing nodes of the current sky position (FP64, every 2^node_log2 samples,
-// from one step before sample 0 on): the Roemer delay at the detector time, and
+// from kNodeLead steps before sample 0 on): the Roemer delay at the detector time, and
 // at the SSB epoch t_b^j the detector epoch T (T + t_m(T) = t_b^j: the
 // fixed-point start T0 = t_b - t_m(t_b), for which a linear t_m is enough, then
 // one Newton step; |dt_m/dT| ~ 1e-4 puts T0 within ~0.05 s of the root and
@@ -237,7 +261,7 @@ k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
   const int m = (int)blockIdx.x * kNodeOut + t - 1;  // stored by threads 1 .. kNodeOut
   const bool in = m >= 0 && m < g.n_nodes;
   const int step = 1 << g.node_log2;
-  const int ji = (m - 1) * step;
+  const int ji = (m - kNodeLead) * step;
   const double j = (double)ji;
   const double td = g.t0 + j * g.dt;
   const double tb = s.t_b0 + j * g.dt;
@@ -327,7 +351,9 @@ k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
 // sum_r a(r)^2 is the quadratic form a^T M a with M = sum_r W_r W_r^T
 // (and likewise b^T M b, a^T M b), exact algebra in FP64, one thread per
 // detector and step, in blocks of their own of the same launch, so that the
-// FP64 work runs beside the others' FP32 work.  A launch of its own to add the
+// FP64 work runs beside the others' FP32 work.  Callers read A to D as doubles, of
+// which the cubic leaves 6e-12 at steps of 32 s: the node values take in the fourth
+// difference (sum_abc), to 1e-14.  A launch of its own to add the
 // sums and form the coefficients took 7 to 12 us; sums of the edges' samples by
 // the sample blocks, 4 us more for a fence in every block.
 //
@@ -350,7 +376,7 @@ template <typename T, bool C128>
 __device__ __forceinline__ typename C2<T>::type z_sample(const Geo& g, int X, const void* xh, int c128, int k,
                                                          const double (*s_w)[4], const float (*s_wf)[4]) {
   const int r = k & ((1 << g.node_log2) - 1);
-  const int m = X * g.n_nodes + (k >> g.node_log2) + 1;  // < 2^23
+  const int m = X * g.n_nodes + (k >> g.node_log2) + kNodeLead;  // < 2^25
   double xr, xi;
   float xrf = 0.f, xif = 0.f;
   if (C128 && c128) {
@@ -485,12 +511,23 @@ __device__ __noinline__ void sum_abc(const Geo& g, int b, int nb, const Partials
   for (int i = b * kSkyBlock + t; i < kStepParts * total; i += nb * kSkyBlock) {
     const int part = i / total, is = i - part * total;
     const int X = is / steps, sg = is - X * steps;
-    const SkyNode* nd = g.nodes + X * g.n_nodes + sg + 1;
-    const NodeF32* nf = g.nodes32 + X * g.n_nodes + sg + 1;
+    const SkyNode* nd = g.nodes + X * g.n_nodes + sg + kNodeLead;
+    const NodeF32* nf = g.nodes32 + X * g.n_nodes + sg + kNodeLead;
     const bool inner = nf[0].vi_inner & 1;
     if (inner && part > 0) continue;
-    const double av[4] = {nd[-1].a, nd[0].a, nd[1].a, nd[2].a};
-    const double bv[4] = {nd[-1].b, nd[0].b, nd[1].b, nd[2].b};
+    // the six nearest nodes: their mean fourth difference d adds d q(f) to the cubic,
+    // q = (f+1) f (f-1) (f-2) / 24, which c f (1 - f) with the same sum over a step
+    // stands for (to 2e-13 of a, b at a sample), a change of the outer nodes by -2 c d
+    auto node_values = [&](double n0, double n1, double n2, double n3, double n4, double n5, double* v) {
+      const double d = tab->fourth * (0.5 * ((n0 + n5) - 3.0 * (n1 + n4)) + (n2 + n3));
+      v[0] = n1 + d;
+      v[1] = n2;
+      v[2] = n3;
+      v[3] = n4 + d;
+    };
+    double av[4], bv[4];
+    node_values(nd[-2].a, nd[-1].a, nd[0].a, nd[1].a, nd[2].a, nd[3].a, av);
+    node_values(nd[-2].b, nd[-1].b, nd[0].b, nd[1].b, nd[2].b, nd[3].b, bv);
     double aa = 0.0, bb = 0.0, ab = 0.0;
     if (inner) {
 #pragma unroll
@@ -625,7 +662,7 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
     const int j0 = tile * kSkyBlock;
     const int j = j0 + (int)threadIdx.x;
     const int j_last = min(j0 + kSkyBlock, (int)g.n) - 1;
-    const int node_j = (min(j, j_last) >> step_log2) + 1;
+    const int node_j = (min(j, j_last) >> step_log2) + kNodeLead;
     int k0s[kMaxDet];
     T dlts[kMaxDet], was[kMaxDet], wbs[kMaxDet];
 #pragma unroll
@@ -764,7 +801,7 @@ int time_table_entries(double t_lo, double t_hi, double h) {
 cudaError_t launch_time_table(const Geo& g, TimeTab* tab, RotCell* rot, cudaStream_t st) {
   const int blocks = (g.tab_n + 255) / 256;
   k_time_table<<<blocks, 256, 0, st>>>(g, tab);
-  k_rot_cells<<<blocks, 256, 0, st>>>(g.tab_n, tab, rot);
+  k_rot_cells<<<blocks, 256, 0, st>>>(g, rot);
   return cudaGetLastError();
 }
 
@@ -812,8 +849,11 @@ int sample_blocks(int64_t n) {
   const int64_t per = std::min<int64_t>(8, std::max<int64_t>(1, tiles / full));
   return (int)((tiles + per - 1) / per);
 }
-// blocks for the step sums, at most as many as the last one has threads to add
-int step_blocks(int64_t n) { return (int)std::min<int64_t>(std::min(device_sm_count(), kSkyBlock), n / (16 / kStepParts * kSkyBlock) + 1); }
+// Blocks for the step sums, at most as many as the last one has threads to add: one
+// per 256 samples, since an SM takes 16 cycles per FP64 warp instruction and a
+// block's eight warps wait for one another (3001 samples, whole call: 52.8 us with a
+// block per 1024 samples, 47.3 so).
+int step_blocks(int64_t n) { return (int)std::min<int64_t>(std::min(device_sm_count(), kSkyBlock), n / 256 + 1); }
 }  // namespace
 
 size_t sky_partials_bytes(int64_t n) { return 16 + (size_t)step_blocks(n) * 3 * sizeof(double); }

@@ -107,3 +107,24 @@ def test_heterodyne_phase_of_mixed_plans_at_high_frequencies(f_het, dt):
                 g.append(np.concatenate([ga, gb]))
         rms.append((np.abs(g[0] - g[1]) ** 2).mean() / (np.abs(g[1]) ** 2).mean())
     assert np.sqrt(max(0.0, rms[1] - rms[0])) <= 2e-7
+
+
+@pytest.mark.parametrize("precision", [pkg.MIXED, pkg.FP64])
+@pytest.mark.parametrize("n,dt", [(100, 0.5), (3001, 2.0), (20001, 0.25), (60001, 0.5), (40001, 1.0), (9001, 4.0), (4001, 8.0)])
+def test_antenna_integrals_to_fp64_rounding(n, dt, precision):
+    # A, B, C are doubles in both precisions.  Against the oracle's FP64 sums: the
+    # patterns' angles round to ~2^-53 times a few turns on both sides (1e-15), the
+    # interpolant through six nodes 32 s apart leaves 1e-15 of the largest pattern,
+    # and sums of n <= 60001 positive terms round to well below n^(1/2) 2^-53 = 3e-14
+    # (C: of products bounded by (A B)^(1/2)); 1e-13 in all.  Four nodes leave 6e-12.
+    t = small_target(n_samples=n, dt=dt, n_fft=1 << max(10, (n - 1).bit_length()), n_det=2, seed=n, dtype="c64")
+    x = [np.ones(n, np.complex64)] * 2
+    with pkg.FstatPlan.from_target(t, precision) as plan:
+        for X in range(2):
+            plan.set_data(X, x[X], t.sigmas[X])
+        for a, d in ((0.3, -0.6), (3.6, 0.2)):
+            ref = resamp.sky_prep(t, [v.astype(np.complex128) for v in x], a, d)
+            A, B, C, _ = plan.export_sky(a, d)[2]
+            assert abs(A - ref["A"]) <= 1e-13 * ref["A"]
+            assert abs(B - ref["B"]) <= 1e-13 * ref["B"]
+            assert abs(C - ref["C"]) <= 1e-13 * np.sqrt(ref["A"] * ref["B"])

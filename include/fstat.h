@@ -338,7 +338,14 @@ int fstat_get_residency(const fstat_plan* plan, int* ra, int* rb);
  * intermediate (16 B per point in FP32), so the FFT passes of consecutive
  * templates overlap.  Without this call: two above n_fft = 2^21; FP32 plans up
  * to there hand several templates to one launch, on one stream up to 2^16 and
- * two above; FP64 plans use four up to 2^19, else two.  Synchronises. */
+ * two above; FP64 plans use four up to 2^19, else two.  A call with four (two
+ * above 2^19) restores that default.
+ * Memory: a plan starts with four intermediates up to 2^19, else two; the first
+ * call with more templates of one sky position (or fstat_autotune) replaces them by
+ * the block that shared launches use, 2^22 / n_fft intermediates but 4 to 32 of them
+ * (64 MB from 2^17 to 2^20 points, 128 MB at 2^21), or keeps what it has where there
+ * is no room.  A plan set to another count of streams before that never takes the block.
+ * Synchronises. */
 int fstat_set_streams(fstat_plan* plan, int n);
 
 /* Persistent launch of the template loop (Sec. 3 template loop; the paper

@@ -58,10 +58,13 @@ struct fstat_plan {
   // templates overlap
   static constexpr int kMaxStreams = 8;
   int nstream = 2;
-  // FP32 plans: templates share launches, over up to n_z intermediates one
-  // behind the other from Z on (see template_batch); 1: as many as streams
-  int n_z = 1;
-  bool batched = false;
+  // n_z intermediates one behind the other from Z on.  batched (FP32 plans):
+  // templates share launches over them (see template_batch), and the first call
+  // with enough templates takes more (grow_z, once); captured: a batch holds their
+  // addresses, so that the block before that stays (old_z)
+  int n_z = 0;
+  bool batched = false, grown = false, captured = false;
+  std::vector<void*> old_z;
   void* Zs[kMaxStreams] = {};      // Zs[0] aliases Z, Zs[k < n_z] lie in its block
   cudaStream_t side[kMaxStreams] = {};
   cudaEvent_t fork = nullptr;
@@ -170,6 +173,7 @@ void free_all(fstat_plan* p) {
     if (p->side[k]) cudaStreamDestroy(p->side[k]);
     if (p->join[k]) cudaEventDestroy(p->join[k]);
   }
+  for (void* z : p->old_z) cudaFree(z);
   if (p->fork) cudaEventDestroy(p->fork);
   if (p->partials) cudaFree(p->partials);
   if (p->rtab) cudaFree(p->rtab);
@@ -230,33 +234,54 @@ EventPair get_events(fstat_plan* p) {
   return e;
 }
 
-// Intermediates.  One pass of one short transform leaves most of the GPU idle and
-// lasts as long as its chain of loads, barriers and stores (~8 us), so FP32
-// plans give one launch several templates where their intermediates stay in
-// L2 (64 MB; 128 MB at 2^21, where the block is one of two per stream).  Above
-// 2^21 a template fills the GPU, and two streams overlap consecutive passes.
-int z_wanted(int64_t n_fft) {
+// Intermediates.  A plan starts with one per template stream.  One pass of one
+// short transform leaves most of the GPU idle and lasts as long as its chain of
+// loads, barriers and stores (~8 us), so FP32 plans give one launch several
+// templates where their intermediates stay in L2 (64 MB; 128 MB at 2^21, where the
+// block is one of two per stream): at the first call whose launches would take
+// more than there are, since a process may hold many plans with small banks.
+// Above 2^21 a template fills the GPU, and two streams overlap consecutive passes.
+int z_shared(int64_t n_fft) {
   if (n_fft > (int64_t(1) << 21)) return 2;
   return (int)std::min<int64_t>(32, std::max<int64_t>(4, (int64_t(1) << 22) / n_fft));
 }
+// where templates do not share launches (FP64, segment sums): four template
+// streams up to n_fft = 2^19 (2^18 runs 1.6x faster with four than with two),
+// two above (2^21: four are 8% slower)
+int default_streams(int64_t n_fft) { return n_fft <= (int64_t(1) << 19) ? 4 : 2; }
+// streams of launches that share templates (template_batch)
+int shared_streams(int64_t n_fft) { return n_fft <= (int64_t(1) << 16) ? 1 : 2; }
 
-cudaError_t alloc_z(fstat_plan* p) {
+cudaError_t alloc_z(fstat_plan* p, int n) {
   const size_t one = (size_t)p->d.n_fft * p->pair_bytes;
-  cudaError_t e = cudaErrorMemoryAllocation;
-  // (a plan with a cap on its memory keeps what one template per stream takes)
-  if (p->d.precision != FSTAT_FP64 && !p->alloc_cap) {
-    const int n = z_wanted(p->d.n_fft);
-    e = palloc(p, &p->Z, n * one);
-    if (e == cudaSuccess) {
-      p->n_z = n;
-      p->batched = true;
-    } else {
-      cudaGetLastError();
-    }
-  }
-  if (e != cudaSuccess) e = palloc(p, &p->Z, one);
-  for (int k = 0; k < p->n_z && k < fstat_plan::kMaxStreams && e == cudaSuccess; ++k) p->Zs[k] = (char*)p->Z + k * one;
+  void* z = nullptr;
+  const cudaError_t e = palloc(p, &z, n * one);
+  if (e != cudaSuccess) return e;
+  p->Z = z;
+  p->n_z = n;
+  for (int k = 0; k < n && k < fstat_plan::kMaxStreams; ++k) p->Zs[k] = (char*)z + k * one;
   return e;
+}
+
+// Intermediates for groups of n templates of one sky position.  The plan keeps
+// what it has where there is no memory for more (and a plan with a cap on its
+// memory never takes more).
+int grow_z(fstat_plan* p, int64_t n) {
+  const int ns = shared_streams(p->d.n_fft), most = z_shared(p->d.n_fft);
+  if (!p->batched || p->grown || p->alloc_cap || std::min<int64_t>(most, ns * ((n + ns - 1) / ns)) <= p->n_z)
+    return FSTAT_OK;
+  CK(cudaDeviceSynchronize());
+  void* own[fstat_plan::kMaxStreams] = {p->Z};  // the block, and what other calls added to it
+  for (int k = p->n_z; k < fstat_plan::kMaxStreams && k < most; ++k) own[k] = p->Zs[k];
+  p->grown = true;
+  if (alloc_z(p, most) != cudaSuccess) {
+    cudaGetLastError();
+    return FSTAT_OK;
+  }
+  for (void* z : own)
+    if (z && p->captured) p->old_z.push_back(z);
+    else if (z) cudaFree(z);
+  return FSTAT_OK;
 }
 
 // Templates per launch of a group of n, and the streams that the launches rotate
@@ -278,7 +303,7 @@ int template_batch(const fstat_plan* p, const int* ord, int64_t n, int64_t ring,
       if (ord[k] != ord[k - 1] + 1) *streams = 1;
   }
   if (!p->batched) return 1;
-  const int ns = p->d.n_fft <= (int64_t(1) << 16) ? 1 : 2;
+  const int ns = shared_streams(p->d.n_fft);
   int T = (int)std::min<int64_t>(p->n_z / ns, (n + ns - 1) / ns);
   if (ring) {
     while (T & (T - 1)) T &= T - 1;
@@ -475,15 +500,12 @@ int fstat_plan_create(const fstat_plan_desc* desc, fstat_plan** out) {
   // whole columns of whole residues: up to N1 RL <= 2^12 x 16 pairs of padding
   if (e == cudaSuccess)
     e = palloc(p, &p->G, (size_t)(N + (int64_t(1) << (kMaxLog2 + (d.precision == FSTAT_FP64 ? 0 : 4)))) * p->pair_bytes);
-  if (e == cudaSuccess) e = alloc_z(p);
+  p->nstream = default_streams(d.n_fft);
+  p->batched = d.precision != FSTAT_FP64 && !p->alloc_cap;
+  if (e == cudaSuccess) e = alloc_z(p, p->nstream);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
-  // where templates do not share launches (FP64, segment sums): four template
-  // streams up to n_fft = 2^19 (2^18 runs 1.6x faster with four than with two),
-  // two above (2^21: four are 8% slower)
-  p->nstream = d.n_fft <= (int64_t(1) << 19) ? 4 : 2;
   for (int k = 1; k < p->nstream && e == cudaSuccess; ++k) {
-    if (!p->Zs[k]) e = palloc(p, &p->Zs[k], (size_t)d.n_fft * p->pair_bytes);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side[k], cudaStreamNonBlocking);
+    e = cudaStreamCreateWithFlags(&p->side[k], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join[k], cudaEventDisableTiming);
   }
   // timing table over every epoch the timing can reach: the data span
@@ -739,7 +761,9 @@ int enqueue_compute(fstat_plan* p, const fstat_template* h_tmpl, const int* h_or
     const fstat_template& t0 = h_tmpl[h_ord[i]];
     int64_t j = i + 1;
     while (j < n && h_tmpl[h_ord[j]].alpha == t0.alpha && h_tmpl[h_ord[j]].delta == t0.delta) ++j;
-    int rc = run_group(p, t0, force_sky, CoefJob{d_tmpl, d_ord, (int)i, (int)(j - i), spin_spacing(p), d_coef}, st);
+    int rc = po || !(p->fused && fused_ok(p)) ? grow_z(p, j - i) : FSTAT_OK;
+    if (rc) return rc;
+    rc = run_group(p, t0, force_sky, CoefJob{d_tmpl, d_ord, (int)i, (int)(j - i), spin_spacing(p), d_coef}, st);
     if (rc) return rc;
     if (!po && p->fused && fused_ok(p)) {
       rc = enqueue_fused(p, i, j, d_ord, d_coef, twoF, out_rows, st, prof);
@@ -1253,7 +1277,8 @@ int fstat_set_streams(fstat_plan* p, int n) {
     if (!p->join[k]) CK(cudaEventCreateWithFlags(&p->join[k], cudaEventDisableTiming));
   }
   p->nstream = n;
-  p->batched = false;  // one template per launch, over these streams
+  // the default count: as at creation; others: one template per launch, over these streams
+  p->batched = n == default_streams(p->d.n_fft) && p->d.precision != FSTAT_FP64 && !p->alloc_cap;
   return FSTAT_OK;
 }
 
@@ -1471,6 +1496,8 @@ extern "C" int fstat_autotune(fstat_plan* p, void* stream) {
   std::vector<fstat_template> ht(p->h_tmpl, p->h_tmpl + kPipe);
   std::vector<int> ho(p->h_order, p->h_order + kPipe);
   float* out = nullptr;
+  rc = grow_z(p, kPipe);
+  if (rc) return rc;
   int64_t rows = p->batched ? p->n_z : p->nstream;  // a row per template in flight
   if (cudaMalloc(&out, (size_t)rows * p->d.n_fft * sizeof(float)) != cudaSuccess) {
     cudaGetLastError();
@@ -1668,7 +1695,7 @@ int fstat_batch_instantiate(fstat_batch* b, void* stream) {
         cudaEventCreateWithFlags(&x.fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming) != cudaSuccess)
       return fail(FSTAT_ERR_CUDA);
-    // one ordinary run first: sets kernel attributes outside the capture
+    // one ordinary run first: sets kernel attributes and takes memory outside the capture
     rc = enqueue_compute(x.p, x.tmpl.data(), x.ord.data(), n, x.d_tmpl, x.d_ord, x.d_coef, x.twoF, x.out_rows,
                          st, true, false);
     if (rc) return fail(rc);
@@ -1698,7 +1725,10 @@ int fstat_batch_instantiate(fstat_batch* b, void* stream) {
   b->graph = g;
   if (cudaGraphInstantiate(&b->exec, b->graph, 0) != cudaSuccess) return fail(FSTAT_ERR_CUDA);
   cudaGraphGetNodes(b->graph, nullptr, &b->nodes);
-  for (auto& x : b->e) x.p->sky_valid = false;
+  for (auto& x : b->e) {
+    x.p->sky_valid = false;
+    x.p->captured = true;
+  }
   return FSTAT_OK;
 }
 

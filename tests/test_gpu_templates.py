@@ -83,3 +83,83 @@ def test_ring_of_rows_keeps_the_last(log2_n, rows):
         torch.cuda.synchronize()
         for i in range(24 - rows, 24):
             assert torch.equal(out[i % rows], want[i])
+
+
+def test_memory_follows_the_bank():
+    # 2^18 bins: the series' buffers (50 000 samples: 3 MB with padding), tables and
+    # four 4 MB intermediates, 24 MB in all; the 64 MB block only with a larger bank,
+    # in place of the four, and results as before
+    import torch
+
+    n, n_fft = 50_000, 1 << 18
+    t = small_target(n_samples=n, dt=2.0, n_fft=n_fft, n_det=2, seed=7, dtype="c64")
+    rng = np.random.default_rng(7)
+    x = rng.standard_normal((n, 2)).astype(np.float32).view(np.complex64)[:, 0]
+    tm = bank(20, 1, n * 2.0)
+    out = torch.zeros((20, n_fft), dtype=torch.float32, device="cuda")
+
+    def held():
+        torch.cuda.synchronize()
+        return free0 - torch.cuda.mem_get_info()[0]
+
+    def make():
+        plan = pkg.FstatPlan.from_target(t)
+        for X in range(2):
+            plan.set_data(X, x, t.sigmas[X])
+        plan.compute(tm[:4], out=out[:4])
+        return plan
+
+    make().close()  # (modules are loaded)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    with make() as plan:
+        assert held() <= 24 << 20
+        few = out[:4].clone()
+        plan.compute(tm, out=out)
+        assert (64 << 20) < held() <= (24 - 16 + 64) << 20
+        assert torch.equal(out[:4], few)
+        plan.sync()
+
+
+def test_default_stream_count_shares_launches_again():
+    t = small_target(n_samples=20_000, dt=2.0, n_fft=1 << 15, n_det=2, seed=8, dtype="c64")
+    rng = np.random.default_rng(8)
+    x = rng.standard_normal((20_000, 2)).astype(np.float32).view(np.complex64)[:, 0]
+    tm = bank(16, 1, 40_000.0)
+    launches = []
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            plan.set_data(X, x, t.sigmas[X])
+        plan.compute(tm)  # (the per-sky work)
+        for streams in (0, 1, 4):
+            if streams:
+                plan.set_streams(streams)
+            before = plan.launches
+            plan.compute(tm)
+            launches.append(plan.launches - before)
+        plan.sync()
+    assert launches[0] < launches[1] and launches[2] == launches[0]
+
+
+def test_a_captured_batch_keeps_its_intermediates():
+    # a batch of two templates holds the plan's first intermediates; a later call
+    # whose bank takes the larger block leaves them in place
+    import torch
+
+    n = 50_000
+    t = small_target(n_samples=n, dt=2.0, n_fft=1 << 18, n_det=2, seed=9, dtype="c64")
+    rng = np.random.default_rng(9)
+    tm = bank(20, 1, n * 2.0)
+    with pkg.FstatPlan.from_target(t) as plan, pkg.FstatBatch() as batch:
+        for X in range(2):
+            x = rng.standard_normal((n, 2)).astype(np.float32).view(np.complex64)[:, 0]
+            plan.set_data(X, x, t.sigmas[X])
+        out = torch.zeros((2, t.n_fft), dtype=torch.float32, device="cuda")
+        batch.add(plan, tm[:2], out)
+        batch.instantiate()
+        want = plan.compute(tm)
+        out.zero_()
+        batch.launch()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[:2])
+        plan.sync()

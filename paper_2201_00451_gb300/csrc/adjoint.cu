@@ -466,8 +466,11 @@ k_moments(int n_det, int64_t tiles, const float2* __restrict__ xt, const float* 
       const float ra1 = r1x * K.dna[0] + r1y * K.dna[1], rd1 = r1x * K.dnd[0] + r1y * K.dnd[1] + r1z * K.dnd[2];
       ga[1] = rate * ra1 + drate * ra;
       gd[1] = rate * rd1 + drate * rd;
-      ga[2] = 0.5f * rate * (r2x * K.dna[0] + r2y * K.dna[1]);
-      gd[2] = 0.5f * rate * (r2x * K.dnd[0] + r2y * K.dnd[1] + r2z * K.dnd[2]);
+      // the frequency's own curvature, for large second spindowns (read here: kept
+      // over the loop, f2dot costs a spilled register and 1.7 % of the kernel)
+      const float drate2 = 0.5f * *(const volatile float*)&K.f2 * dtau * dtau;
+      ga[2] = 0.5f * rate * (r2x * K.dna[0] + r2y * K.dna[1]) + drate * ra1 + drate2 * ra;
+      gd[2] = 0.5f * rate * (r2x * K.dnd[0] + r2y * K.dnd[1] + r2z * K.dnd[2]) + drate * rd1 + drate2 * rd;
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {  // a, b

@@ -229,3 +229,28 @@ def test_large_spindown_of_a_short_series_matches_oracle():
         v, gr = og.grad(t, x, th)
         assert abs(two_f[i] - v) <= 1e-4 * abs(v) + 1e-3
         assert np.all(np.abs((g[i] - gr) * s)[:2] <= 2e-3 * abs(v) + 2e-3), (g[i] * s, gr * s)
+
+
+@pytest.mark.parametrize("f1dot,f2dot,n", [(-0.04, 0.0, 2501), (0.03, -1e-5, 2501), (-0.1, 2e-4, 801)])
+def test_sky_gradient_at_large_spindowns_matches_oracle(f1dot, f2dot, n):
+    # the large-spindown branch, all four components: over a block the frequency
+    # moves by f1dot tau, and with it dPhi/dalpha and dPhi/ddelta; tolerances as above.
+    # 2F turns within 1e-5 rad of sky here, so the oracle's sky differences are
+    # extrapolated from steps of 2e-8 and 4e-8 (within 2e-4 of smaller steps'; its
+    # default step of 1e-7 is off by up to 0.25)
+    t = small_target(n_samples=n, dt=2.0, n_fft=1 << 13, n_det=2, n_inj=1, rho2_range=(150.0, 150.0), seed=48,
+                     f1dots=(f1dot,), f2dots=(f2dot,), dtype="c128")
+    x = synth.make_data(t)
+    inj = t.injections[0]
+    s = _scales(t)
+    base = np.array([inj.f0, inj.f1dot, inj.alpha, inj.delta])
+    rows = [base, base + 0.4 * s]
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            plan.set_data(X, x[X], t.sigmas[X])
+        two_f, g = (v.cpu().numpy() for v in plan.grad(_cands(rows, f2dot=f2dot)))
+    for i, th in enumerate(rows):
+        (v, g1), (_, g2) = (og.grad(t, x, th, f2dot=f2dot, h_sky=h) for h in (2e-8, 4e-8))
+        gr = (4.0 * g1 - g2) / 3.0
+        assert abs(two_f[i] - v) <= 1e-4 * abs(v) + 1e-3
+        assert np.all(np.abs((g[i] - gr) * s) <= 2e-3 * abs(v) + 2e-3), (g[i] * s, gr * s)

@@ -15,10 +15,12 @@
 // The direct sum over all B bins is issue-bound at B terms per sample;
 // 3600 = 16 x 15 x 15 needs about 46.  Two detectors x 480 SFTs of 3600 bins
 // from pinned memory to 2F of two templates: 9436 us with the direct sums
-// (4205 us of kernel per detector), 737 us here.  A band of prime length
-// keeps the direct sum (4001 bins: 4665 -> 4307 us).
+// (4205 us of kernel per detector), 508 us here.  A band of prime length
+// keeps the direct sum (480 SFTs of 4001 bins from device memory: 4.3 ms).
 
 #include <math.h>
+
+#include <algorithm>
 
 #include "fstat_internal.cuh"
 #include "sft.cuh"
@@ -48,7 +50,9 @@ struct SftPlan {
 // B as a product of radices: primes above max_radix stand alone (direct
 // passes), the rest is packed greedily into the largest radices that divide
 // what is left (few passes; a radix-R butterfly costs ~R multiply-adds per
-// point, a pass one exchange through shared memory).
+// point, a pass one exchange through shared memory).  Direct passes come last, the
+// longest at the end: its outputs go to several CTAs, and it has a shared-memory
+// buffer to spare for the roots.
 SftPlan sft_factors(int B, int max_r) {
   SftPlan p{};
   int rest = B;
@@ -75,6 +79,7 @@ SftPlan sft_factors(int B, int max_r) {
     rest /= r;
   }
   if (p.np == 0) p.r[p.np++] = 1;
+  std::sort(std::stable_partition(p.r, p.r + p.np, [&](int r) { return r <= max_r; }), p.r + p.np);
   return p;
 }
 
@@ -187,13 +192,14 @@ __device__ __forceinline__ void pass_r(const typename C2<T>::type* src, const Ou
 
 // one pass of any length r by its defining sum: kSftOut outputs q of one
 // butterfly per thread share each input; the root index (k step + q B/r) s
-// advances by an exactly reduced step per term.  A band of prime length is
-// one such pass, whose outputs spread over the grid's y
+// advances by an exactly reduced step per term.  The last pass's outputs spread
+// over the grid's y, whose CTAs have all formed the passes before it
 template <typename T>
 __device__ __forceinline__ void pass_direct(const typename C2<T>::type* src, const Out<T>& out, int B, int ns, int r) {
   using V = typename C2<T>::type;
   const int nb = B / r, step = B / (ns * r), groups = (r + kSftOut - 1) / kSftOut;
-  for (int u = blockIdx.y * kSftThreads + threadIdx.x; u < nb * groups; u += kSftThreads * gridDim.y) {
+  const int y = out.last ? blockIdx.y : 0, ny = out.last ? gridDim.y : 1;
+  for (int u = y * kSftThreads + threadIdx.x; u < nb * groups; u += kSftThreads * ny) {
     const int g = u / nb, b = u - g * nb, hi = b / ns, k = b - hi * ns;
     int e[kSftOut], j[kSftOut];
     V y[kSftOut];
@@ -224,7 +230,10 @@ __device__ __forceinline__ void pass_direct(const typename C2<T>::type* src, con
   }
 }
 
-template <typename T, typename TIn>
+// SPARE: the roots do not fit beside the data and the last pass is a direct one, which
+// takes them into the buffer that it does not write (a kernel of its own: the others'
+// pointer to the roots stays fixed, 3 % of 480 SFTs of 3600 bins)
+template <typename T, typename TIn, bool SPARE>
 __global__ void __launch_bounds__(kSftThreads)
 k_sft_to_xh(const TIn* __restrict__ bins, const typename C2<T>::type* __restrict__ roots, int B, SftPlan plan,
             int roots_in_smem, double f_het, double t_start, double t_sft, double inv_m,
@@ -262,6 +271,12 @@ k_sft_to_xh(const TIn* __restrict__ bins, const typename C2<T>::type* __restrict
     const int r = plan.r[p];
     out.last = p + 1 == plan.np;
     out.p = out.last ? xh + (int64_t)s * B : nxt;
+    if constexpr (SPARE)
+      if (out.last) {
+        for (int i = threadIdx.x; i < B; i += kSftThreads) nxt[i] = roots[i];
+        out.roots = nxt;
+        __syncthreads();
+      }
     switch (r) {
 #define FSTAT_SFT_R(R) \
   case R: if constexpr (R <= max_radix<T>()) { pass_r<T, R>(cur, out, B, ns); break; }
@@ -287,17 +302,29 @@ cudaError_t run_sft(const void* bins, int64_t n_sft, int B, double f_het, double
   size_t smem = (size_t)(plan.np > 1 ? 2 : 1) * B * sizeof(V);
   const bool in_smem = smem + (size_t)B * sizeof(V) <= kSftSmemMax;
   if (in_smem) smem += (size_t)B * sizeof(V);
+  const int last = plan.r[plan.np - 1], groups = (last + kSftOut - 1) / kSftOut;
+  const bool direct = last > max_radix<T>();
+  const auto kernel = direct && !in_smem ? k_sft_to_xh<T, TIn, true> : k_sft_to_xh<T, TIn, false>;
   // (the limit belongs to the kernel, not to this call: every call sets the same
   // value, so that none lowers it between another thread's setting and launch)
-  cudaError_t e =
-      cudaFuncSetAttribute(k_sft_to_xh<T, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSftSmemMax);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSftSmemMax);
   if (e != cudaSuccess) return e;
   k_sft_roots<T><<<(B + 255) / 256, 256, 0, st>>>(B, (V*)roots);
-  const bool direct = plan.np == 1 && plan.r[0] > max_radix<T>();
-  const dim3 grid((unsigned)n_sft, direct ? (unsigned)((B + kSftThreads * kSftOut - 1) / (kSftThreads * kSftOut)) : 1);
-  k_sft_to_xh<T, TIn><<<grid, kSftThreads, smem, st>>>((const TIn*)bins, (const V*)roots, B, plan, in_smem,
-                                                                  f_het, t_start, t_sft, 1.0 / (double)m_raw, (V*)xh,
-                                                                  err);
+  // The last pass, where it is a direct one, over as many CTAs per SFT as have
+  // threads for it and, behind other passes (formed by each of them), as the GPU
+  // holds.  us per call, one CTA per SFT with roots that do not fit read from L1 -> so:
+  // 1 SFT of 3998 = 2 x 1999 bins 818 -> 236, of 4193 = 7 x 599 314 -> 99; 1 of 12003 =
+  // 3 x 4001 18400 -> 414, 480 of them 100900 -> 17600 (one direct sum over the whole
+  // band: 449, 405, 1217, 38400).
+  unsigned split = 1;
+  if (direct) {
+    split = (unsigned)(((int64_t)(B / last) * groups + kSftThreads - 1) / kSftThreads);
+    const int64_t room = (int64_t)device_sm_count() * std::max<int64_t>(1, (228 * 1024) / (int64_t)(smem + 1024));
+    if (plan.np > 1) split = (unsigned)std::min<int64_t>(split, std::max<int64_t>(1, room / n_sft));
+  }
+  const dim3 grid((unsigned)n_sft, split);
+  kernel<<<grid, kSftThreads, smem, st>>>((const TIn*)bins, (const V*)roots, B, plan, in_smem, f_het, t_start, t_sft,
+                                          1.0 / (double)m_raw, (V*)xh, err);
   return cudaGetLastError();
 }
 

@@ -182,3 +182,44 @@ def test_two_threads_with_different_band_lengths():
     for job, want in zip(jobs, alone):
         assert np.array_equal(job[0].export_data(0), want)
         job[0].close()
+
+
+@pytest.mark.parametrize("precision,tol", [(pkg.MIXED, 2e-5), (pkg.FP64, 1e-12)])
+@pytest.mark.parametrize("nb,n_sft", [(17 * 2, 1), (31 * 37, 1), (31 * 37, 40), (2 * 1999, 1), (3 * 1999, 5), (6 * 1009, 2),
+                                      (3 * 4001, 1), (3 * 4001, 2), (2 * 17 * 353, 1)])
+def test_bands_with_large_primes(nb, n_sft, precision, tol):
+    # a direct last pass over several CTAs per SFT, behind small or other direct passes,
+    # its roots beside the data or in the spare buffer; tolerances as above
+    if precision == pkg.FP64 and nb > 7040:
+        pytest.skip("beyond the FP64 limit")
+    t_sft = 1800.0
+    q0 = int(100.0 * t_sft) - nb // 2
+    t = small_target(n_samples=n_sft * nb, dt=t_sft / nb, n_fft=1 << max(10, (n_sft * nb - 1).bit_length()), n_det=1,
+                     f_het=100.0, seed=127, dtype="c64")
+    rng = np.random.default_rng(nb)
+    b = (rng.standard_normal((n_sft, nb)) + 1j * rng.standard_normal((n_sft, nb))).astype(np.complex64)
+    ref = sft.xh_from_band(b.astype(np.complex128), q0, t.t0, t_sft, 2 * nb, 100.0)
+    with pkg.FstatPlan.from_target(t, precision) as plan:
+        plan.set_sfts(0, b, q0, t_sft, 2 * nb, 1.0)
+        got = plan.export_data(0)
+    assert np.max(np.abs(got - ref)) <= tol * np.max(np.abs(ref))
+
+
+def test_a_band_with_a_large_prime_costs_no_more_than_a_prime_one():
+    # 3 x 4001 bins hold a third of the terms of the prime 12007: no longer call
+    # (it was 15 times as long with one CTA and its roots in L1)
+    import time
+
+    took = []
+    for nb in (12007, 3 * 4001):
+        t_sft = 1800.0
+        t = small_target(n_samples=nb, dt=t_sft / nb, n_fft=1 << 14, n_det=1, f_het=100.0, seed=128, dtype="c64")
+        b = torch.view_as_complex(torch.randn((1, nb, 2), device="cuda"))
+        with pkg.FstatPlan.from_target(t) as plan:
+            runs = []
+            for _ in range(12):
+                t0 = time.perf_counter()
+                plan.set_sfts(0, b, int(100.0 * t_sft) - nb // 2, t_sft, 2 * nb, 1.0)  # (synchronises)
+                runs.append(time.perf_counter() - t0)
+            took.append(sorted(runs)[len(runs) // 2])
+    assert took[1] <= 1.2 * took[0], took

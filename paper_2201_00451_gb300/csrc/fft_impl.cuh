@@ -119,11 +119,6 @@ template <typename T, int L, int C, int V> struct PeakSmem {
   static constexpr size_t BYTES = KEYS_END + (SEP ? SF : 0);
 };
 
-template <typename T, int L, int C, int V = 0> constexpr bool cfg_ok() {
-  using S = Shape<T, L, V>;
-  return C * S::TPC >= 32 && C * S::TPC <= 1024 && Buf<T, L, C, V>::ONE <= kSmemCap;
-}
-
 // 16-byte asynchronous global -> shared copies (completion tracked by
 // commit groups; cp.async.wait_group is a hardware wait, not a spin loop).
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -504,45 +499,19 @@ template <int R, bool HALF> struct Spin<float, R, HALF> {
     *cs = cv;
     *sn = -sv;
   }
-  __device__ __forceinline__ void next() {}
 };
-// FP64: the same differences as factors, r <- r m, m <- m k, k <- k l, one
-// next() after each sample s = 0, 1, ..  (Up to four samples the polynomial and
-// its sine/cosine are evaluated at each: fewer operations than three starts.)
+// FP64: the polynomial and its sine/cosine at every sample.  (The differences as
+// factors, r <- r m, m <- m k, .., take two thirds of the operations but no less
+// time, 64 templates at 2^18 4013 us against 4014, and leave 1e-15 to 4e-14 where
+// this leaves 3e-17 to 6e-15.)
 template <int R, bool HALF> struct Spin<double, R, HALF> {
-  static constexpr bool EACH = (HALF ? R / 2 : R) <= 4;
-  double2 r, m, k, l;
   const TmplCoef& c;
   int x0, D;
-  static __device__ __forceinline__ double2 turn(double ph) {
-    double2 w;
-    sincospi(-2.0 * (ph - rint(ph)), &w.y, &w.x);
-    return w;
-  }
-  static __device__ __forceinline__ double2 mul(double2 a, double2 b) {
-    return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-  }
-  __device__ __forceinline__ Spin(const TmplCoef& c_, int x0_, int D_) : c(c_), x0(x0_), D(D_) {
-    if constexpr (EACH) return;
-    const double x = (double)x0;
-    r = turn(((c.p[3] * x + c.p[2]) * x + c.p[1]) * x + c.p[0]);
-    m = turn((c.q[2] * x + c.q[1]) * x + c.q[0]);
-    k = turn(c.r[1] * x + c.r[0]);
-    l = {c.c3, c.s3};
-  }
+  __device__ __forceinline__ Spin(const TmplCoef& c_, int x0_, int D_) : c(c_), x0(x0_), D(D_) {}
   __device__ __forceinline__ void rot(int s, double* cs, double* sn) {
-    if constexpr (EACH) {
-      const double x = (double)(x0 + s * D);
-      r = turn(((c.p[3] * x + c.p[2]) * x + c.p[1]) * x + c.p[0]);
-    }
-    *cs = r.x;
-    *sn = r.y;
-  }
-  __device__ __forceinline__ void next() {
-    if constexpr (EACH) return;
-    r = mul(r, m);
-    m = mul(m, k);
-    k = mul(k, l);
+    const double x = (double)(x0 + s * D);
+    const double ph = ((c.p[3] * x + c.p[2]) * x + c.p[1]) * x + c.p[0];
+    sincospi(-2.0 * (ph - rint(ph)), sn, cs);
   }
 };
 
@@ -576,7 +545,6 @@ __device__ __forceinline__ void pass_a_tile(int tile, typename PairMem<T>::type*
       } else {
         v[s] = pzero<T>();
       }
-      spin.next();
     }
   };
   const bool half = (int64_t)n1 * (L / 2) >= (int64_t)n;

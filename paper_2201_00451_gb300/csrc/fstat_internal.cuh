@@ -59,11 +59,11 @@ struct CoefJob {
 //   d2(x) = d1(x + D) - d1(x)       = r0 + r1 x
 //   d3    = d2(x + D) - d2(x)
 // FP32 path: double-float coefficients (hi + lo carries ~48 bits) and d3 in
-// units of 2^-32 cycles; FP64 path: doubles, and exp(-2 pi i d3).
+// units of 2^-32 cycles; FP64 path: phi's coefficients in doubles.
 struct TmplCoef {
   float phi[4][2], d1[3][2], d2[2][2];  // [power][hi, lo]
   int d3, J;
-  double p[4], q[3], r[2], c3, s3;
+  double p[4];
 };
 
 // Spindown phase polynomial of one template (eqs. Fa, Fb: Phi_s =
@@ -72,7 +72,6 @@ struct TmplCoef {
 // [0, n - 1], so |x| <= 2^24 stays exact in FP32 wherever the reference time
 // lies; p0, a phase common to every sample that cancels in 2F, is reduced mod
 // 1, as are the other coefficients (x is an integer) where they reach a cycle.
-template <bool F64>  // with the FP64 path's factor of d3
 __device__ inline TmplCoef spin_coef(double jr, int64_t n, double dt, double f1dot, double f2dot, double D) {
   double J = rint(jr);
   if (!(J >= 0.0)) J = 0.0;
@@ -85,11 +84,8 @@ __device__ inline TmplCoef spin_coef(double jr, int64_t n, double dt, double f1d
   c.p[2] = c2 - 3.0 * c3 * e;
   c.p[1] = -2.0 * c2 * e + 3.0 * c3 * e * e;
   c.p[0] = c2 * e * e - c3 * e * e * e;
-  c.q[0] = D * (c.p[1] + D * (c.p[2] + D * c.p[3]));
-  c.q[1] = D * (2.0 * c.p[2] + D * 3.0 * c.p[3]);
-  c.q[2] = D * 3.0 * c.p[3];
-  c.r[0] = D * D * (2.0 * c.p[2] + D * 6.0 * c.p[3]);
-  c.r[1] = D * D * 6.0 * c.p[3];
+  double d1[3] = {D * (c.p[1] + D * (c.p[2] + D * c.p[3])), D * (2.0 * c.p[2] + D * 3.0 * c.p[3]), D * 3.0 * c.p[3]};
+  double d2[2] = {D * D * (2.0 * c.p[2] + D * 6.0 * c.p[3]), D * D * 6.0 * c.p[3]};
   auto split = [](double* v, float (*f)[2], int m) {
     for (int q = 0; q < m; ++q) {
       if (q == 0 || fabs(v[q]) >= 1.0) v[q] -= rint(v[q]);
@@ -100,11 +96,9 @@ __device__ inline TmplCoef spin_coef(double jr, int64_t n, double dt, double f1d
   double d3 = D * D * D * 6.0 * c.p[3];
   d3 -= rint(d3);
   split(c.p, c.phi, 4);
-  split(c.q, c.d1, 3);
-  split(c.r, c.d2, 2);
+  split(d1, c.d1, 3);
+  split(d2, c.d2, 2);
   c.d3 = (int)(unsigned)(long long)rint(d3 * 4294967296.0);
-  c.c3 = c.s3 = 0.0;
-  if (F64) sincospi(-2.0 * d3, &c.s3, &c.c3);
   c.J = (int)J;
   return c;
 }
@@ -295,7 +289,7 @@ void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* cons
 // kernel that fills them (FP64 sincos, once per plan).
 int time_table_entries(double t_lo, double t_hi, double h);
 cudaError_t launch_time_table(const Geo& g, TimeTab* tab, RotCell* rot, cudaStream_t st);
-void launch_tmpl_coef(const SkyPos& pos, const Geo& g, int precision, const CoefJob& job, cudaStream_t st);
+void launch_tmpl_coef(const SkyPos& pos, const Geo& g, const CoefJob& job, cudaStream_t st);
 // samples between the inputs of one of pass A's first butterflies
 int64_t pass_a_spacing(int log2n, int log2_n2);
 void launch_check_finite(const void* x, int dtype, int64_t n, int* err, cudaStream_t st);

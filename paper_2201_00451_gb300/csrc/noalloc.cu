@@ -83,7 +83,7 @@ __global__ void k_noalloc_setup(const float4* __restrict__ g, int64_t n, int n1,
     g_scratch_sky.kAf = (float)(2.0 * a.A / D);
     g_scratch_sky.kBf = (float)(2.0 * a.B / D);
     g_scratch_sky.kCf = (float)(4.0 * a.C / D);
-    g_scratch_coef = spin_coef<false>(-a.tau0 / a.dt, n, a.dt, a.f1dot, a.f2dot, a.spacing);
+    g_scratch_coef = spin_coef(-a.tau0 / a.dt, n, a.dt, a.f1dot, a.f2dot, a.spacing);
     return;
   }
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)(gridDim.x - 1) * blockDim.x)

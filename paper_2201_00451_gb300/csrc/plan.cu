@@ -341,7 +341,7 @@ int run_sky(fstat_plan* p, double alpha, double delta, const CoefJob& job, cudaS
 int run_group(fstat_plan* p, const fstat_template& t, bool force, const CoefJob& job, cudaStream_t st) {
   if (force || !(p->sky_valid && p->sky_alpha == t.alpha && p->sky_delta == t.delta))
     return run_sky(p, t.alpha, t.delta, job, st);
-  launch_tmpl_coef(p->pos, p->geo, p->d.precision, job, st);
+  launch_tmpl_coef(p->pos, p->geo, job, st);
   ++p->n_launches;
   CK(cudaGetLastError());
   return FSTAT_OK;

@@ -216,16 +216,14 @@ __global__ void k_resample_table(Geo g, ResTab* t) {
 }
 
 // Spindown polynomial of template i of the job (see TmplCoef).
-template <bool F64>
 __device__ __forceinline__ void tmpl_coef(const CoefJob& c, double j_ref, double dt, int64_t n, int i) {
   if (i >= c.count) return;
   const fstat_template tp = c.tmpl[c.order[c.first + i]];
-  c.out[c.first + i] = spin_coef<F64>(j_ref, n, dt, tp.f1dot, tp.f2dot, c.spacing);
+  c.out[c.first + i] = spin_coef(j_ref, n, dt, tp.f1dot, tp.f2dot, c.spacing);
 }
-template <bool F64>
 __global__ void __launch_bounds__(128)
 k_tmpl_coef(const __grid_constant__ CoefJob job, double j_ref, double dt, int64_t n) {
-  tmpl_coef<F64>(job, j_ref, dt, n, (int)blockIdx.x * 128 + (int)threadIdx.x);
+  tmpl_coef(job, j_ref, dt, n, (int)blockIdx.x * 128 + (int)threadIdx.x);
 }
 
 // Timing nodes of the current sky position (FP64, every 2^node_log2 samples,
@@ -627,7 +625,7 @@ k_resample(const __grid_constant__ Geo g, const __grid_constant__ XhArgs xh, typ
   if (block < 0) {
     if ((int)blockIdx.x < sum_blocks) sum_abc<T>(g, (int)blockIdx.x, sum_blocks, part, sky, err);
     else
-      tmpl_coef<sizeof(T) == sizeof(double)>(job, j_ref, g.dt, g.n, ((int)blockIdx.x - sum_blocks) * kSkyBlock + (int)threadIdx.x);
+      tmpl_coef(job, j_ref, g.dt, g.n, ((int)blockIdx.x - sum_blocks) * kSkyBlock + (int)threadIdx.x);
     return;
   }
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -893,10 +891,9 @@ void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* cons
                                                               job, pos.j_ref);
 }
 
-void launch_tmpl_coef(const SkyPos& pos, const Geo& g, int precision, const CoefJob& job, cudaStream_t st) {
+void launch_tmpl_coef(const SkyPos& pos, const Geo& g, const CoefJob& job, cudaStream_t st) {
   if (job.count == 0) return;
-  const auto k = precision == FSTAT_FP64 ? k_tmpl_coef<true> : k_tmpl_coef<false>;
-  k<<<(job.count + 127) / 128, 128, 0, st>>>(job, pos.j_ref, g.dt, g.n);
+  k_tmpl_coef<<<(job.count + 127) / 128, 128, 0, st>>>(job, pos.j_ref, g.dt, g.n);
 }
 
 // Scan an input series for NaN/Inf.

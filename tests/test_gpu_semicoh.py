@@ -125,3 +125,32 @@ def test_argument_checks():
         pkg.semicoherent([plans[0], po], tm, t.t_reference)
     for p in plans + [po]:
         p.close()
+
+
+def test_segments_with_different_splits_and_rows():
+    # all segments use the first plan's intermediates one after the other, each in its
+    # own layout: the sum equals the segments' own rows, slid and added in order
+    S, n_seg, dt, n_fft = 3, 40_001, 1.0, 1 << 16
+    t = small_target(n_samples=S * n_seg, dt=dt, n_fft=n_fft, n_det=2, seed=96, dtype="c64")
+    rng = np.random.default_rng(96)
+    x = [(rng.standard_normal(S * n_seg) + 1j * rng.standard_normal(S * n_seg)).astype(np.complex64) for _ in range(2)]
+    segs, data, plans = _plans(t, S, x)
+    df = 1.0 / (n_fft * dt)
+    tm = np.zeros(5, dtype=pkg.TEMPLATE_DTYPE)
+    tm["alpha"], tm["delta"] = 0.4, -0.3
+    tm["f1dot"] = np.array([-3.0, -1.0, 0.0, 1.0, 2.0]) * df / (n_seg * dt)
+    for p, n1, cb in zip(plans, (32, 2048, 512), (0, 2, 8)):
+        p.set_split(n1)
+        p.set_cta(0, cb, 0, 0)
+    got = pkg.semicoherent(plans, tm, t.t_reference)
+    want = torch.zeros_like(got)
+    for s, (seg, p) in enumerate(zip(segs, plans)):
+        rows = p.compute(tm)
+        for i in range(len(tm)):
+            k = semicoh.segment_shift(df, seg.t_reference - t.t_reference, float(tm["f1dot"][i]), 0.0)
+            lo, hi = max(0, -k), min(n_fft, n_fft - k)
+            want[i, lo:hi] += rows[i, lo + k:hi + k]
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
+    for p in plans:
+        p.close()

@@ -85,6 +85,31 @@ def test_ring_of_rows_keeps_the_last(log2_n, rows):
             assert torch.equal(out[i % rows], want[i])
 
 
+@pytest.mark.parametrize("log2_n", [13, 18, 20])
+@pytest.mark.parametrize("rows", [1, 3])
+def test_ring_of_rows_that_the_streams_do_not_divide(log2_n, rows):
+    # the default plan's own choice for these rings: one template per launch, a row
+    # with one stream
+    import torch
+
+    n = (1 << log2_n) * 5 // 7
+    t = small_target(n_samples=n, dt=2.0, n_fft=1 << log2_n, n_det=2, seed=1, dtype="c64")
+    rng = np.random.default_rng(rows)
+    tm = bank(24, 1, n * 2.0)
+    with pkg.FstatPlan.from_target(t) as plan, pkg.FstatBatch() as batch:
+        for X in range(2):
+            x = rng.standard_normal((n, 2)).astype(np.float32).view(np.complex64)[:, 0]
+            plan.set_data(X, x, t.sigmas[X])
+        out = torch.zeros((rows, t.n_fft), dtype=torch.float32, device="cuda")
+        batch.add(plan, tm, out, out_rows=rows)
+        batch.instantiate()
+        batch.launch()
+        torch.cuda.synchronize()
+        want = plan.compute(tm)
+        for i in range(24 - rows, 24):
+            assert torch.equal(out[i % rows], want[i])
+
+
 def test_memory_follows_the_bank():
     # 2^18 bins: the series' buffers (50 000 samples: 3 MB with padding), tables and
     # four 4 MB intermediates, 24 MB in all; the 64 MB block only with a larger bank,
@@ -163,3 +188,28 @@ def test_a_captured_batch_keeps_its_intermediates():
         torch.cuda.synchronize()
         assert torch.equal(out, want[:2])
         plan.sync()
+
+
+@pytest.mark.parametrize("log2_n,n1,n", [(21, 256, 600_001), (21, 256, 1_400_001), (20, 256, 1_000_003), (20, 1024, 700_001),
+                                          (16, 32, 40_001)])
+def test_staged_columns_and_row_counts_give_the_same_bits(log2_n, n1, n):
+    # every distinct kernel of a split: pass A's columns staged where there is room
+    # (0; 16 and 18 require it at 8192 and 4096 points) and straight into registers
+    # (2), 1 to 8 rows per tile of pass B
+    t = small_target(n_samples=n, dt=1.0, n_fft=1 << log2_n, n_det=2, seed=11, dtype="c64")
+    rng = np.random.default_rng(11)
+    tm = bank(3, 1, float(n))
+    need = {13: 16, 12: 18}.get(log2_n - (n1.bit_length() - 1))
+    got = []
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            x = rng.standard_normal((n, 2)).astype(np.float32).view(np.complex64)[:, 0]
+            plan.set_data(X, x, t.sigmas[X])
+        plan.set_split(n1)
+        for va, cb in [(2, 0), (0, 0)] + ([(need, 0)] if need else []) + ([(2, c) for c in (1, 2, 4, 8)] if n1 >= 512 else []):
+            plan.set_cta(0, cb, va, 0)
+            got.append(plan.compute(tm).cpu().numpy())
+        plan.sync()
+    assert np.isfinite(got[0]).all()
+    for g in got[1:]:
+        assert np.array_equal(g, got[0])

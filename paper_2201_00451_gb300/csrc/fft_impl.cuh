@@ -500,18 +500,33 @@ template <int R, bool HALF> struct Spin<float, R, HALF> {
     *sn = -sv;
   }
 };
-// FP64: the polynomial and its sine/cosine at every sample.  (The differences as
-// factors, r <- r m, m <- m k, .., take two thirds of the operations but no less
-// time, 64 templates at 2^18 4013 us against 4014, and leave 1e-15 to 4e-14 where
-// this leaves 3e-17 to 6e-15.)
+// FP64: the polynomial at every sample, and for columns of 256 points or more its
+// factor as a 256th root of unity (of the column's own table tw) times a turn of at
+// most 1/512, whose Taylor series are cut at 1e-17.  Like sincospi at every sample it
+// leaves 4e-17 to 4e-15 (excursions of 0.005 to 17 cycles); the differences as
+// factors, r <- r m, m <- m k, .., leave 1e-15 to 4e-14.  Eight templates, us, with
+// those, with sincospi and so: 200 001 samples at 2^18 577, 602, 550; 500 001 at 2^20
+// 2274, 2380, 2254; 4 000 001 at 2^22 10749, 11940, 10890.
 template <int R, bool HALF> struct Spin<double, R, HALF> {
   const TmplCoef& c;
   int x0, D;
   __device__ __forceinline__ Spin(const TmplCoef& c_, int x0_, int D_) : c(c_), x0(x0_), D(D_) {}
-  __device__ __forceinline__ void rot(int s, double* cs, double* sn) {
+  template <int L> __device__ __forceinline__ void rot(int s, const double2* __restrict__ tw, double* cs, double* sn) {
     const double x = (double)(x0 + s * D);
     const double ph = ((c.p[3] * x + c.p[2]) * x + c.p[1]) * x + c.p[0];
-    sincospi(-2.0 * (ph - rint(ph)), sn, cs);
+    if constexpr (L < 256) {
+      sincospi(-2.0 * (ph - rint(ph)), sn, cs);
+    } else {
+      constexpr double kRint = 6755399441055744.0;  // 1.5 2^52: adds an integer to the low word
+      constexpr double p = 6.283185307179586, p2 = p * p;
+      const double t = fma(ph, 256.0, kRint);
+      const double r = fma(t - kRint, -1.0 / 256.0, ph), r2 = r * r;  // exact
+      const double2 w = __ldg(tw + (__double2loint(t) & 255) * (L / 256));
+      const double sr = r * fma(r2, fma(r2, p * p2 * p2 / 120.0, -p * p2 / 6.0), p);
+      const double e = r2 * fma(r2, fma(r2, -p2 * p2 * p2 / 720.0, p2 * p2 / 24.0), -p2 / 2.0);  // cosine - 1
+      *cs = fma(w.x, e, fma(w.y, sr, w.x));
+      *sn = fma(w.y, e, fma(-w.x, sr, w.y));
+    }
   }
 };
 
@@ -540,7 +555,8 @@ __device__ __forceinline__ void pass_a_tile(int tile, typename PairMem<T>::type*
       const int n2 = t + s * S::TPC;
       if (col + n1 * n2 < n) {
         T cs, sn;
-        spin.rot(s, &cs, &sn);
+        if constexpr (sizeof(T) == 8) spin.template rot<L>(s, twL, &cs, &sn);
+        else spin.rot(s, &cs, &sn);
         v[s] = pmul(pload(buf + (kDense ? gc.at(n2) : pad_idx(n2, S::PS))), cs, sn);
       } else {
         v[s] = pzero<T>();

@@ -348,3 +348,24 @@ def test_spindown_phase_excursion_beyond_range_is_rejected():
             plan.compute(t.templates())
         assert e.value.code == -7
         plan.sync()
+
+
+@pytest.mark.parametrize("n1", [256, 128, 64, 32])
+@pytest.mark.parametrize("n", [3001, 5003, 8000])
+def test_fp64_spindown_of_every_column_length(n, n1):
+    # columns of 32 to 256 points: the factor from sincospi below 256, from the
+    # column's roots at 256; the lower half of the columns filled or more; some 10
+    # cycles of spindown phase.  FP64 tolerance as above
+    t = small(seed=41, n_samples=n, f1dots=(-3e-7, 1e-8), f2dots=(0.0, 2e-11), dtype="c128")
+    x = synth.make_data(t)
+    tm = t.templates()
+    assert_parity(run_gpu(t, x, tm, precision=pkg.FP64, split=n1), resamp.fstat(t, x, tm), rel=1e-7, abs_=1e-7)
+
+
+@pytest.mark.parametrize("n1,n", [(128, 40_001), (64, 60_001), (32, 65_536), (32, 30_000)])
+def test_fp64_spindown_of_long_columns(n1, n):
+    # 512 to 2048 points, both radices of the first step, whole and ragged
+    t = small(seed=42, n_samples=n, n_fft=1 << 16, f1dots=(-1e-9,), f2dots=(0.0, 1e-14), dtype="c128")
+    x = synth.make_data(t)
+    tm = t.templates()
+    assert_parity(run_gpu(t, x, tm, precision=pkg.FP64, split=n1), resamp.fstat(t, x, tm), rel=1e-7, abs_=1e-7)

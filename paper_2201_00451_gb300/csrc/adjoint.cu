@@ -26,7 +26,7 @@
 // Bound by FP32 issue: ~22 instructions per candidate and sample plus ~480
 // per block.  256 candidates of the 10-day two-detector data: 11.7 ms with the
 // phase, the patterns and 29 sums evaluated at every sample (~300
-// instructions), 1.25 ms here; one candidate 5.2 ms -> 0.14 ms (items of 2^14
+// instructions), 1.19 ms here; one candidate 5.2 ms -> 0.08 ms (items of 2^14
 // samples instead of 2^17 fill the GPU).
 
 #include <math.h>
@@ -245,8 +245,7 @@ __device__ __forceinline__ double pat_sum(const double* u, const double* v, cons
 // A warp per candidate.  The chain of FP64 operations is what this kernel lasts (64 us
 // with a thread per candidate, whatever their number), so the eleven sums of each
 // detector go to lanes of their own.  With k_finalize's CTA per candidate a call for
-// one candidate over 10 days takes 82 us instead of 137, for 256 of them 1183
-// instead of 1246.
+// one candidate over 10 days takes 82 us instead of 137, for 256 of them 63 us less.
 constexpr int kSums = 11;
 __global__ void __launch_bounds__(32)
 k_cand_consts(const __grid_constant__ Geo g, const __grid_constant__ Harmonics h, const fstat_candidate* __restrict__ cand,
@@ -539,8 +538,8 @@ k_moments(int n_det, int64_t tiles, const float2* __restrict__ xt, const float* 
 }
 
 // sum the chunk partials (fixed order) and apply the chain rule in FP64, one
-// warp per candidate; partial[chunk][cand][kAcc]
-// (a CTA per candidate: a warp alone took 30 us for the 211 chunks of 10 days)
+// CTA per candidate (a warp alone took 30 us for the 211 chunks of 10 days);
+// partial[chunk][cand][kAcc]
 __global__ void __launch_bounds__(kWarps * 32)
 k_finalize(const double* __restrict__ partial, const CandConst* __restrict__ cc, int n_cand, int n_chunks,
            float* __restrict__ twoF, float* __restrict__ grad) {

@@ -134,9 +134,10 @@ template <typename PM> __device__ __forceinline__ void cp_pair(PM* dst, const PM
   if constexpr (sizeof(PM) == 32) cp_async16((char*)dst + 16, (const char*)src + 16);
 }
 
-// Bulk tensor copies (TMA) for pass B's tiles: one thread issues a few 2D
-// box copies of the intermediate into shared memory, completion is counted
-// in bytes on an mbarrier, and every thread waits on the barrier's phase.
+// Bulk copies: pass A's staged columns and pass B's tiles (fft_warp.cuh) as
+// contiguous blocks, the persistent launch's pass-B tiles as 2D boxes through a
+// tensor map (TMA).  One thread issues them, completion is counted in bytes on an
+// mbarrier, and every thread waits on the barrier's phase.
 // Each wait gives up after kWaitLimit polls (a GPU that stopped delivering
 // copies must not hang the kernel): it then records FSTAT_ERR_TIMEOUT and
 // the kernel returns.
@@ -439,11 +440,11 @@ __device__ __forceinline__ void store_pass0(const Pair<T>* v, typename PairMem<T
 
 // ----------------------------------------------------- spindown phase
 // e^{-i 2 pi phi} at the samples of one first-pass butterfly, x_s = x0 + s D
-// (TmplCoef).  The polynomial and its first two differences are evaluated once
-// per butterfly, the samples follow by differences: three integer adds, a
-// conversion and a sine/cosine each instead of a double-float cubic.
+// (TmplCoef).
 //
-// FP32: double-float Horner with error-free products and sums (explicitly
+// FP32: the polynomial and its first two differences are evaluated once per
+// butterfly, the samples follow by differences: three integer adds, a conversion
+// and a sine/cosine each instead of a double-float cubic.  Double-float Horner with error-free products and sums (explicitly
 // rounded, so the compiler cannot contract them), then phases modulo a cycle
 // in units of 2^-32, whose adds are exact.  The units' rounding grows with the
 // distance from the sample that the differences start at: at most 1.2e-8

@@ -270,7 +270,7 @@ k_wpass_a(const float4* __restrict__ G, int lcs, int n, int n1, const TmplCoef* 
 }
 
 // ------------------------------------------------------------- pass B
-constexpr int kSubB = 256;  // longest sub-transform of pass B (a tensor copy's box)
+constexpr int kSubB = 256;  // longest sub-transform of pass B
 template <int L, int CB> using WB = WShape<L, CB, kSubB>;
 
 // A tile = CB neighbouring rows k2 = one contiguous block of the intermediate,

@@ -282,7 +282,7 @@ size_t sky_partials_bytes(int64_t n);  // (zeroed once)
 size_t resample_table_bytes();
 cudaError_t launch_resample_table(const Geo& g, struct ResTab* t, cudaStream_t st);
 // Steps (iii)-(v) for one sky position, and the spindown coefficients of job's
-// templates (count 0: none).  Four launches.
+// templates (count 0: none).  Three launches.
 void launch_sky(const Geo& g, int precision, const SkyPos& pos, const void* const* xh, const int* xh_dtype, void* G,
                 int n1, GCol gc, void* partials, SkyConst* sky, int* err, const CoefJob& job, cudaStream_t st);
 // Timing table: entries needed to cover [t_lo, t_hi] at spacing h, and the

@@ -80,8 +80,7 @@ struct fstat_plan {
   TwiddleTables tt{};
   int ca = 0, cb = 0;            // CTA shapes of pass A / pass B (0 = default)
   int cb_pk = -1, vb_pk = -1;    // pass B of the peaks mode when tuned apart (-1: cb, vb)
-  int va = 0, vb = 0;            // schedules of pass A / pass B (bit 0 radix-8 first, bit 1 one buffer,
-                                 // bit 2 pass B tile loads by TMA, bit 3 pass A three CTAs per SM)
+  int va = 0, vb = 0;            // schedule codes of pass A / pass B (fstat_set_cta)
   int ra = 0, rb = 0;            // persistent CTAs per SM of pass A / pass B (0 = all resident)
   int* d_err = nullptr;   // [0] sticky kernel error, [1] scratch for input checks
   int* h_err = nullptr;   // pinned
@@ -610,8 +609,7 @@ int finish_series(fstat_plan* p, int det, double sigma, cudaStream_t st) {
   p->sigma_ref = ref;
   p->geo.inv_sigma_ref = 1.0 / ref;
   p->geo.isf = (float)p->geo.inv_sigma_ref;
-  for (int X = 0; X < p->d.n_det; ++X)
-    {
+  for (int X = 0; X < p->d.n_det; ++X) {
     p->geo.w[X] = p->have[X] ? ref * ref / (2.0 * p->sigma[X] * p->sigma[X]) : 0.0;
     p->geo.wf[X] = (float)p->geo.w[X];
   }

@@ -237,14 +237,16 @@ k_tmpl_coef(const __grid_constant__ CoefJob job, double j_ref, double dt, int64_
 // cell of T0, whose cubic it leaves by 0.05 s in 30 s at most.
 // Between nodes every per-sample quantity is the cubic interpolant through
 // the four nearest nodes: t_m, T and a, b are smooth on the scale of the
-// node spacing (rotation: (w_rot h)^4 R_E/c ~ 1e-14 s at h = 32 s), so the
-// interpolation error is below the FP64 rounding of the quantities.
+// node spacing (rotation: (w_rot h)^4 R_E/c ~ 1e-14 s at h = 32 s), so for the
+// times the interpolation error is below their FP64 rounding; a, b are within
+// 6e-12 of the largest at 32 s (of which FP32 keeps 6e-8; FP64 plans' nodes lie
+// closer, and A, B, C take in one more difference, see sum_abc).
 //
 // Bound by the FP64 pipe (~80 operations per node and detector), hence as few
 // nodes as that accuracy allows (node_step_log2), no FP64 division, and the
-// cubics above.  Two detectors, 10 days at 0.5 s: 10.1 us (63.7 with a node every
+// cubics above.  Two detectors, 10 days at 0.5 s: 10.6 us (63.7 with a node every
 // 16 samples and Lagrange sums; 23.5 with the wider steps alone); 120 days at
-// 1 s: 95 us (348, 251).
+// 1 s: 99 us (348, 251).
 // Each block computes three nodes more than it stores, for the changes to the
 // next node and the inner mark (NodeF32).
 constexpr int kNodeThreads = 128, kNodeOut = kNodeThreads - 3;
@@ -356,9 +358,9 @@ k_sky_nodes(const __grid_constant__ Geo g, const __grid_constant__ SkyPos s) {
 // the sample blocks, 4 us more for a fence in every block.
 //
 // Bound by instruction issue (55 % of the slots; half of the warps resident) and the
-// wait for a tile's samples.  Two detectors, D = 8, 10 days at 0.5 s: 69 us, where
+// wait for a tile's samples.  Two detectors, D = 8, 10 days at 0.5 s: 70 us, where
 // step (iii) as a pass of its own over memory and 25 instructions a tap took
-// 17 + 17 + 122; 120 days at 1 s: 390 us (42 + 42 + 683).  D = 16, 400 001 samples:
+// 17 + 17 + 122; 120 days at 1 s: 386 us (42 + 42 + 683).  D = 16, 400 001 samples:
 // 24 us (45 with the constants of ResTab formed by every block).
 constexpr int kWin = kSkyBlock + 2 * kMaxD + 8;  // staged window, samples (covers the drift)
 

@@ -254,3 +254,25 @@ def test_sky_gradient_at_large_spindowns_matches_oracle(f1dot, f2dot, n):
         gr = (4.0 * g1 - g2) / 3.0
         assert abs(two_f[i] - v) <= 1e-4 * abs(v) + 1e-3
         assert np.all(np.abs((g[i] - gr) * s) <= 2e-3 * abs(v) + 2e-3), (g[i] * s, gr * s)
+
+
+@pytest.mark.parametrize("n,dt", [(100, 2.0), (300, 1.0), (511, 2.0), (1023, 1.0), (2047, 2.0), (2048, 2.0), (4096, 3.7), (8192, 0.5)])
+def test_gradient_of_short_series(n, dt):
+    # a block of samples is a large part of a short series: its truncated terms must
+    # stay below FP32 rounding, of which 2F and its f and f1dot derivatives keep ~1e-6
+    # (2e-7 per sample, cosines of at most a turn at 3e-7, sums over n samples that
+    # cancel by up to 10); 1e-5 of the largest component of the candidates
+    t = small_target(n_samples=n, dt=dt, n_fft=1 << 13, n_det=2, seed=49, dtype="c128", f_het=100.0)
+    rng = np.random.default_rng(n)
+    x = [rng.standard_normal(n) + 1j * rng.standard_normal(n) for _ in range(2)]
+    T = n * dt
+    rows = [np.array([100.0 + u / dt, v / T ** 2, 0.4, -0.3]) for u, v in rng.uniform(-0.3, 0.3, (12, 2))]
+    with pkg.FstatPlan.from_target(t) as plan:
+        for X in range(2):
+            plan.set_data(X, x[X], t.sigmas[X])
+        two_f, g = (v.cpu().numpy().astype(float) for v in plan.grad(_cands(rows)))
+    ref = [og.grad(t, x, th) for th in rows]
+    s = np.array([1.0 / T, 1.0 / T ** 2])
+    got = np.column_stack([two_f, g[:, :2] * s])
+    want = np.array([[v, *(gr[:2] * s)] for v, gr in ref])
+    assert np.all(np.abs(got - want) <= 1e-5 * np.abs(want).max(axis=0)), np.abs(got - want).max(axis=0) / np.abs(want).max(axis=0)

@@ -50,9 +50,10 @@ struct SftPlan {
 // B as a product of radices: primes above max_radix stand alone (direct
 // passes), the rest is packed greedily into the largest radices that divide
 // what is left (few passes; a radix-R butterfly costs ~R multiply-adds per
-// point, a pass one exchange through shared memory).  Direct passes come last, the
-// longest at the end: its outputs go to several CTAs, and it has a shared-memory
-// buffer to spare for the roots.
+// point, a pass one exchange through shared memory).  Direct passes come first,
+// where a warp's lanes read the same roots, or (direct_last) last, the longest at the
+// end: its outputs can go to several CTAs, and it has a shared-memory buffer to spare
+// for the roots.
 SftPlan sft_factors(int B, int max_r) {
   SftPlan p{};
   int rest = B;
@@ -79,8 +80,10 @@ SftPlan sft_factors(int B, int max_r) {
     rest /= r;
   }
   if (p.np == 0) p.r[p.np++] = 1;
-  std::sort(std::stable_partition(p.r, p.r + p.np, [&](int r) { return r <= max_r; }), p.r + p.np);
   return p;
+}
+void direct_last(SftPlan& p, int max_r) {
+  std::sort(std::stable_partition(p.r, p.r + p.np, [&](int r) { return r <= max_r; }), p.r + p.np);
 }
 
 // exp(2 pi i j / B), j < B, computed in FP64
@@ -297,31 +300,35 @@ template <typename T, typename TIn>
 cudaError_t run_sft(const void* bins, int64_t n_sft, int B, double f_het, double t_start, double t_sft,
                     int64_t m_raw, void* roots, void* xh, int* err, cudaStream_t st) {
   using V = typename C2<T>::type;
-  const SftPlan plan = sft_factors(B, max_radix<T>());
+  SftPlan plan = sft_factors(B, max_radix<T>());
   // data buffers, and the roots beside them where they fit (else from L1)
   size_t smem = (size_t)(plan.np > 1 ? 2 : 1) * B * sizeof(V);
   const bool in_smem = smem + (size_t)B * sizeof(V) <= kSftSmemMax;
   if (in_smem) smem += (size_t)B * sizeof(V);
-  const int last = plan.r[plan.np - 1], groups = (last + kSftOut - 1) / kSftOut;
-  const bool direct = last > max_radix<T>();
-  const auto kernel = direct && !in_smem ? k_sft_to_xh<T, TIn, true> : k_sft_to_xh<T, TIn, false>;
+  // The longest direct pass over as many CTAs per SFT as have threads for it and, behind
+  // other passes (formed by each of them), as the GPU holds.  us per call, one CTA per
+  // SFT with roots that do not fit read from L1 -> so: 1 SFT of 3998 = 2 x 1999 bins
+  // 818 -> 236, of 4193 = 7 x 599 314 -> 99; 1 of 12003 = 3 x 4001 18400 -> 414, 480 of
+  // them 100900 -> 17600 (one direct sum over the whole band: 449, 405, 1217, 38400).
+  // With one CTA and its roots at hand direct passes stay first (182 SFTs of 938 = 14 x
+  // 67 bins to 2F: 139 us, 143 with the direct one last).
+  const int longest = *std::max_element(plan.r, plan.r + plan.np);
+  unsigned split = 1;
+  bool spare = false;
+  if (longest > max_radix<T>()) {
+    const int groups = (longest + kSftOut - 1) / kSftOut;
+    split = (unsigned)(((int64_t)(B / longest) * groups + kSftThreads - 1) / kSftThreads);
+    const int64_t room = (int64_t)device_sm_count() * std::max<int64_t>(1, (228 * 1024) / (int64_t)(smem + 1024));
+    if (plan.np > 1) split = (unsigned)std::min<int64_t>(split, std::max<int64_t>(1, room / n_sft));
+    spare = !in_smem;
+    if (split > 1 || spare) direct_last(plan, max_radix<T>());
+  }
+  const auto kernel = spare ? k_sft_to_xh<T, TIn, true> : k_sft_to_xh<T, TIn, false>;
   // (the limit belongs to the kernel, not to this call: every call sets the same
   // value, so that none lowers it between another thread's setting and launch)
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSftSmemMax);
   if (e != cudaSuccess) return e;
   k_sft_roots<T><<<(B + 255) / 256, 256, 0, st>>>(B, (V*)roots);
-  // The last pass, where it is a direct one, over as many CTAs per SFT as have
-  // threads for it and, behind other passes (formed by each of them), as the GPU
-  // holds.  us per call, one CTA per SFT with roots that do not fit read from L1 -> so:
-  // 1 SFT of 3998 = 2 x 1999 bins 818 -> 236, of 4193 = 7 x 599 314 -> 99; 1 of 12003 =
-  // 3 x 4001 18400 -> 414, 480 of them 100900 -> 17600 (one direct sum over the whole
-  // band: 449, 405, 1217, 38400).
-  unsigned split = 1;
-  if (direct) {
-    split = (unsigned)(((int64_t)(B / last) * groups + kSftThreads - 1) / kSftThreads);
-    const int64_t room = (int64_t)device_sm_count() * std::max<int64_t>(1, (228 * 1024) / (int64_t)(smem + 1024));
-    if (plan.np > 1) split = (unsigned)std::min<int64_t>(split, std::max<int64_t>(1, room / n_sft));
-  }
   const dim3 grid((unsigned)n_sft, split);
   kernel<<<grid, kSftThreads, smem, st>>>((const TIn*)bins, (const V*)roots, B, plan, in_smem, f_het, t_start, t_sft,
                                           1.0 / (double)m_raw, (V*)xh, err);
